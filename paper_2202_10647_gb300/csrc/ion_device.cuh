@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "fp64_math.cuh"
 #include "ionize.h"
 
 namespace ion {
@@ -24,6 +25,7 @@ struct SpeciesTable {
   double a2[ION_MAX_Z];
   double b[ION_MAX_Z];
   double C[ION_MAX_Z];
+  double rmax[ION_MAX_Z];  // the largest 1/|E| whose product with C is within the cutoff
 };
 
 // Exponent (2/3)(Q/n*)^3 E_a/|E| above which W is set to 0; in the log2 units
@@ -48,6 +50,7 @@ struct StagedF64 {
   double a[ION_MAX_Z + 1];  // a2 + log2(dt)
   double b[ION_MAX_Z + 1];
   double C[ION_MAX_Z + 1];
+  double rmax[ION_MAX_Z + 1];
 };
 
 __device__ __forceinline__ void split_f64(double x, float& hi, float& lo) {
@@ -76,6 +79,7 @@ __device__ __forceinline__ void stage_f64(const SpeciesTable* t, double log2dt,
     s->a[k] = t->a2[k] + log2dt;
     s->b[k] = t->b[k];
     s->C[k] = t->C[k];
+    s->rmax[k] = t->rmax[k];
   }
 }
 
@@ -238,6 +242,8 @@ __device__ __forceinline__ float rate_ff_f32(const StagedF32& t, int k, const Fi
 }
 
 // The field's part of the FP64 exponent, once per cell: log2|E| and 1/|E|.
+// (Comparisons in this path are on the bits, as integers: an FP64 comparison
+// occupies the FP64 pipe like an addition.)
 struct FieldF64 {
   double lg, rE;
   bool zero;
@@ -245,37 +251,50 @@ struct FieldF64 {
 
 __device__ __forceinline__ FieldF64 field_f64(double E_in) {
   FieldF64 f;
-  const double E = fabs(E_in);
-  f.zero = !(E > kEmin) || isinf(E);
-  f.lg = f.zero ? 0.0 : log2(E);
-  f.rE = f.zero ? 0.0 : 1.0 / E;
+  const long long b = __double_as_longlong(E_in) & 0x7fffffffffffffffll;
+  // !(|E| > kEmin), infinite or NaN
+  f.zero = !(b > __double_as_longlong(kEmin) && b < 0x7ff0000000000000ll);
+  const double E = f.zero ? 1.0 : __longlong_as_double(b);
+  f.lg = log2_f64(E);
+  f.rE = rcp_f64(E);
   return f;
 }
 
-// W_k dt in FP64.  C/|E| is taken as C (1/|E|), one rounding more than a
-// division: a relative error of 2^-52 in a term below 1010, far under the
-// 1e-12 the FP64 form is held to.
+// log2(W_k dt): the exponent of Eq. 1 in two fused multiply-adds.  C/|E| is
+// taken as C (1/|E|), a relative error of 2^-52 in a term below 1010, far
+// under the 1e-12 the FP64 form is held to.
+__device__ __forceinline__ double exponent_f64(double a, double b, double C,
+                                               const FieldF64& f) {
+  return fma(-C, f.rE, fma(-b, f.lg, a));
+}
+
+// C/|E| past the cutoff, where Eq. 1 is 0 (both positive: ordered as bits).
+__device__ __forceinline__ bool past_cutoff(double rE, double rmax) {
+  return __double_as_longlong(rE) > __double_as_longlong(rmax);
+}
+
+// W_k dt in FP64.
 __device__ __forceinline__ double rate_dt_f64(const StagedF64& t, int k, const FieldF64& f) {
-  if (f.zero) return 0.0;
-  const double q = t.C[k] * f.rE;
-  if (q > kCutoffLog2) return 0.0;
-  double y = t.a[k] - t.b[k] * f.lg - q;
-  y = fmin(y, 1000.0);
-  return exp2(y);
+  if (f.zero || past_cutoff(f.rE, t.rmax[k])) return 0.0;
+  return exp2_f64(exponent_f64(t.a[k], t.b[k], t.C[k], f));
 }
 
 __device__ __forceinline__ double rate_dt_f64(const StagedF64& t, int k, double E_in) {
   return rate_dt_f64(t, k, field_f64(E_in));
 }
 
+// y clamped to at most 1000, then to at least the floor whose order_f64 is given.
+__device__ __forceinline__ double clamp_log2(double y, double floor, long long floor_order) {
+  if (hi_word(y) >= 0x408f4000) y = 1000.0;
+  return order_f64(y) < floor_order ? floor : y;
+}
+
 // log2(W_k dt) in FP64 straight from the exponent of rate_dt_f64 (no exp2 /
 // log2 round trip), clamped below at `floor`, which also stands for W = 0.
 __device__ __forceinline__ double log2_rate_f64(const StagedF64& t, int k, const FieldF64& f,
                                                 double floor) {
-  if (f.zero) return floor;
-  const double q = t.C[k] * f.rE;
-  if (q > kCutoffLog2) return floor;
-  return fmax(fmin(t.a[k] - t.b[k] * f.lg - q, 1000.0), floor);
+  if (f.zero || past_cutoff(f.rE, t.rmax[k])) return floor;
+  return clamp_log2(exponent_f64(t.a[k], t.b[k], t.C[k], f), floor, order_f64(floor));
 }
 
 // ---------------------------------------------------------------------------

@@ -350,14 +350,19 @@ int check_common(const char* who, const float* P, int K, const float* x, int64_t
 }
 
 // ---- training data ---------------------------------------------------------
-// x = clamp(2 (log2|E| - l2lo) / (l2hi - l2lo) - 1, -1, 1) in FP64.
-__global__ void mlp_inputs_kernel(const float* E, int64_t n, double l2lo, double l2hi,
-                                  float* x) {
+// x = clamp(2 (log2|E| - l2lo) / (l2hi - l2lo) - 1, -1, 1) in FP64, scale =
+// 2 / (l2hi - l2lo); the clamp after the rounding to float (rounding keeps
+// the order).  Bound by the FP64 pipe (a field's 12 instructions); 1,048,576
+// fields: 94 us with log2() and a division, 23 us now.
+__global__ void mlp_inputs_kernel(const float* __restrict__ E, int64_t n, double l2lo,
+                                  double scale, float* __restrict__ x) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double l2 = log2(fabs((double)E[i]));
-  const double v = 2.0 * (l2 - l2lo) / (l2hi - l2lo) - 1.0;
-  x[i] = (float)fmin(fmax(v, -1.0), 1.0);  // fmax of NaN and -1 is -1
+  const float e = fabsf(E[i]);
+  // zero, denormal, infinite and NaN fields take the library's log2
+  const double l2 = e >= 1.17549435e-38f && e <= 3.40282347e38f ? log2_f64(f64_of_f32(e))
+                                                                : log2((double)e);
+  x[i] = fminf(fmaxf((float)fma(l2 - l2lo, scale, -1.0), -1.0f), 1.0f);  // NaN: -1
 }
 
 constexpr int kColThreads = 1024;
@@ -516,7 +521,7 @@ int ion_mlp_inputs(const float* E, int64_t n, double l2lo, double l2hi, float* x
     return ion::set_error(ION_EINVAL, "ion_mlp_inputs: E and x must be non-NULL, 4-byte aligned");
   const int64_t blocks = (n + 255) / 256;
   mlp_inputs_kernel<<<(unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      E, n, l2lo, l2hi, x);
+      E, n, l2lo, 2.0 / (l2hi - l2lo), x);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     return ion::set_error(ION_ECUDA, "ion_mlp_inputs launch: %s", cudaGetErrorString(e));
