@@ -17,6 +17,7 @@
 // bf16 pairs (split_round) and takes the SFU tanh, as the tensor-core
 // inference does; the backward pass then treats the rounding as the identity
 // (straight-through).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -365,39 +366,221 @@ __global__ void mlp_inputs_kernel(const float* __restrict__ E, int64_t n, double
   x[i] = fminf(fmaxf((float)fma(l2 - l2lo, scale, -1.0), -1.0f), 1.0f);  // NaN: -1
 }
 
-constexpr int kColThreads = 1024;
+// ---- standardization -------------------------------------------------------
+// Y (n rows of K) is read once for both moments and once to be scaled.
+// Moments: a block holds a slice of rows in registers, kHold values per
+// thread, every thread on one column (threads = a multiple of K), and takes
+// the slice's column sums and then its squared deviations from the slice's
+// own means; mlp_moments_combine adds the slices up,
+//   M2 = sum_s M2_s + sum_s n_s (mean_s - mean)^2
+// (T. F. Chan, G. H. Golub, R. J. LeVeque, "Algorithms for computing the
+// sample variance", Am. Stat. 37, 1983), in a fixed order.  The slices'
+// means and M2 wait in T, which the last kernel then overwrites.
+// Bound: 3 FP64 instructions per value for the moments (2 lanes per clock and
+// SM), memory for the scaling.  1,048,576 x 18 values: two passes of 18 blocks
+// took 2 x 918 us, scaling by an FP64 division 335 us; now 140 us (107 us of
+// FP64 issue) and 15 us to combine the slices, and 40 us (34 us of traffic;
+// 124 us with an FP64 product instead of the pairs).
+constexpr int kStdThreads = 256;
+constexpr int kHold = 32;
 
-// One block per column k of Y (n rows of K): the sum over the rows in a
-// fixed order (thread t takes rows t, t + 1024, ...; then a tree over the
-// threads).  Without `mean`: out[k] = sum / n.  With it: out[k] =
-// max(sqrt(sum (Y - mean_k)^2 / (n - 1)), min_scale).
-__global__ void __launch_bounds__(kColThreads)
-    mlp_column_kernel(const double* Y, int64_t n, int K, const double* mean, double min_scale,
-                      double* out) {
-  __shared__ double part[kColThreads];
-  const int k = blockIdx.x;
-  const double m = mean ? mean[k] : 0.0;
-  double acc = 0.0;
-  for (int64_t r = threadIdx.x; r < n; r += kColThreads) {
-    const double d = Y[r * K + k] - m;
-    acc += mean ? d * d : d;
-  }
-  part[threadIdx.x] = acc;
+int std_columns(int K) { return kStdThreads / K * K; }             // threads at work
+int64_t std_rows(int K) { return (int64_t)(kStdThreads / K) * kHold; }  // rows of a slice
+
+// The block's column sums of v, in a fixed order: groups of 16 rows by their
+// first thread, then the groups by the threads of row 0, which alone receive
+// them (the others' FP64 additions would be issued for nothing).
+__device__ __forceinline__ double column_sum(double v, double* part, int K, int rows) {
+  const int row = threadIdx.x / K;
   __syncthreads();
-  for (int w = kColThreads / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    out[k] = mean ? fmax(sqrt(part[0] / (double)(n - 1)), min_scale) : part[0] / (double)n;
+  part[threadIdx.x] = v;
+  __syncthreads();
+  const bool lead = row < rows && (row & 15) == 0;
+  double s = v;
+  if (lead)
+    for (int r = 1; r < 16 && row + r < rows; ++r) s += part[threadIdx.x + r * K];
+  __syncthreads();
+  if (lead) part[threadIdx.x] = s;
+  __syncthreads();
+  if (row == 0)
+    for (int r = 16; r < rows; r += 16) s += part[threadIdx.x + r * K];
+  return s;
 }
 
-__global__ void mlp_normalize_kernel(const double* Y, int64_t n, int K, const double* mean,
-                                     const double* scale, float* T) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n * K) return;
-  const int k = (int)(i % K);
-  T[i] = (float)((Y[i] - mean[k]) / scale[k]);
+// An FP64 value kept in two floats' place (T is only 4-byte aligned).
+__device__ __forceinline__ void put_f64(float* p, double v) {
+  p[0] = __int_as_float(__double2loint(v));
+  p[1] = __int_as_float(__double2hiint(v));
+}
+__device__ __forceinline__ double get_f64(const float* p) {
+  return __hiloint2double(__float_as_int(p[1]), __float_as_int(p[0]));
+}
+
+// Slice blockIdx.x of the rows: its column means and M2 into
+// part_out[(2 slice + which) K + k].
+__global__ void __launch_bounds__(kStdThreads)
+    mlp_moments_kernel(const double* __restrict__ Y, int64_t n, int K, float* part_out) {
+  __shared__ double part[kStdThreads], means[kMaxOut];
+  const int rows = kStdThreads / K;
+  const int64_t r0 = blockIdx.x * (int64_t)rows * kHold;
+  const int ns = (int)min((int64_t)rows * kHold, n - r0);  // rows of this slice
+  const int row = threadIdx.x / K, k = threadIdx.x % K;
+  const bool on = row < rows;
+  const double* y = Y + r0 * K + threadIdx.x;
+  double v[kHold], s = 0.0;
+#pragma unroll
+  for (int i = 0; i < kHold; ++i)
+    v[i] = on && row + i * rows < ns ? __ldcs(y + (int64_t)i * rows * K) : 0.0;
+#pragma unroll
+  for (int i = 0; i < kHold; ++i) s += v[i];
+  const double sum = column_sum(s, part, K, rows);
+  if (row == 0) means[k] = sum / (double)ns;
+  __syncthreads();
+  const double mean = means[k];
+  double q = 0.0;
+#pragma unroll
+  for (int i = 0; i < kHold; ++i) {
+    if (on && row + i * rows < ns) {
+      const double d = v[i] - mean;
+      q = fma(d, d, q);
+    }
+  }
+  const double m2 = column_sum(q, part, K, rows);
+  if (row == 0) {
+    float* o = part_out + 4 * (int64_t)blockIdx.x * K;
+    put_f64(o + 2 * k, mean);
+    put_f64(o + 2 * (K + k), m2);
+  }
+}
+
+// Block k: the mean and scale of column k from the slices' means and M2.
+__global__ void __launch_bounds__(kStdThreads)
+    mlp_moments_combine(const float* __restrict__ part_in, int64_t n, int K, int64_t slices,
+                        double min_scale, double* mean_out, double* scale_out) {
+  __shared__ double part[kStdThreads];
+  const int k = blockIdx.x;
+  const int64_t per = (int64_t)(kStdThreads / K) * kHold;
+  auto total = [&](double v) {
+    __syncthreads();
+    part[threadIdx.x] = v;
+    __syncthreads();
+    for (int w = kStdThreads / 2; w > 0; w >>= 1) {
+      if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
+      __syncthreads();
+    }
+    return part[0];
+  };
+  double s = 0.0;
+  for (int64_t i = threadIdx.x; i < slices; i += kStdThreads)
+    s = fma(get_f64(part_in + 4 * i * K + 2 * k), (double)min(per, n - i * per), s);
+  const double mean = total(s) / (double)n;
+  double q = 0.0;
+  for (int64_t i = threadIdx.x; i < slices; i += kStdThreads) {
+    const double d = get_f64(part_in + 4 * i * K + 2 * k) - mean;
+    q += fma(d * d, (double)min(per, n - i * per), get_f64(part_in + 4 * i * K + 2 * (K + k)));
+  }
+  const double m2 = total(q);
+  if (threadIdx.x == 0) {
+    mean_out[k] = mean;
+    scale_out[k] = fmax(sqrt(m2 / (double)(n - 1)), min_scale);
+  }
+}
+
+// A double as hi + lo (2^-48 relative), hi its leading 24 bits, by integer
+// instructions and one int-to-float conversion; ok is false outside
+// 2^-60..2^60 (and for 0).
+__device__ __forceinline__ void split_bits(double x, float& hi, float& lo, bool& ok) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const uint32_t ex = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
+  ok = ex - (1023u - 60u) < 120u;
+  hi = __uint_as_float(sign | (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29));
+  // the 29 bits below, in units of 2^(exponent - 52)
+  lo = (float)(l & 0x1fffffffu) *
+       __uint_as_float(sign | ((ex - (1023u + 52u - 127u)) << 23));
+}
+
+// T = (Y - mean) / scale rounded to float.  Taken in FP32 pairs (2^-44
+// relative to |Y| + |mean|, about 40 FP32 and integer instructions where the
+// FP64 subtraction, product and conversion cost the time of 190); where that
+// error could change the rounded result (A. Ziv, "Fast evaluation of
+// elementary mathematical functions with correctly rounded last bit", ACM
+// TOMS 17, 1991), about one value in 10^5, or a value leaves the pairs'
+// range, in FP64.  Every thread stays on one column.
+__global__ void __launch_bounds__(kStdThreads)
+    mlp_normalize_kernel(const double* __restrict__ Y, int64_t n, int K,
+                         const double* __restrict__ mean, const double* __restrict__ scale,
+                         float* __restrict__ T) {
+  constexpr int kUnroll = 8;
+  const int rows = kStdThreads / K;
+  if ((int)threadIdx.x >= rows * K) return;
+  const int64_t step = (int64_t)rows * K;
+  const int k = threadIdx.x % K;
+  const double m = mean[k], sc = scale[k], inv = 1.0 / sc;
+  float mh, ml, ih, il;
+  bool pairs, iok;
+  split_bits(m, mh, ml, pairs);
+  if (m == 0.0) {
+    mh = ml = 0.0f;
+    pairs = true;
+  }
+  split_bits(inv, ih, il, iok);
+  pairs = pairs && iok;
+  auto one = [&](double y) -> float {
+    float yh, yl;
+    bool ok;
+    split_bits(y, yh, yl, ok);
+    // d = y - mean, q = d / scale as hi + lo
+    const float s = yh - mh, z = s - yh;
+    const float dl = ((yh - (s - z)) - (mh + z)) + (yl - ml);
+    const float p = s * ih;
+    const float e = fmaf(s, ih, -p) + fmaf(s, il, dl * ih);
+    const float err = (fabsf(yh) + fabsf(mh)) * ih * 0x1p-43f;
+    const float up = p + (e + err), down = p + (e - err);
+    if (pairs && ok && up == down && fabsf(p) >= 0x1p-60f) return up;
+    if (__double_as_longlong(y) == __double_as_longlong(m) && m - m == 0.0) return 0.0f;
+    return (float)((y - m) / sc);
+  };
+  const int64_t all = n * K, stride = gridDim.x * step * kUnroll;
+  for (int64_t i = blockIdx.x * step * kUnroll + threadIdx.x; i < all; i += stride) {
+    double y[kUnroll];
+    if (i + (kUnroll - 1) * step < all) {
+#pragma unroll
+      for (int j = 0; j < kUnroll; ++j) y[j] = __ldcs(Y + i + j * step);
+#pragma unroll
+      for (int j = 0; j < kUnroll; ++j) T[i + j * step] = one(y[j]);
+    } else {
+      for (int64_t c = i; c < all; c += step) T[c] = one(Y[c]);
+    }
+  }
+}
+
+// Fewer rows than hold the slices' means and M2 in T: one block per column,
+// mean and then scale.
+__global__ void __launch_bounds__(kStdThreads)
+    mlp_moments_small(const double* __restrict__ Y, int64_t n, int K, double min_scale,
+                      double* mean_out, double* scale_out) {
+  __shared__ double part[kStdThreads];
+  const int k = blockIdx.x;
+  double mean = 0.0;
+  for (int pass = 0; pass < 2; ++pass) {
+    double acc = 0.0;
+    for (int64_t r = threadIdx.x; r < n; r += kStdThreads) {
+      const double d = Y[r * K + k] - mean;
+      acc += pass ? d * d : d;
+    }
+    __syncthreads();
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    for (int w = kStdThreads / 2; w > 0; w >>= 1) {
+      if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
+      __syncthreads();
+    }
+    if (!pass) mean = part[0] / (double)n;
+  }
+  if (threadIdx.x == 0) {
+    mean_out[k] = mean;
+    scale_out[k] = fmax(sqrt(part[0] / (double)(n - 1)), min_scale);
+  }
 }
 
 }  // namespace
@@ -545,10 +728,19 @@ int ion_mlp_standardize(const double* Y, int64_t n, int K, double min_scale, dou
                           "ion_mlp_standardize: Y, mean_out, scale_out (8-byte aligned) and T "
                           "(4-byte aligned) must be non-NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  mlp_column_kernel<<<K, kColThreads, 0, s>>>(Y, n, K, nullptr, min_scale, mean_out);
-  mlp_column_kernel<<<K, kColThreads, 0, s>>>(Y, n, K, mean_out, min_scale, scale_out);
-  const int64_t blocks = (n * K + 255) / 256;
-  mlp_normalize_kernel<<<(unsigned)blocks, 256, 0, s>>>(Y, n, K, mean_out, scale_out, T);
+  const int64_t slices = (n + std_rows(K) - 1) / std_rows(K);
+  // a slice's means and M2 take four floats per column of T: four rows
+  if (n >= 4 * slices) {
+    mlp_moments_kernel<<<(unsigned)slices, kStdThreads, 0, s>>>(Y, n, K, T);
+    mlp_moments_combine<<<K, kStdThreads, 0, s>>>(T, n, K, slices, min_scale, mean_out,
+                                                  scale_out);
+  } else {
+    mlp_moments_small<<<K, kStdThreads, 0, s>>>(Y, n, K, min_scale, mean_out, scale_out);
+  }
+  const int64_t per = (int64_t)std_columns(K) * 8;
+  const int64_t need = (n * K + per - 1) / per;
+  mlp_normalize_kernel<<<(unsigned)std::min<int64_t>(need, 4096), kStdThreads, 0, s>>>(
+      Y, n, K, mean_out, scale_out, T);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     return ion::set_error(ION_ECUDA, "ion_mlp_standardize launch: %s", cudaGetErrorString(e));

@@ -53,3 +53,29 @@ def test_mlp_inputs_special_fields():
         ref = np.where(np.isnan(v), -1.0, np.clip(v, -1.0, 1.0)).astype(np.float32)
         # float rounding of an FP64 value within a few 1e-16: one ulp where it is a tie
         assert np.all(np.abs(x - ref) <= np.spacing(np.abs(ref)))
+
+
+@pytest.mark.parametrize("K", [1, 2, 18, 63])
+@pytest.mark.parametrize("slices", [0.1, 1, 2.5])
+def test_mlp_standardize_slices(K, slices):
+    """Row counts around the slices the moments are summed by (0.1: the
+    one-block-per-column form), and columns outside the range of the FP32
+    pairs: constant, zero, huge, tiny, far from their spread.  The targets
+    are the FP64 quotient's float, value for value."""
+    rows = 256 // K * 32
+    for n in {max(2, int(rows * slices) - 1), max(2, int(rows * slices)), int(rows * slices) + 3}:
+        rng = np.random.default_rng(n * 64 + K)
+        Y = rng.normal(0.0, 1.0, (n, K)) * rng.uniform(0.1, 30.0, K) + rng.uniform(-60, 5, K)
+        special = [np.full(n, -40.0), np.zeros(n), rng.normal(size=n) * 1e30,
+                   rng.normal(size=n) * 1e-25, 1000.0 + rng.normal(size=n) * 1e-3,
+                   np.where(np.arange(n) % 3 == 0, -40.0, rng.uniform(-40, 5, n))]
+        for k, col in enumerate(special[: K - 1] if K > 1 else special[5:]):
+            Y[:, k] = col
+        mean, scale, T = ionize.mlp_standardize(torch.tensor(Y, device="cuda"), 1e-3)
+        m, s = mean.cpu().numpy(), scale.cpu().numpy()
+        # a sum of n rounds each addition by 2^-53 of at most n max|Y|
+        tol = 1e-13 * np.abs(Y).max(0)
+        assert np.all(np.abs(m - Y.mean(0)) <= tol)
+        ref = np.maximum(Y.std(0, ddof=1), 1e-3)
+        assert np.all(np.abs(s - ref) <= 1e-12 * ref + tol)
+        assert np.array_equal(T.cpu().numpy(), ((Y - m) / s).astype(np.float32))
