@@ -4,14 +4,11 @@
 // tensor-core inference.  Network and parameter layout: mlp_device.cuh.
 //
 //   loss  L = (1/(B K)) sum_b sum_k (y_bk - t_bk)^2
-//   mlp_fwd, mlp_bwd  one thread per sample: the forward pass, then the
-//                   backward pass down to dL/dz1; they write the per-sample
-//                   factors of the weight gradients (h1, h2, dL/dz1, dL/dz2,
-//                   dL/dy).
-//   mlp_grad_part   one thread per parameter and batch slice: the sum over
-//                   the slice's samples of the outer-product terms.
-//   mlp_grad_sum    sums the slices in a fixed order (deterministic), and the
-//                   per-block loss partials.
+//   mlp_train_kernel  a block per tile of 64 samples: forward pass, backward
+//                   pass and the tile's part of the gradient, all products as
+//                   register tiles over shared memory.
+//   mlp_grad_sum    sums the blocks' parts and losses in a fixed order
+//                   (deterministic).
 //   mlp_adam        Adam with bias-corrected moments.
 // With ION_MLP_BF16 the forward pass rounds W2, W3, h1 and h2 to their
 // bf16 pairs (split_round) and takes the SFU tanh, as the tensor-core
@@ -30,47 +27,37 @@ namespace mlp {
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kSlices = 16;
+// Samples of a training tile, and threads of its block: 16 x 16, each with 4
+// samples x 4 units of every 64 x 64 product.
+constexpr int kTile = 64;
+constexpr int kTrainThreads = 256;
+constexpr int kLd = kTile + 4;  // row length in shared memory
 
-struct Acts {
-  float* h1;    // [B][H]
-  float* h2;    // [B][H]
-  float* dz1;   // [B][H]
-  float* dz2;   // [B][H]
-  float* dy;    // [B][KP]
-  float* part;  // [kSlices][nparams]
-  float* lossp; // [blocks]
+struct Parts {
+  float* grad;  // [blocks][nparams]
+  float* loss;  // [blocks]
 };
 
 size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
-int fwd_blocks(int64_t B) { return (int)((B + kThreads - 1) / kThreads); }
+int64_t train_tiles(int64_t B) { return (B + kTile - 1) / kTile; }
+
+// Room for one part per tile (the grid never exceeds the tiles) up to
+// kMaxParts of them.
+constexpr int kMaxParts = 256;
+int64_t most_parts(int64_t B) { return std::min<int64_t>(train_tiles(B), kMaxParts); }
 
 size_t ws_bytes(int K, int64_t B) {
-  const size_t b = (size_t)B;
-  return 4 * round256(4 * b * H) + round256(4 * b * padded_out(K)) +
-         round256(4 * (size_t)kSlices * nparams(K)) + round256(4 * (size_t)fwd_blocks(B));
+  return round256(4 * (size_t)most_parts(B) * nparams(K)) + round256(4 * (size_t)most_parts(B));
 }
 
-Acts bind(void* ws, int K, int64_t B) {
+Parts bind(void* ws, int K, int64_t B) {
   char* p = static_cast<char*>(ws);
-  const size_t b = (size_t)B;
-  Acts a;
-  a.h1 = reinterpret_cast<float*>(p);
-  p += round256(4 * b * H);
-  a.h2 = reinterpret_cast<float*>(p);
-  p += round256(4 * b * H);
-  a.dz1 = reinterpret_cast<float*>(p);
-  p += round256(4 * b * H);
-  a.dz2 = reinterpret_cast<float*>(p);
-  p += round256(4 * b * H);
-  a.dy = reinterpret_cast<float*>(p);
-  p += round256(4 * b * padded_out(K));
-  a.part = reinterpret_cast<float*>(p);
-  p += round256(4 * (size_t)kSlices * nparams(K));
-  a.lossp = reinterpret_cast<float*>(p);
-  return a;
+  return {reinterpret_cast<float*>(p),
+          reinterpret_cast<float*>(p + round256(4 * (size_t)most_parts(B) * nparams(K)))};
 }
+
+int fwd_blocks(int64_t B) { return (int)((B + kThreads - 1) / kThreads); }
 
 // The network staged in shared memory; output rows k >= K are zero.
 template <int KP>
@@ -103,162 +90,295 @@ __device__ __forceinline__ void stage(const float* __restrict__ P, int K, Net<KP
 // product over the register arrays (h1, y, dy, acc) fully unrolled, so the
 // arrays stay in registers at a modest code size.
 
-// Training forward pass: h1, z2 (pre-activation of layer 2), h2, dL/dy and
-// the block's partial of sum (y - t)^2.
-template <int KP, bool Q>
-__global__ void __launch_bounds__(kThreads)
-    mlp_fwd(const float* __restrict__ P, int K, const float* __restrict__ x,
-            const float* __restrict__ t, int B, float two_over_BK, Acts a) {
-  __shared__ Net<KP> n;
-  __shared__ float red[kThreads / 32];
-  stage<KP, Q>(P, K, n);
-  __syncthreads();
-  const int b = blockIdx.x * kThreads + threadIdx.x;
-  const bool on = b < B;
-  const int bb = on ? b : 0;
-  const float xb = on ? x[b] : 0.0f;
-  float h1[H];
+// ---- training --------------------------------------------------------------
+// Shared memory of a training block: the weights in both orders (a product
+// reads its inner index first), and the tile's activations and their
+// gradients as [unit][sample], which serves both the products over units (an
+// inner index at a time) and those over samples (four samples at a time).
+template <int KP>
+struct Train {
+  float W1[H], b1[H], b2[H], b3[KP];
+  float W2[H][kLd], W2T[H][kLd];    // [o][i], [i][o]
+  float W3[KP][kLd], W3T[H][KP];    // [k][o], [o][k]
+  float h1[H][kLd], h2[H][kLd];     // [unit][sample]
+  float d2[H][kLd];                 // dL/dz2
+  float dy[KP][kLd];                // dL/dy
+  float x[kTile];
+  float red[kTrainThreads / 32];
+};
+
+// acc[a][b] += sum over c < n of A[c][4 ty + a] B[c][4 tx + b], c in order.
+template <int n, int ldb>
+__device__ __forceinline__ void tile_product(float (&acc)[4][4], const float (*A)[kLd],
+                                             const float (*Bm)[ldb], int tx, int ty) {
+#pragma unroll 8
+  for (int c = 0; c < n; ++c) {
+    const float4 u = *reinterpret_cast<const float4*>(&A[c][4 * ty]);
+    const float4 w = *reinterpret_cast<const float4*>(&Bm[c][4 * tx]);
+    const float ua[4] = {u.x, u.y, u.z, u.w}, wb[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-  for (int i = 0; i < H; ++i) {
-    const float h = gelu<Q>(fmaf(n.W1[i], xb, n.b1[i]));
-    h1[i] = Q ? split_round(h) : h;
-    if (on) a.h1[(int64_t)b * H + i] = h1[i];
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ua[a], wb[b], acc[a][b]);
   }
-  float y[KP];
+}
+
+// acc[a][b] += sum over the tile's samples s of A[ty + 16 a][s] B[tx + 16 b][s].
+template <int NA>
+__device__ __forceinline__ void sample_product(float (&acc)[NA][4], const float (*A)[kLd],
+                                               const float (*Bm)[kLd], int tx, int ty) {
+#pragma unroll 2
+  for (int s = 0; s < kTile; s += 4) {
+    float4 u[NA], w[4];
 #pragma unroll
-  for (int k = 0; k < KP; ++k) y[k] = n.b3[k];
-#pragma unroll 1
-  for (int o = 0; o < H; ++o) {
-    float z = n.b2[o];
+    for (int a = 0; a < NA; ++a) u[a] = *reinterpret_cast<const float4*>(&A[ty + 16 * a][s]);
 #pragma unroll
-    for (int i = 0; i < H; ++i) z = fmaf(n.W2[o * H + i], h1[i], z);
-    float h = gelu<Q>(z);
-    h = Q ? split_round(h) : h;
-    if (on) {
-      a.dz2[(int64_t)bb * H + o] = z;  // z2, overwritten by dL/dz2 later
-      a.h2[(int64_t)bb * H + o] = h;
+    for (int b = 0; b < 4; ++b) w[b] = *reinterpret_cast<const float4*>(&Bm[tx + 16 * b][s]);
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        acc[a][b] = fmaf(u[a].x, w[b].x, acc[a][b]);
+        acc[a][b] = fmaf(u[a].y, w[b].y, acc[a][b]);
+        acc[a][b] = fmaf(u[a].z, w[b].z, acc[a][b]);
+        acc[a][b] = fmaf(u[a].w, w[b].w, acc[a][b]);
+      }
+  }
+}
+
+__device__ __forceinline__ void put4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+
+// Loss and gradient of the block's tiles.  The work is six small products
+// (129 M multiply-adds for 8192 samples of a 64-64-18 network, 3.2 us at the
+// FP32 rate of 152 SMs); one thread per sample left 64 blocks of 4 warps in
+// a serial loop over units (41 + 40 us) and a gradient pass that read
+// every activation 64 times (64 us).  A tile of 64 samples per block gives 128
+// blocks their 8 warps, 16 accumulators per 2 shared-memory loads, keeps all
+// activations on the chip, and takes each tanh once (the derivatives stay in
+// registers until the backward pass).  Per sample every sum runs in the
+// order of the serial loop.  18 us at that size, and 4 us to add the parts
+// (latency: two warps per scheduler; the products issue in about 5 us).
+template <int KP, bool Q>
+__global__ void __launch_bounds__(kTrainThreads)
+    mlp_train_kernel(const float* __restrict__ P, int K, const float* __restrict__ x,
+                     const float* __restrict__ t, int B, float two_over_BK, Parts out) {
+  constexpr int KJ = KP / 16;  // outputs per thread
+  extern __shared__ __align__(16) unsigned char train_smem[];
+  Train<KP>& S = *reinterpret_cast<Train<KP>*>(train_smem);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  {
+    // weights: a thread has column o of the transposes (no bank conflicts)
+    for (int i = tid; i < H; i += kTrainThreads) {
+      S.W1[i] = P[off_W1() + i];
+      S.b1[i] = P[off_b1() + i];
+      S.b2[i] = P[off_b2() + i];
+    }
+    for (int k = tid; k < KP; k += kTrainThreads) S.b3[k] = k < K ? P[off_b3(K) + k] : 0.0f;
+    const int o = tid & 63, q = tid >> 6;
+#pragma unroll
+    for (int i = 16 * q; i < 16 * q + 16; ++i) {
+      const float w = P[off_W2() + o * H + i];
+      const float v = Q ? split_round(w) : w;
+      S.W2[o][i] = v;
+      S.W2T[i][o] = v;
     }
 #pragma unroll
-    for (int k = 0; k < KP; ++k) y[k] = fmaf(n.W3[k * H + o], h, y[k]);
+    for (int k = q; k < KP; k += 4) {
+      const float w = k < K ? P[off_W3() + k * H + o] : 0.0f;
+      const float v = Q ? split_round(w) : w;
+      S.W3[k][o] = v;
+      S.W3T[o][k] = v;
+    }
   }
-  float l = 0.0f;
+  float gW2[4][4], gW3[KJ][4], gw1[4], gb1[4], gb2[4], gb3[KJ], loss = 0.0f;
 #pragma unroll
-  for (int k = 0; k < KP; ++k) {
-    const float d = (on && k < K) ? y[k] - t[(int64_t)b * K + k] : 0.0f;
-    l = fmaf(d, d, l);
-    if (on) a.dy[(int64_t)b * KP + k] = two_over_BK * d;  // dL/dy
+  for (int a = 0; a < 4; ++a) {
+    gw1[a] = gb1[a] = gb2[a] = 0.0f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) gW2[a][b] = 0.0f;
   }
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
+  for (int a = 0; a < KJ; ++a) {
+    gb3[a] = 0.0f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) gW3[a][b] = 0.0f;
+  }
+
+  for (int64_t s0 = (int64_t)blockIdx.x * kTile; s0 < B; s0 += (int64_t)gridDim.x * kTile) {
+    const int n = (int)min((int64_t)kTile, B - s0);
+    __syncthreads();  // the previous tile's products are done
+    if (tid < kTile) S.x[tid] = tid < n ? x[s0 + tid] : 0.0f;
+    __syncthreads();
+    // layer 1: samples 4 ty + a, units 4 tx + b; g1, g2 the derivatives
+    float g1[4][4], g2[4][4], acc[4][4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int i = 4 * tx + b;
+      float h[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const float z = fmaf(S.W1[i], S.x[4 * ty + a], S.b1[i]);
+        float th;
+        h[a] = gelu<Q>(z, th);
+        if (Q) h[a] = split_round(h[a]);
+        g1[a][b] = gelu_grad(z, th);
+        acc[a][b] = S.b2[i];
+      }
+      put4(&S.h1[i][4 * ty], h[0], h[1], h[2], h[3]);
+    }
+    __syncthreads();
+    tile_product<H, kLd>(acc, S.h1, S.W2T, tx, ty);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      float h[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        float th;
+        h[a] = gelu<Q>(acc[a][b], th);
+        if (Q) h[a] = split_round(h[a]);
+        g2[a][b] = gelu_grad(acc[a][b], th);
+      }
+      put4(&S.h2[4 * tx + b][4 * ty], h[0], h[1], h[2], h[3]);
+    }
+    __syncthreads();
+    // outputs k = tx + 16 j of samples 4 ty + a, and dL/dy
+    float y[4][KJ];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int j = 0; j < KJ; ++j) y[a][j] = S.b3[tx + 16 * j];
+#pragma unroll 8
+    for (int o = 0; o < H; ++o) {
+      const float4 u = *reinterpret_cast<const float4*>(&S.h2[o][4 * ty]);
+      const float ua[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int j = 0; j < KJ; ++j) {
+        const float w = S.W3T[o][tx + 16 * j];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) y[a][j] = fmaf(w, ua[a], y[a][j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < KJ; ++j) {
+      const int k = tx + 16 * j;
+      float d[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const bool on = 4 * ty + a < n && k < K;
+        const float e = on ? y[a][j] - t[(s0 + 4 * ty + a) * K + k] : 0.0f;
+        loss = fmaf(e, e, loss);
+        d[a] = two_over_BK * e;
+        gb3[j] += d[a];
+      }
+      put4(&S.dy[k][4 * ty], d[0], d[1], d[2], d[3]);
+    }
+    __syncthreads();
+    // dL/dz2 = (dL/dy W3) g2
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
+    tile_product<KP, kLd>(acc, S.dy, S.W3, tx, ty);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      float d[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        d[a] = acc[a][b] * g2[a][b];
+        gb2[b] += d[a];
+        acc[a][b] = 0.0f;
+      }
+      put4(&S.d2[4 * tx + b][4 * ty], d[0], d[1], d[2], d[3]);
+    }
+    sample_product<KJ>(gW3, S.dy, S.h2, tx, ty);
+    __syncthreads();
+    // dL/dz1 = (dL/dz2 W2) g1
+    tile_product<H, kLd>(acc, S.d2, S.W2, tx, ty);
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const float d = acc[a][b] * g1[a][b];
+        gb1[b] += d;
+        gw1[b] = fmaf(d, S.x[4 * ty + a], gw1[b]);
+      }
+    sample_product<4>(gW2, S.d2, S.h1, tx, ty);
+  }
+
+  // the block's part: the matrices from their owners, the vectors summed over
+  // the 16 sample groups in order
+  float* part = out.grad + (int64_t)blockIdx.x * nparams(K);
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) part[off_W2() + (ty + 16 * a) * H + tx + 16 * b] = gW2[a][b];
+#pragma unroll
+  for (int a = 0; a < KJ; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (ty + 16 * a < K) part[off_W3() + (ty + 16 * a) * H + tx + 16 * b] = gW3[a][b];
   __syncthreads();
-  if (threadIdx.x == 0) {
+  float(*v)[kLd] = S.h1;  // rows: W1, b1, b2 x 16 groups, then b3 in S.h2
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    v[ty][4 * tx + b] = gw1[b];
+    v[16 + ty][4 * tx + b] = gb1[b];
+    v[32 + ty][4 * tx + b] = gb2[b];
+  }
+#pragma unroll
+  for (int j = 0; j < KJ; ++j) S.h2[ty][tx + 16 * j] = gb3[j];
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, s);
+  if ((tid & 31) == 0) S.red[tid >> 5] = loss;
+  __syncthreads();
+  {
+    const int which = tid >> 6, c = tid & 63;
+    float s = 0.0f;
+    const float(*r)[kLd] = which < 3 ? &v[16 * which] : &S.h2[0];
+#pragma unroll
+    for (int g = 0; g < 16; ++g) s += r[g][c];
+    if (which == 0) part[off_W1() + c] = s;
+    if (which == 1) part[off_b1() + c] = s;
+    if (which == 2) part[off_b2() + c] = s;
+    if (which == 3 && c < K) part[off_b3(K) + c] = s;
+  }
+  if (tid == 0) {
     float s = 0.0f;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w];
-    a.lossp[blockIdx.x] = s;
+    for (int w = 0; w < kTrainThreads / 32; ++w) s += S.red[w];
+    out.loss[blockIdx.x] = s;
   }
 }
 
-// Training backward pass: dL/dz2 (in place of z2) and dL/dz1.
-template <int KP, bool Q>
-__global__ void __launch_bounds__(kThreads)
-    mlp_bwd(const float* __restrict__ P, int K, const float* __restrict__ x, int B, Acts a) {
-  __shared__ Net<KP> n;
-  stage<KP, Q>(P, K, n);
-  __syncthreads();
-  const int b = blockIdx.x * kThreads + threadIdx.x;
-  if (b >= B) return;
-  const float xb = x[b];
-  float dy[KP], acc[H];
-#pragma unroll
-  for (int k = 0; k < KP; ++k) dy[k] = a.dy[(int64_t)b * KP + k];
-#pragma unroll
-  for (int i = 0; i < H; ++i) acc[i] = 0.0f;
-#pragma unroll 1
-  for (int o = 0; o < H; ++o) {
-    float g = 0.0f;
-#pragma unroll
-    for (int k = 0; k < KP; ++k) g = fmaf(dy[k], n.W3[k * H + o], g);
-    const float z = a.dz2[(int64_t)b * H + o];
-    float th;
-    gelu<Q>(z, th);
-    const float d = g * gelu_grad(z, th);  // dL/dz2
-    a.dz2[(int64_t)b * H + o] = d;
-#pragma unroll
-    for (int i = 0; i < H; ++i) acc[i] = fmaf(d, n.W2[o * H + i], acc[i]);
-  }
-#pragma unroll
-  for (int i = 0; i < H; ++i) {
-    const float z1 = fmaf(n.W1[i], xb, n.b1[i]);
-    float th;
-    gelu<Q>(z1, th);
-    a.dz1[(int64_t)b * H + i] = acc[i] * gelu_grad(z1, th);
-  }
-}
-
-// Parameter p's sum over the samples of slice blockIdx.y.
-__global__ void __launch_bounds__(kThreads)
-    mlp_grad_part(int K, int KP, const float* __restrict__ x, int B, Acts a) {
-  const int np = nparams(K);
-  const int p = blockIdx.x * kThreads + threadIdx.x;
-  if (p >= np) return;
-  const int s = blockIdx.y;
-  const int b0 = (int)((int64_t)B * s / kSlices), b1 = (int)((int64_t)B * (s + 1) / kSlices);
-  // each parameter is the sum over samples of u[b] * v[b]
-  const float* u;
-  const float* v = nullptr;  // nullptr: v = 1 (biases)
-  int64_t su, sv = 0;
-  if (p < off_b1()) {  // W1[i]: dz1[b][i] x[b]
-    u = a.dz1 + p;
-    su = H;
-    v = x;
-    sv = 1;
-  } else if (p < off_W2()) {  // b1[i]
-    u = a.dz1 + (p - off_b1());
-    su = H;
-  } else if (p < off_b2()) {  // W2[o][i]: dz2[b][o] h1[b][i]
-    const int q = p - off_W2();
-    u = a.dz2 + q / H;
-    su = H;
-    v = a.h1 + q % H;
-    sv = H;
-  } else if (p < off_W3()) {  // b2[o]
-    u = a.dz2 + (p - off_b2());
-    su = H;
-  } else if (p < off_b3(K)) {  // W3[k][o]: dy[b][k] h2[b][o]
-    const int q = p - off_W3();
-    u = a.dy + q / H;
-    su = KP;
-    v = a.h2 + q % H;
-    sv = H;
-  } else {  // b3[k]
-    u = a.dy + (p - off_b3(K));
-    su = KP;
-  }
-  float acc = 0.0f;
-  if (v) {
-    for (int b = b0; b < b1; ++b) acc = fmaf(u[(int64_t)b * su], v[(int64_t)b * sv], acc);
-  } else {
-    for (int b = b0; b < b1; ++b) acc += u[(int64_t)b * su];
-  }
-  a.part[(int64_t)s * np + p] = acc;
-}
-
-__global__ void __launch_bounds__(kThreads)
-    mlp_grad_sum(int np, int nloss, Acts a, float* __restrict__ grad, float* __restrict__ loss,
-                 float inv_BK) {
-  const int p = blockIdx.x * kThreads + threadIdx.x;
+// The parts summed in a fixed order: 32 parameters per block, its 8 warps
+// take the parts w, w + 8, ... and are then added in order.
+__global__ void __launch_bounds__(256)
+    mlp_grad_sum(int np, int nparts, Parts in, float* __restrict__ grad,
+                 float* __restrict__ loss, float inv_BK) {
+  __shared__ float red[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
+  float g = 0.0f;
   if (p < np) {
-    float g = 0.0f;
-#pragma unroll
-    for (int s = 0; s < kSlices; ++s) g += a.part[(int64_t)s * np + p];
-    grad[p] = g;
+#pragma unroll 8
+    for (int b = w; b < nparts; b += 8) g += in.grad[(int64_t)b * np + p];
   }
-  if (p == 0 && loss) {
+  red[w][lane] = g;
+  if (blockIdx.x == 0 && w == 0 && loss) {
     float l = 0.0f;
-    for (int i = 0; i < nloss; ++i) l += a.lossp[i];
-    *loss = l * inv_BK;
+    for (int i = lane; i < nparts; i += 32) l += in.loss[i];
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
+    if (lane == 0) *loss = l * inv_BK;
+  }
+  __syncthreads();
+  if (w == 0 && p < np) {
+    float s = red[0][lane];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) s += red[i][lane];
+    grad[p] = s;
   }
 }
 
@@ -311,18 +431,30 @@ __global__ void __launch_bounds__(kThreads)
     if (k < K) y_out[(int64_t)b * K + k] = y[k];
 }
 
-template <int KP>
-cudaError_t launch_fwd_bwd(bool q, const float* P, int K, const float* x, const float* t, int B,
-                           float two_over_BK, const Acts& a, cudaStream_t s) {
-  const int g = fwd_blocks(B);
-  if (q) {
-    mlp_fwd<KP, true><<<g, kThreads, 0, s>>>(P, K, x, t, B, two_over_BK, a);
-    mlp_bwd<KP, true><<<g, kThreads, 0, s>>>(P, K, x, B, a);
-  } else {
-    mlp_fwd<KP, false><<<g, kThreads, 0, s>>>(P, K, x, t, B, two_over_BK, a);
-    mlp_bwd<KP, false><<<g, kThreads, 0, s>>>(P, K, x, B, a);
-  }
+template <int KP, bool Q>
+cudaError_t launch_train(const float* P, int K, const float* x, const float* t, int B,
+                         float two_over_BK, const Parts& a, int* nparts, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_train_kernel<KP, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(Train<KP>));
+  if (e != cudaSuccess) return e;
+  // one block per SM (the shared memory's limit), each with an equal share
+  const int64_t tiles = train_tiles(B), cap = std::min(sms, kMaxParts);
+  const int64_t each = (tiles + cap - 1) / cap;
+  *nparts = (int)((tiles + each - 1) / each);
+  mlp_train_kernel<KP, Q><<<*nparts, kTrainThreads, sizeof(Train<KP>), s>>>(P, K, x, t, B,
+                                                                            two_over_BK, a);
   return cudaGetLastError();
+}
+
+template <int KP>
+cudaError_t launch_train(bool q, const float* P, int K, const float* x, const float* t, int B,
+                         float two_over_BK, const Parts& a, int* nparts, cudaStream_t s) {
+  return q ? launch_train<KP, true>(P, K, x, t, B, two_over_BK, a, nparts, s)
+           : launch_train<KP, false>(P, K, x, t, B, two_over_BK, a, nparts, s);
 }
 
 template <int KP>
@@ -613,31 +745,29 @@ int ion_mlp_loss_grad(const float* P, int K, const float* x, const float* t, int
                           "%zu bytes",
                           ws_bytes(K, B));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const Acts a = bind(workspace, K, B);
+  const Parts a = bind(workspace, K, B);
   const bool q = (flags & ION_MLP_BF16) != 0;
   const float two_over_BK = (float)(2.0 / ((double)B * K));
-  const int KP = padded_out(K);
+  int nparts = 0;
   cudaError_t e;
-  switch (KP) {
+  switch (padded_out(K)) {
     case 16:
-      e = launch_fwd_bwd<16>(q, P, K, x, t, (int)B, two_over_BK, a, s);
+      e = launch_train<16>(q, P, K, x, t, (int)B, two_over_BK, a, &nparts, s);
       break;
     case 32:
-      e = launch_fwd_bwd<32>(q, P, K, x, t, (int)B, two_over_BK, a, s);
+      e = launch_train<32>(q, P, K, x, t, (int)B, two_over_BK, a, &nparts, s);
       break;
     case 48:
-      e = launch_fwd_bwd<48>(q, P, K, x, t, (int)B, two_over_BK, a, s);
+      e = launch_train<48>(q, P, K, x, t, (int)B, two_over_BK, a, &nparts, s);
       break;
     default:
-      e = launch_fwd_bwd<64>(q, P, K, x, t, (int)B, two_over_BK, a, s);
+      e = launch_train<64>(q, P, K, x, t, (int)B, two_over_BK, a, &nparts, s);
       break;
   }
   if (e == cudaSuccess) {
     const int np = nparams(K);
-    const dim3 grid((np + kThreads - 1) / kThreads, kSlices);
-    mlp_grad_part<<<grid, kThreads, 0, s>>>(K, KP, x, (int)B, a);
-    mlp_grad_sum<<<(np + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-        np, fwd_blocks(B), a, grad, loss, (float)(1.0 / ((double)B * K)));
+    mlp_grad_sum<<<(np + 31) / 32, 256, 0, s>>>(np, nparts, a, grad, loss,
+                                                (float)(1.0 / ((double)B * K)));
     e = cudaGetLastError();
   }
   if (e != cudaSuccess)
