@@ -507,7 +507,7 @@ int run_batch(const ion_batch_job* jobs, int njobs, double dt_fs, const ion_step
   if (f64) {
     e = cudaMemsetAsync(a.ws.hdr, 0, ion::kHdrWords * sizeof(uint32_t), s);
     for (int j = 0; j < njobs && e == cudaSuccess; ++j)
-      e = ion::launch_step_f64(a.job[j], a.pol, a.ws.hdr, s);
+      e = ion::launch_step_f64(a.job[j], a.pol, a.ws.hdr, j == 0, s);
   } else {
     e = ion::launch_batch_f32(a, sh, jobs[0].species->num_sms, s);
   }

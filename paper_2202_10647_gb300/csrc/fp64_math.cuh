@@ -185,6 +185,15 @@ __device__ __forceinline__ double f64_of_f32(float x) {
   return __hiloint2double((b << 1) ? (int)h : 0, (int)(b << 29));
 }
 
+// A double's leading 24 bits as a float, without the FP64 pipe: truncated
+// towards 0, its size held within the normal floats (0 becomes about 1e-38).
+__device__ __forceinline__ float f32_of_f64(double x) {
+  const uint32_t h = (uint32_t)hi_word(x);
+  const uint32_t m = min(max(h & 0x7fffffffu, 0x38100000u), 0x47efffffu);
+  return __uint_as_float((h & 0x80000000u) | ((m - 0x38000000u) << 3) |
+                         ((uint32_t)lo_word(x) >> 29));
+}
+
 // Order of two doubles by integer comparison (x, y not NaN; -0 below +0).
 __device__ __forceinline__ long long order_f64(double x) {
   const long long b = __double_as_longlong(x);
@@ -221,6 +230,12 @@ __device__ __forceinline__ double rcp_f64(double E) {
   return e > 1020 ? 0.0 : __hiloint2double(hi_word(q) - (e << 20), lo_word(q));
 }
 
+// a / b for a normal b up to 2^1020.
+__device__ __forceinline__ double div_f64(double a, double b) {
+  const double r = rcp_f64(__longlong_as_double(__double_as_longlong(b) & 0x7fffffffffffffffll));
+  return a * __hiloint2double(hi_word(r) ^ (hi_word(b) & (int)0x80000000), lo_word(r));
+}
+
 // 2^y; y is clamped to [-1200, 1000] (-1200: 0 after rounding).
 __device__ __forceinline__ double exp2_f64(double y) {
   const int yh = hi_word(y);
@@ -240,5 +255,9 @@ __device__ __forceinline__ double exp2_f64(double y) {
   // below the normal range: scaled up by 2^256, then back with one rounding
   return __hiloint2double(hi_word(v) + ((e + 256) << 20), lo_word(v)) * 0x1p-256;
 }
+
+// e^z for z <= 0: the product with log2 e rounds once, |z| 2^-53 relative to
+// e^z, at most 0.37 2^-53 absolute.
+__device__ __forceinline__ double exp_f64(double z) { return exp2_f64(z * 0x1.71547652b82fep+0); }
 
 }  // namespace ion

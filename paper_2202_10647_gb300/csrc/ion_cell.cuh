@@ -89,16 +89,6 @@ struct F32Form {
   }
 };
 
-struct F64Form {
-  using T = double;
-  using Staged = StagedF64;
-  using Field = FieldF64;
-  __device__ static Field field(double E) { return field_f64(E); }
-  __device__ static double rate(const StagedF64& t, int k, const Field& f) {
-    return rate_dt_f64(t, k, f);
-  }
-};
-
 // Warp-aggregated append of (value, tag) for the lanes with `take` set: one
 // atomic per warp.  Every lane of the warp calls this.
 __device__ __forceinline__ void warp_append(uint32_t* counter, uint32_t* queue,
@@ -247,24 +237,6 @@ __device__ __forceinline__ bool finish_cell(const JobIO& J, const Policy& pol,
       if (r < w - 1) lam[r] = F::rate(tab, lo + r, f);
   }
   return update_cell<T, WM>(J, pol, c, lo, hi, v, lam, allow_fb, change);
-}
-
-// The same, loading the window from global memory; W bounds the width.
-template <class F, int W>
-__device__ __forceinline__ bool global_cell(const JobIO& J, const Policy& pol,
-                                            const typename F::Staged& tab, int c,
-                                            typename F::T Ec, int lo, int hi,
-                                            bool allow_fb, typename F::T* change = nullptr) {
-  using T = typename F::T;
-  const T* __restrict__ N = static_cast<const T*>(J.N);
-  T v[W];
-  const T* p = N + (int64_t)lo * J.ld + c;
-#pragma unroll
-  for (int r = 0; r < W; ++r) {
-    v[r] = r < hi - lo + 1 ? __ldcs(p) : T(0);
-    p += J.ld;
-  }
-  return finish_cell<F, W>(J, pol, tab, c, Ec, lo, hi, v, allow_fb, change);
 }
 
 }  // namespace ion

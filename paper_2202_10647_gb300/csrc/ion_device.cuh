@@ -335,11 +335,13 @@ __device__ constexpr float kThrF32[19] = {
     0.284591f, 0.431847f,    0.605168f,   0.801103f,  1.01652f,   1.24869f,
     1.49528f,  1.75432f,     2.02414f,    2.30334f,   2.59073f,   2.88531f,
     3.18621f};
-__device__ constexpr double kThrF64[20] = {
-    2e-17,     6.32456e-09, 4.93242e-06, 0.000148017, 0.00119136, 0.00493242,
-    0.0139108, 0.0307836,   0.0578509,   0.0968455,   0.148911,   0.214675,
-    0.294354,  0.387859,    0.494882,    0.614969,    0.747572,   0.892092,
-    1.04791,   1.21439};
+// (The FP64 thresholds are floats too: they meet an FP32 upper bound of the
+// rate, as an FP64 comparison occupies the FP64 pipe like an addition.)
+__device__ constexpr float kThrF64[20] = {
+    2e-17f,     6.32456e-09f, 4.93242e-06f, 0.000148017f, 0.00119136f, 0.00493242f,
+    0.0139108f, 0.0307836f,   0.0578509f,   0.0968455f,   0.148911f,   0.214675f,
+    0.294354f,  0.387859f,    0.494882f,    0.614969f,    0.747572f,   0.892092f,
+    1.04791f,   1.21439f};
 
 // 1/n! for n = 0..17 (the Taylor branch needs n <= 4 + 12), in each
 // precision (the FP32 path reads no double: conversions run on the FP64 pipe).
@@ -374,25 +376,34 @@ struct DDParams<float> {
   }
   __device__ static __forceinline__ float div(float a, float b) { return __fdividef(a, b); }
   __device__ static __forceinline__ float inv_fact(int n) { return kInvFactF[n]; }
+  __device__ static __forceinline__ float expn(float z) { return exp(z); }
+  // what the choices of a divided difference's form look at
+  __device__ static __forceinline__ float key(float z) { return z; }
 };
 
 template <>
 struct DDParams<double> {
-  static constexpr double tau = 0.25;
+  static constexpr float tau = 0.25f;
   static constexpr int RMAX = 12;
-  static constexpr double prop_max = 0.5;
+  static constexpr float prop_max = 0.5f;
   static constexpr int PMAX = 18;
   static constexpr bool kUniform = false;  // terms(s) of them
-  static constexpr double end_ratio = 4.0;
-  __device__ static __forceinline__ int terms(double x, int rmax) {
+  static constexpr float end_ratio = 4.0f;
+  __device__ static __forceinline__ int terms(float x, int rmax) {
     int R = 0;
 #pragma unroll
     for (int i = 0; i < 20; ++i)
       if (i < rmax) R += x > kThrF64[i] ? 1 : 0;
     return R;
   }
-  __device__ static __forceinline__ double div(double a, double b) { return a / b; }
+  __device__ static __forceinline__ double div(double a, double b) { return div_f64(a, b); }
   __device__ static __forceinline__ double inv_fact(int n) { return kInvFact[n]; }
+  __device__ static __forceinline__ double expn(double z) { return exp_f64(z); }
+  // the leading 24 bits choose: a form taken at a spread 2^-23 of the node's
+  // size off its threshold is as accurate, and where that is large (a node
+  // below -2^20) every value is 0; equal nodes have equal keys, so that no
+  // difference divides by 0
+  __device__ static __forceinline__ float key(double z) { return f32_of_f64(z); }
 };
 
 // mask of the contiguous node range [j, i]
@@ -463,21 +474,26 @@ __device__ __forceinline__ void dd_exp_ranges(const T (&z)[NR], const T (&ez)[NR
 #pragma unroll
   for (int i = 0; i < NR; ++i) D[1 << i] = ez[i];
   // spread of every range from running extremes
-  T S[NR][NR];
+  float zk[NR], S[NR][NR], zmax = 0.0f;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    zk[i] = P::key(z[i]);
+    if (i < nlive) zmax = fmaxf(zmax, fabsf(zk[i]));
+  }
   bool close = false;  // some live range has spread below TAU
-  T smax = T(0);       // the largest such spread
+  float smax = 0.0f;   // the largest such spread
 #pragma unroll
   for (int j = 0; j < NR; ++j) {
-    T mn = z[j], mx = z[j];
+    float mn = zk[j], mx = zk[j];
 #pragma unroll
     for (int i = j + 1; i < NR; ++i) {
-      mn = fmin(mn, z[i]);
-      mx = fmax(mx, z[i]);
-      const T s = mx - mn;
+      mn = fminf(mn, zk[i]);
+      mx = fmaxf(mx, zk[i]);
+      const float s = mx - mn;
       S[j][i] = s;
       if (i < nlive) {
         close = close || s < P::tau;
-        smax = s < P::tau ? fmax(smax, s) : smax;
+        smax = s < P::tau ? fmaxf(smax, s) : smax;
       }
     }
   }
@@ -486,19 +502,21 @@ __device__ __forceinline__ void dd_exp_ranges(const T (&z)[NR], const T (&ez)[NR
   for (int a = 0; a < NR; ++a)
 #pragma unroll
     for (int b = 0; b < NR; ++b) C[a][b] = T(0);
-  if (close) taylor_chains<T, NR>(z, P::kUniform ? P::RMAX : P::terms(smax, P::RMAX), C);
+  // (a spread of truncated keys lies within 2^-23 of their size of the nodes')
+  if (close)
+    taylor_chains<T, NR>(
+        z, P::kUniform ? P::RMAX : P::terms(fmaf(0x1p-22f, zmax, smax), P::RMAX), C);
 #pragma unroll
   for (int len = 2; len <= NR; ++len) {
 #pragma unroll
     for (int j = 0; j + len <= NR; ++j) {
       const int i = j + len - 1;
-      const T s = S[j][i];
-      const T dz = z[i] - z[j];
+      const float s = S[j][i], dk = fabsf(zk[i] - zk[j]);
       T d;
       if (s < P::tau) {
         d = ez[j] * C[j][i];
       } else if (len > 2 && i < nlive &&
-                 (fabs(dz) < P::tau || s > P::end_ratio * fabs(dz))) {
+                 (dk < P::tau || s > P::end_ratio * dk)) {
         // the range's own nodes, padded with z = 0 (the largest a node can be)
         d = dd_set<T>(z[j], z[j + 1], z[j + 2 < NR ? j + 2 : j],
                       len > 3 ? z[j + 3 < NR ? j + 3 : j] : T(0),
@@ -506,7 +524,8 @@ __device__ __forceinline__ void dd_exp_ranges(const T (&z)[NR], const T (&ez)[NR
                       ez[j + 2 < NR ? j + 2 : j], len > 3 ? ez[j + 3 < NR ? j + 3 : j] : T(1),
                       len > 4 ? ez[j + 4 < NR ? j + 4 : j] : T(1), len);
       } else {
-        d = P::div(D[range_mask(j + 1, i)] - D[range_mask(j, i - 1)], dz);
+        d = P::div(D[range_mask(j + 1, i)] - D[range_mask(j, i - 1)],
+                   z[i] - z[j]);
       }
       D[range_mask(j, i)] = d;
     }
@@ -543,10 +562,10 @@ __device__ __noinline__ T dd_set(T z0, T z1, T z2, T z3, T z4, T e0, T e1, T e2,
     for (int j = 0; j + len <= m; ++j) {
       const int i = j + len - 1;
       const T zi = z[i], s = zi - z[j];
-      if (s >= P::tau) {
+      if (P::key(zi) - P::key(z[j]) >= P::tau) {
         d[j] = P::div(d[j + 1] - d[j], s);
       } else {
-        const int R = P::kUniform ? P::RMAX : P::terms(s, P::RMAX);
+        const int R = P::kUniform ? P::RMAX : P::terms((float)s, P::RMAX);
         T H[P::RMAX + 1];
         H[0] = T(1);
 #pragma unroll
@@ -562,7 +581,7 @@ __device__ __noinline__ T dd_set(T z0, T z1, T z2, T z3, T z4, T e0, T e1, T e2,
 #pragma unroll
         for (int r = P::RMAX; r >= 0; --r)
           if (r <= R) acc = fma(H[r], P::inv_fact(len - 1 + r), acc);
-        d[j] = exp(zi) * acc;
+        d[j] = P::expn(zi) * acc;
       }
     }
   }
@@ -609,6 +628,51 @@ __device__ __forceinline__ T taylor_propagate(T (&v)[WM], const T (&lam)[WM],
   return dne;
 }
 
+// 1/k! of the FP64 series (constant memory: one entry per term at a uniform
+// index).
+__constant__ const double kInvFactC[18 + 1] = {
+    1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040,
+    1.0 / 40320, 1.0 / 362880, 1.0 / 3628800, 1.0 / 39916800, 1.0 / 479001600,
+    1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0,
+    1.0 / 20922789888000.0, 1.0 / 355687428096000.0, 1.0 / 6402373705728000.0};
+
+// The same in FP64 for a window of exactly W states, in R terms: the series
+// of the flow across each boundary, F_r = sum_k W_r dt u_r^(k-1) / k!, so that a term
+// takes three FP64 instructions per boundary (flow, its share, the state's
+// next u = inflow - outflow) and none for the top state, which only
+// receives; N'_r = N_r + F_{r-1} - F_r, and the freed electrons are sum F.
+// (The term-by-term form above takes four per slot.)
+template <int W>
+__device__ __forceinline__ double taylor_flow_f64(double (&v)[W], const double (&lam)[W], int R) {
+  double u[W - 1], F[W - 1];
+#pragma unroll
+  for (int r = 0; r < W - 1; ++r) {
+    u[r] = v[r];
+    F[r] = 0.0;
+  }
+#pragma unroll 1
+  for (int k = 1; k <= R; ++k) {
+    const double ck = kInvFactC[k];
+    double in = 0.0;
+#pragma unroll
+    for (int r = 0; r < W - 1; ++r) {
+      const double flow = lam[r] * u[r];
+      F[r] = fma(flow, ck, F[r]);
+      u[r] = r > 0 ? in - flow : -flow;
+      in = flow;
+    }
+  }
+  double dne = F[0];
+  v[0] -= F[0];
+#pragma unroll
+  for (int r = 1; r < W - 1; ++r) {
+    v[r] += F[r - 1] - F[r];
+    dne += F[r];
+  }
+  v[W - 1] += F[W - 2];
+  return dne;
+}
+
 // ---------------------------------------------------------------------------
 // Windowed update of one cell (Eqs. 3-9) with the divided-difference
 // (Bateman) coefficients.
@@ -631,7 +695,7 @@ __device__ __forceinline__ T dd_update(T (&v)[WM], const T (&lam)[WM], int w) {
   for (int r = 0; r < NR; ++r) {
     const T l = r < w - 1 ? lam[r] : T(0);
     z[r] = -l;
-    ez[r] = exp(-l);
+    ez[r] = DDParams<T>::expn(-l);
   }
   // (Rates fall along the window in the usual ladder near threshold, each
   // state harder to ionize than the one below, and rise far above the

@@ -149,7 +149,8 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
 // kernel of the same call (step_f32.cu).
 cudaError_t launch_stiff_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_fb_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
-cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr,
+// `first`: nothing has run since the header was cleared.
+cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr, bool first,
                             cudaStream_t s);
 LaunchShape default_shape();
 bool valid_shape(const LaunchShape& s);
