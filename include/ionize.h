@@ -510,7 +510,9 @@ ION_API int ion_surrogate_rates(const ion_surrogate* s, const float* E, int64_t 
  * (a perturbation of the rate matrix by dA moves the solution of Eq. 3 by
  * at most |dA| in the 1-norm); if it is below pop_tol the network's rates
  * are used, otherwise (and outside the range) the rates of Eq. 1; pop_tol 0
- * never uses the network.  A cell
+ * never uses the network.  (Where the arrays allow the streaming kernel, a
+ * cell whose rates of Eq. 1, lowered by twice their validation bound, already
+ * exceed pop_tol takes Eq. 1 without asking the network.)  A cell
  * with some rate W dt > 1 always takes the rates of Eq. 1 (its bound would
  * exceed any useful tolerance) and is finished in the Bateman form by
  * ion_step's record kernel.  The update itself is ion_step's (Taylor or
@@ -533,8 +535,8 @@ ION_API int ion_step_surrogate(const ion_surrogate* s, const float* E, float* N,
  * (ion_surrogate_rates, ion_step_surrogate) makes the first tensor-core
  * wait of each tile poll, 64 times, an mbarrier that nothing arrives at, so
  * that the wait gives up exactly as a wait that ran out of its limit would:
- * ion_step_surrogate leaves every cell untouched and sets word 5 of the
- * workspace header, ion_surrogate_rates writes NaN rates, and each CTA waits
+ * ion_step_surrogate leaves every cell it would ask the network about
+ * untouched and sets word 5 of the workspace header, ion_surrogate_rates writes NaN rates, and each CTA waits
  * (bounded) for the matrix products it skipped before it frees its tensor
  * memory.  on = 0 restores the normal waits.  Synchronous (one 4-byte copy
  * to the device).  Errors: ION_EINVAL, ION_ECUDA. */

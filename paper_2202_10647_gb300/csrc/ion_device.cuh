@@ -356,6 +356,31 @@ __device__ constexpr float kInvFactF[18] = {
     1.0f / 6227020800.0f, 1.0f / 87178291200.0f, 1.0f / 1307674368000.0f,
     1.0f / 20922789888000.0f, 1.0f / 355687428096000.0f};
 
+// Terms of the FP32 series at most (2 W dt <= kThrF32[kEasyTerms]) and their
+// 1/k! (constant memory: the term loop reads one entry per term at a
+// warp-uniform index).
+constexpr int kEasyTerms = 18;
+__constant__ const float kInvFactF32[kEasyTerms + 1] = {
+    1.0f,
+    1.0f,
+    1.0f / 2,
+    1.0f / 6,
+    1.0f / 24,
+    1.0f / 120,
+    1.0f / 720,
+    1.0f / 5040,
+    1.0f / 40320,
+    1.0f / 362880,
+    1.0f / 3628800,
+    1.0f / 39916800,
+    1.0f / 479001600,
+    1.0f / 6227020800.0f,
+    1.0f / 87178291200.0f,
+    1.0f / 1307674368000.0f,
+    1.0f / 20922789888000.0f,
+    1.0f / 355687428096000.0f,
+    1.0f / 6402373705728000.0f};
+
 template <typename T>
 struct DDParams;
 

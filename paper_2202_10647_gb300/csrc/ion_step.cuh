@@ -19,7 +19,7 @@ constexpr int kHdrTimeout = 5;   // surrogate step: non-zero if a bounded wait g
 constexpr int kHdrRecNarrow = 6; // records of windows of <= kRecNarrow states (from the front)
 constexpr int kHdrRecWide = 7;   // records of wider windows (from the back of the arrays)
 constexpr int kHdrChunk = 8;     // streaming kernels: next chunk or group to hand out
-constexpr int kHdrHot = 9;       // (reserved)
+constexpr int kHdrNet = 9;       // surrogate step: cells left to the network kernel
 constexpr int kHdrCons = 10;     // ION_CONSERVATION_CHECK: largest |change of sum_k N_k|
 constexpr int kHdrWords = 11;
 // Records of at most this many window states take the short divided-difference
@@ -103,6 +103,19 @@ struct BatchArgs {
   Scratch ws;
 };
 
+// Which cells the surrogate step leaves to the network (net_candidate in
+// step_f32.cu): the trained range, the tolerance, and the validation bounds as
+// gates.
+struct NetSelect {
+  const float* gate;  // [nbins][Z]: beta (1 + beta)^-2, beta = 2^bound - 1
+  float gate_min;     // the smallest of them
+  int nbins;
+  float bin_a, bin_b;  // bin = floor(bin_a log2|E| + bin_b)
+  float l2lo, l2hi;
+  float pop_tol;
+  uint32_t* list;  // the cells left (their number in header word kHdrNet)
+};
+
 // Launch shape of the FP32 streaming kernel (chosen by default or by
 // ion_autotune).
 struct LaunchShape {
@@ -149,6 +162,12 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
 // kernel of the same call (step_f32.cu).
 cudaError_t launch_stiff_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_fb_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
+// One species' cells stepped with the rates of Eq. 1, except those the
+// network could serve, which are listed and left untouched.  The header is
+// already cleared.  *fits: whether the arrays allow it (nothing is launched
+// otherwise).
+cudaError_t launch_net_select_f32(BatchArgs& a, const NetSelect& sel, int num_sms, bool* fits,
+                                  cudaStream_t s);
 // `first`: nothing has run since the header was cleared.
 cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr, bool first,
                             cudaStream_t s);

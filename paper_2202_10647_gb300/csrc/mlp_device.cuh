@@ -11,6 +11,8 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 
+#include "f32x2.cuh"
+
 namespace ion {
 namespace mlp {
 
@@ -70,13 +72,16 @@ __device__ __forceinline__ float gelu(float z) {
   return gelu<Fast>(z, t);
 }
 
-// gelu<true>(2 zh) from zh, bit for bit (every step is the same operation
-// scaled by a power of two), with one multiplication less: the inference
-// kernels keep W1, b1, W2 and b2 halved (exactly), so that their
-// pre-activations arrive halved.
-__device__ __forceinline__ float gelu_half(float zh) {
-  const float u = zh * fmaf(8.0f * (kGeluC * kGeluA), zh * zh, 2.0f * kGeluC);
-  return fmaf(zh, tanh_approx(u), zh);
+// gelu<true>(2 zh) of two values from their halves zh, bit for bit (every
+// step is the same operation scaled by a power of two), with one
+// multiplication less: the inference kernels keep W1, b1, W2 and b2 halved
+// (exactly), so that their pre-activations arrive halved.
+__device__ __forceinline__ f32x2 gelu_half2(f32x2 zh) {
+  constexpr float c3 = 8.0f * (kGeluC * kGeluA), c1 = 2.0f * kGeluC;
+  const f32x2 u = mul2(zh, fma2(pack2(c3, c3), mul2(zh, zh), pack2(c1, c1)));
+  float a, b;
+  unpack2(u, a, b);
+  return fma2(zh, pack2(tanh_approx(a), tanh_approx(b)), zh);
 }
 
 // dg/dz given the tanh of the forward pass.

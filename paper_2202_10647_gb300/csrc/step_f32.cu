@@ -50,29 +50,6 @@ template <int Q>
 constexpr float lam_easy() {
   return Q == 1 ? 1.5f : 1.0f;
 }
-constexpr int kEasyTerms = 18;
-// 1/k! for the Taylor terms of the streaming kernel (constant memory: the
-// term loop reads one entry per term at a warp-uniform index)
-__constant__ const float kInvFactF32[kEasyTerms + 1] = {
-    1.0f,
-    1.0f,
-    1.0f / 2,
-    1.0f / 6,
-    1.0f / 24,
-    1.0f / 120,
-    1.0f / 720,
-    1.0f / 5040,
-    1.0f / 40320,
-    1.0f / 362880,
-    1.0f / 3628800,
-    1.0f / 39916800,
-    1.0f / 479001600,
-    1.0f / 6227020800.0f,
-    1.0f / 87178291200.0f,
-    1.0f / 1307674368000.0f,
-    1.0f / 20922789888000.0f,
-    1.0f / 355687428096000.0f,
-    1.0f / 6402373705728000.0f};
 // Rates with W dt above this are recomputed in float-float arithmetic.
 constexpr float kLamPrecise = 1.0f / 64.0f;
 
@@ -209,16 +186,45 @@ __device__ __forceinline__ void append_records(const Scratch& S, int job, int c0
   }
 }
 
+// Whether the network may serve a cell with window rates lam (Eq. 1) of w
+// states.  The network kernel turns a cell down when 2 sum max(lam_net, floor) beta
+// + floor reaches pop_tol; with lam_net no smaller than lam lowered by twice
+// its validation bound, lam (1 + beta)^-2, that sum is at least 2 sum lam
+// gate.  A cell turned down here would be turned down there as well, unless
+// the network were further off than that, and takes Eq. 1 in either case.
+// (The bin and the range by the field's fast logarithm: 1e-6 off moves a
+// cell by a bin at most, well within the factor.)
+template <int WM>
+__device__ __forceinline__ bool net_candidate(const NetSelect& sel, int Z, const FieldF32& f,
+                                              int lo, int w, const float (&lam)[WM],
+                                              float lmax) {
+  // no gate is smaller than gate_min: most cells are turned down without a look
+  if (2.0f * lmax * sel.gate_min > sel.pop_tol || f.zero) return false;
+  if (!(f.lg >= sel.l2lo - 1e-4f && f.lg <= sel.l2hi + 1e-4f)) return false;
+  int bin = (int)floorf(fmaf(sel.bin_a, f.lg, sel.bin_b));
+  bin = min(max(bin, 0), sel.nbins - 1);
+  const float* g = sel.gate + bin * Z + lo;
+  float err = 0.0f;
+#pragma unroll
+  for (int r = 0; r < WM - 1; ++r)
+    if (r < w - 1) err = fmaf(lam[r], __ldg(g + r), err);
+  return 1.998f * err < sel.pop_tol;
+}
+
 // CONS (the call has ION_CONSERVATION_CHECK; a separate instantiation, so
 // that the other calls carry none of it): cmax becomes the larger of itself
 // and the bits of |sum_r v'_r - sum_r v_r| of each cell finished here.
-template <int Q, int WM, bool AD, bool CONS>
+// NET (the surrogate step's first kernel): cells the network may serve are left untouched
+// too, marked in net[j].
+template <int Q, int WM, bool AD, bool CONS, bool NET = false>
 __device__ __forceinline__ void easy_cells(const JobIO& J, const Policy& pol,
                                            const StagedF32& tab, const PlaneRows<Q>& P,
                                            int lane, int c0, const float (&Ev)[Q],
                                            const int (&lo)[Q], const int (&hi)[Q],
                                            const bool (&ok)[Q], bool uni, bool (&stiff)[Q],
-                                           float thr_lane, uint32_t& cmax) {
+                                           float thr_lane, uint32_t& cmax,
+                                           const NetSelect* sel = nullptr,
+                                           bool* net = nullptr) {
   int w[Q];
   float v[Q][WM];
 #pragma unroll
@@ -253,6 +259,10 @@ __device__ __forceinline__ void easy_cells(const JobIO& J, const Policy& pol,
 #pragma unroll
     for (int r = 0; r < WM - 1; ++r) lmax = fmaxf(lmax, lam[j][r]);
     stiff[j] = lmax > lam_easy<Q>();
+    if constexpr (NET) {
+      net[j] = w[j] >= 2 && net_candidate<WM>(*sel, J.Z, f, base, w[j], lam[j], lmax);
+      stiff[j] = stiff[j] || net[j];
+    }
     xl = fmaxf(xl, stiff[j] ? 0.0f : 2.0f * lmax);
   }
   // the warp's largest 2 max(W dt) (non-negative floats order like their
@@ -717,9 +727,8 @@ constexpr size_t lean_smem() {
   return sizeof(StagedF32) + (size_t)W * kStages * sizeof(LStage<Q>);
 }
 
-template <int Q, int W, bool CONS>
-__global__ void __maxnreg__(stream_regs<Q>())
-    ion_lean_kernel(const __grid_constant__ BatchArgs a) {
+template <int Q, int W, bool CONS, bool NET>
+__device__ __forceinline__ void lean_body(const BatchArgs& a, const NetSelect* sel) {
   static_assert(Q == 1 || Q == 2, "one 16-byte front copy per lane at most");
   static_assert(kRun == kStages, "a run of chunks fills the stages in order");
   using V = typename VecOf<Q>::T;
@@ -782,7 +791,8 @@ __global__ void __maxnreg__(stream_regs<Q>())
       cp_async_s<16>(s_base + s * kStageBytes + f_dst, f_src + (size_t)g * f_stride);
     cp_async_commit();
   };
-  // bit s: the chunk in stage s is cold (every cell below its cold field)
+  // bit s: the chunk in stage s is cold (every cell below its cold field; the
+  // surrogate step's first kernel takes none as cold, the network may serve it)
   uint32_t coldm = 0;
   auto issue_planes = [&](int s, uint32_t g) {
     if (g < nchunks) {
@@ -799,7 +809,7 @@ __global__ void __maxnreg__(stream_regs<Q>())
         w[j] = window_ok(lo[j], hj, Z) ? hj - lo[j] + 1 : 0;
         c = c && (w[j] <= 1 || fabsf(vget(e, j)) < tab.ecold[min(lo[j], ION_MAX_Z)]);
       }
-      const bool cold = __all_sync(kFull, c);
+      const bool cold = !NET && __all_sync(kFull, c);
       coldm = cold ? (coldm | (1u << s)) : (coldm & ~(1u << s));
       const uint32_t c0 = g * (uint32_t)kChunk + (uint32_t)(Q * lane);
       const uint32_t pd = s_base + s * kStageBytes + p_dst;
@@ -832,6 +842,7 @@ __global__ void __maxnreg__(stream_regs<Q>())
 
   const float thr_lane = lane < kEasyTerms ? kThrF32[lane] : __int_as_float(0x7f800000);
   uint32_t cmax = 0;  // largest |change of sum_k N_k| (bits), ION_CONSERVATION_CHECK
+  uint32_t plain = 0;  // NET: cells on Eq. 1's rates
   // Chunk k lives in stage k mod 4, and the wait discipline is that of
   // ion_stream_kernel: fronts three chunks ahead, planes two.
   uint32_t run_next = fetch_run();
@@ -929,15 +940,38 @@ __global__ void __maxnreg__(stream_regs<Q>())
       }
     } else {
       const int WMw = __reduce_max_sync(kFull, wl);
+      bool net[Q];
+#pragma unroll
+      for (int j = 0; j < Q; ++j) net[j] = false;
       if (WMw <= 2)
-        easy_cells<Q, 2, false, CONS>(J, a.pol, tab, st.P, lane, c0, Ev, lo, hi, ok, uni,
-                                       stiff, thr_lane, cmax);
+        easy_cells<Q, 2, false, CONS, NET>(J, a.pol, tab, st.P, lane, c0, Ev, lo, hi, ok, uni,
+                                           stiff, thr_lane, cmax, sel, net);
       else if (WMw <= 4)
-        easy_cells<Q, 4, false, CONS>(J, a.pol, tab, st.P, lane, c0, Ev, lo, hi, ok, uni,
-                                       stiff, thr_lane, cmax);
+        easy_cells<Q, 4, false, CONS, NET>(J, a.pol, tab, st.P, lane, c0, Ev, lo, hi, ok, uni,
+                                           stiff, thr_lane, cmax, sel, net);
       else
-        easy_cells<Q, 6, false, CONS>(J, a.pol, tab, st.P, lane, c0, Ev, lo, hi, ok, uni,
-                                       stiff, thr_lane, cmax);
+        easy_cells<Q, 6, false, CONS, NET>(J, a.pol, tab, st.P, lane, c0, Ev, lo, hi, ok, uni,
+                                           stiff, thr_lane, cmax, sel, net);
+      if constexpr (NET) {
+        unsigned m[Q], n = 0;
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+          m[j] = __ballot_sync(kFull, net[j]);
+          n += __popc(m[j]);
+          plain += ok[j] && hi[j] > lo[j] && !net[j] ? 1u : 0u;
+          stiff[j] = stiff[j] && !net[j];
+        }
+        if (n) {
+          unsigned i = 0;
+          if (lane == 0) i = atomicAdd(&a.ws.hdr[kHdrNet], n);
+          i = __shfl_sync(kFull, i, 0);
+#pragma unroll
+          for (int j = 0; j < Q; ++j) {
+            if (net[j]) sel->list[i + __popc(m[j] & ((1u << lane) - 1u))] = (uint32_t)(c0 + j);
+            i += __popc(m[j]);
+          }
+        }
+      }
       // stiff cells: their inputs (as loaded) go to the record queue
       append_records<Q>(a.ws, 0, c0, Ev, lo, hi, stiff, st.P, lane);
     }
@@ -946,7 +980,35 @@ __global__ void __maxnreg__(stream_regs<Q>())
   cp_async_wait<0>();
   if constexpr (CONS) warp_max_into(&a.ws.hdr[kHdrCons], cmax);
 
-  tail_records(a, kChunk, gw, TW, lane);
+  if constexpr (NET) {
+    plain = __reduce_add_sync(kFull, plain);
+    if (lane == 0 && plain) atomicAdd(&a.ws.hdr[kHdrPlain], plain);
+    // the last, partial chunk is the network kernel's, which decides on every cell itself
+    if (gw == TW - 1) {
+      const int tail0 = (J.ncells / kChunk) * kChunk, n = J.ncells - tail0;
+      unsigned i = 0;
+      if (lane == 0 && n) i = atomicAdd(&a.ws.hdr[kHdrNet], (unsigned)n);
+      i = __shfl_sync(kFull, i, 0);
+      for (int t = lane; t < n; t += 32) sel->list[i + t] = (uint32_t)(tail0 + t);
+    }
+  } else {
+    tail_records(a, kChunk, gw, TW, lane);
+  }
+}
+
+template <int Q, int W, bool CONS>
+__global__ void __maxnreg__(stream_regs<Q>())
+    ion_lean_kernel(const __grid_constant__ BatchArgs a) {
+  lean_body<Q, W, CONS, false>(a, nullptr);
+}
+
+// The surrogate step's first kernel: the same over the cells the network could
+// not serve.
+template <int Q, int W>
+__global__ void __maxnreg__(stream_regs<Q>())
+    ion_net_select_kernel(const __grid_constant__ BatchArgs a,
+                          const __grid_constant__ NetSelect sel) {
+  lean_body<Q, W, false, true>(a, &sel);
 }
 
 // The stiff-cell records, one per thread.  W bounds the width; the window
@@ -1119,6 +1181,7 @@ struct StreamVariant {
   bool adaptive;
   bool lean;  // ion_lean_kernel (one species, the paper's window rule)
   bool cons;  // ION_CONSERVATION_CHECK
+  bool net;   // ion_net_select_kernel
   size_t (*smem)(int);
 };
 
@@ -1135,7 +1198,7 @@ size_t lean_smem_of(int) {
 #define ION_VARIANT(Q, W, AD, C)                                                     \
   {                                                                                  \
     reinterpret_cast<const void*>(&ion_stream_kernel<Q, W, AD, C>), Q, W, AD, false, C, \
-        &smem_of<Q, W>                                                               \
+        false, &smem_of<Q, W>                                                               \
   }
 #define ION_VARIANTS(AD, C)                                                       \
   ION_VARIANT(1, 2, AD, C), ION_VARIANT(1, 4, AD, C), ION_VARIANT(1, 8, AD, C),    \
@@ -1144,23 +1207,26 @@ size_t lean_smem_of(int) {
 #define ION_LEAN(Q, W, C)                                                              \
   {                                                                                    \
     reinterpret_cast<const void*>(&ion_lean_kernel<Q, W, C>), Q, W, false, true, C,      \
-        &lean_smem_of<Q, W>                                                            \
+        false, &lean_smem_of<Q, W>                                                            \
   }
 #define ION_LEANS(C)                                                              \
   ION_LEAN(1, 2, C), ION_LEAN(1, 4, C), ION_LEAN(1, 8, C), ION_LEAN(2, 2, C),      \
       ION_LEAN(2, 4, C), ION_LEAN(2, 8, C)
 const StreamVariant kVariants[] = {ION_VARIANTS(false, false), ION_VARIANTS(true, false),
                                    ION_VARIANTS(false, true),  ION_VARIANTS(true, true),
-                                   ION_LEANS(false),           ION_LEANS(true)};
+                                   ION_LEANS(false),           ION_LEANS(true),
+                                   {reinterpret_cast<const void*>(&ion_net_select_kernel<2, 8>), 2,
+                                    8, false, true, false, true, &lean_smem_of<2, 8>}};
 #undef ION_LEANS
 #undef ION_LEAN
 #undef ION_VARIANTS
 #undef ION_VARIANT
 
 const StreamVariant* find_variant(int Q, int W, bool adaptive = false, bool lean = false,
-                                  bool cons = false) {
+                                  bool cons = false, bool net = false) {
   for (const auto& v : kVariants)
-    if (v.Q == Q && v.W == W && v.adaptive == adaptive && v.lean == lean && v.cons == cons)
+    if (v.Q == Q && v.W == W && v.adaptive == adaptive && v.lean == lean && v.cons == cons &&
+        v.net == net)
       return &v;
   return nullptr;
 }
@@ -1276,6 +1342,26 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
   if ((e = cudaLaunchKernel(v->fn, blocks, v->W * 32, args, smem, s)) != cudaSuccess) return e;
   if ((e = launch_stiff_f32(a, num_sms, s)) != cudaSuccess) return e;
   return launch_fb_f32(a, num_sms, s);
+}
+
+cudaError_t launch_net_select_f32(BatchArgs& a, const NetSelect& sel, int num_sms, bool* fits,
+                                  cudaStream_t s) {
+  const StreamVariant* v = find_variant(2, 8, false, true, false, true);
+  *fits = v && lean_fits(a, 2);
+  if (!*fits) return cudaSuccess;
+  a.job[0].chunk0 = 0;
+  a.nchunks = a.job[0].ncells / 64;
+  const size_t smem = v->smem(1);
+  int fit = 0;
+  cudaError_t e = resident_blocks(*v, 1, smem, &fit);
+  if (e != cudaSuccess) return e;
+  if (fit < 1) return cudaErrorInvalidConfiguration;
+  const int64_t need = ((int64_t)a.nchunks + v->W - 1) / v->W;
+  int blocks = (int)(need < (int64_t)fit * num_sms ? need : (int64_t)fit * num_sms);
+  if (blocks < 1) blocks = 1;  // the tail still needs a warp
+  NetSelect n = sel;
+  void* args[] = {&a, &n};
+  return cudaLaunchKernel(v->fn, blocks, v->W * 32, args, smem, s);
 }
 
 // The record kernel's grid is one wave of resident blocks: a second, partial

@@ -1,8 +1,9 @@
 // surrogate.cu -- the rate surrogate at inference on the tensor cores.
 //
-// One CTA of 128 threads owns a tile of 128 cells at a time (thread t <->
-// cell t of the tile <-> row t of the MMAs <-> lane t of tensor memory):
-//   1. each thread evaluates layer 1 of its cell (one input, 64 GELUs),
+// A CTA owns a tile of 128 cells at a time: four network warps (thread t <->
+// cell t of the tile <-> row t of the MMAs <-> lane t of tensor memory) and
+// four cell warps (thread 128 + t <-> cell t), a tile behind them:
+//   1. each network thread evaluates layer 1 of its cell (one input, 64 GELUs),
 //      splits h1 into bf16 pairs, hi = bf16(h1) and lo = bf16(h1 - hi) (the
 //      weights are split the same way), and stores both parts in its lane
 //      of tensor memory (tcgen05.st), where the MMAs read the A operand;
@@ -14,18 +15,20 @@
 //      its training error rather than bf16 rounding (a 1-64-64-18 network
 //      on Ar-like rates: median rate error 0.5 % against 2 % with single
 //      bf16 operands);
-//   3. every thread reads its row of the accumulators (tcgen05.ld), adds b2,
+//   3. every network thread reads its row of the accumulators (tcgen05.ld), adds b2,
 //      applies the GELU and stores h2 (hi and lo) over h1;
 //   4. layer 3 likewise (N = the output count padded to 16, 32, 48 or 64),
 //      reusing the same accumulator columns;
-//   5. the outputs, scaled to log2 W, are staged column-major in shared
-//      memory (conflict-free for any window position), and each thread
-//      finishes its cell: ion_surrogate_rates writes all Z rates;
+//   5. the outputs are handed over column-major in shared memory
+//      (conflict-free for any window position), and each cell thread scales those
+//      it needs to log2 W: ion_surrogate_rates writes all Z rates;
 //      ion_step_surrogate picks the window's rates (network or Eq. 1, by the
 //      validation bound) and finishes cells whose rates all have W dt <= 1
 //      with the Taylor form.  Cells with a larger rate become records for
 //      ion_step's record kernel (Bateman form, rates of Eq. 1), followed by
-//      its FP64-coefficient pass.
+//      its FP64-coefficient pass.  Where it can, the step first runs the
+//      streaming kernel over the cells the network could not serve, and the
+//      network kernel on a list of the others.
 // Waits on the mbarrier are bounded; a wait that gives up marks the call as
 // failed (header word / NaN rates), frees the tensor memory and returns.
 #include <algorithm>
@@ -45,7 +48,8 @@ namespace sg {
 
 using mlp::H;
 
-constexpr int kM = 128;            // cells per tile = MMA M = threads per CTA
+constexpr int kM = 128;            // cells per tile = MMA M
+constexpr int kCta = 2 * kM;       // threads per CTA: network warps and cell warps
 // Tensor memory per CTA: columns [0, 64) the accumulators (layer 3 reuses
 // them), [64, 96) the hi parts of the A operand (two bf16 per 32-bit column,
 // the lower K index in the low half), [96, 128) its lo parts.
@@ -54,7 +58,7 @@ constexpr uint32_t kColAhi = 64, kColAlo = 96;
 constexpr uint32_t kSpinLimit = 1u << 22;
 
 // Scalars and short vectors of the network and its scaling.
-struct Consts {
+struct alignas(16) Consts {
   float W1h[H], b1h[H], b2h[H];  // W1, b1, b2 halved (the W2 image is halved too)
   float yoff[64], yscale[64];    // log2 W_k = yscale_k acc_k + yoff_k
   float xa, xb;        // x = xa log2|E| + xb
@@ -164,11 +168,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// A pair of activations as bf16 pairs (mlp::split_round): hi holds
-// bf16(a), bf16(b); lo holds the rounded remainders.
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+// Two activations as bf16 pairs (mlp::split_round): hi holds bf16(a),
+// bf16(b); lo holds the rounded remainders.
+__device__ __forceinline__ void split2(f32x2 g, uint32_t& hi, uint32_t& lo) {
+  float a, b;
+  unpack2(g, a, b);
   hi = pack_bf16(a, b);
-  lo = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+  const f32x2 h = pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+  unpack2(fma2(h, pack2(-1.0f, -1.0f), g), a, b);  // g - h, exact
+  lo = pack_bf16(a, b);
 }
 
 // 8 columns of this thread's lane from 8 registers.
@@ -194,20 +202,34 @@ __device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
       : "memory");
 }
 
-// One layer's products for the 128-row tile once every thread has stored its
+// Named barriers of a CTA (0 is __syncthreads): the network warps among
+// themselves; Y written (network warps arrive, cell warps wait); Y read (the
+// other way round).
+constexpr int kBarNet = 1, kBarYFull = 2, kBarYFree = 3;
+template <int Id, int N>
+__device__ __forceinline__ void bar_sync() {
+  asm volatile("bar.sync %0, %1;" ::"n"(Id), "n"(N) : "memory");
+}
+template <int Id, int N>
+__device__ __forceinline__ void bar_arrive() {
+  asm volatile("bar.arrive %0, %1;" ::"n"(Id), "n"(N) : "memory");
+}
+
+// One layer's products for the 128-row tile once every network thread has stored its
 // row of the A operand (hi and lo parts) in tensor memory: per 16-wide slice
 // kk of K, A_hi W_hi + A_hi W_lo + A_lo W_hi into the accumulators.  Every
-// thread calls this; thread 0 issues.  Returns false if the bounded wait
-// gave up (the tile is then skipped, and the CTA's drain waits for the
-// commit in flight).  dead_first: the wait polls `sdead` instead (the test
-// hook of ion_surrogate_test_timeout).
+// network thread calls this; thread 0 issues, the first warp waits for the
+// commit and the others sleep at the barrier.  Returns false if the bounded wait
+// gave up (*gave_up is set; the CTA's drain waits for the commit in flight).
+// dead_first: the wait polls `sdead` instead (the test hook of
+// ion_surrogate_test_timeout).
 __device__ __forceinline__ bool layer_products(uint32_t tmem, uint32_t sBhi, uint32_t sBlo,
                                                uint32_t idesc, int t, uint32_t sbar,
                                                uint32_t& phase, bool dead_first,
-                                               uint32_t sdead) {
+                                               uint32_t sdead, volatile uint32_t* gave_up) {
   tmem_wait_st();
   tc_fence_before();
-  __syncthreads();
+  bar_sync<kBarNet, kM>();
   if (t == 0) {
     tc_fence_after();
 #pragma unroll
@@ -219,11 +241,13 @@ __device__ __forceinline__ bool layer_products(uint32_t tmem, uint32_t sBhi, uin
     }
     mma_commit(sbar);
   }
-  const bool ok = dead_first ? mbar_wait(sdead, 0u, 64u) : mbar_wait(sbar, phase);
+  if (t < 32 && !(dead_first ? mbar_wait(sdead, 0u, 64u) : mbar_wait(sbar, phase)))
+    *gave_up = 1u;
+  __syncwarp();
   phase ^= 1u;
-  if (__syncthreads_or(!ok)) return false;
+  bar_sync<kBarNet, kM>();
   tc_fence_after();
-  return true;
+  return *gave_up == 0u;
 }
 
 // ---- shared-memory plan ---------------------------------------------------
@@ -241,7 +265,7 @@ __host__ __device__ constexpr Plan plan_of(int KP) {
   p.tab = p.consts + (uint32_t)((sizeof(Consts) + 15) / 16 * 16);
   p.bar = p.tab + (uint32_t)((sizeof(StagedF32) + 15) / 16 * 16);
   p.slot = p.bar + 16;  // two barriers: the MMA commits', and one never arrived at
-  p.total = p.slot + 8 + 1024;  // + slack for aligning the base to 1024
+  p.total = p.slot + 16 + 1024;  // + slack for aligning the base to 1024
   return p;
 }
 
@@ -255,30 +279,54 @@ struct StepArgs {
   int64_t ldw;
   int64_t ncells;
   const float* E;
+  // step mode: the cells to take (the number in header word kHdrNet), or
+  // nullptr for all of [0, ncells)
+  const uint32_t* list;
 };
 
-// Taylor-form update of one cell whose rates all have W dt <= 1 (w <= WM,
-// v its window's populations, zero past w): the same series, window slide
-// and stores as ion_step's streaming kernel.  WM: the warp's width bound.
+// A warp's cells whose rates all have W dt <= 1, in the Taylor form of the
+// streaming kernel (w states in lane, at most WM; lanes with w < 2 do
+// nothing).  The warp runs `terms` terms, those of its largest rate; a lane
+// adds the terms its own x = 2 max(W dt) asks for (thr_lane: kThrF32[lane]), so that
+// its result does not depend on the cells beside it in the list, whose order
+// varies.  v and lam hold zeros past w and w - 1.
 template <int WM>
-__device__ __forceinline__ void taylor_cell(const StepArgs& a, int c, int lo, int hi,
-                                            const float (&v6)[ION_MAX_WINDOW],
-                                            const float (&lam6)[ION_MAX_WINDOW], float lmax) {
+__device__ __forceinline__ void taylor_cells(const StepArgs& a, int c, int lo, int w,
+                                             const float (&v6)[ION_MAX_WINDOW],
+                                             const float (&lam6)[ION_MAX_WINDOW], int terms,
+                                             float x, float thr_lane) {
   const JobIO& J = a.J;
-  float* __restrict__ N = static_cast<float*>(J.N);
-  const int w = hi - lo + 1;
-  float dne = 0.0f;
-  int nlo = lo, nhi = hi;
-  if (w >= 2) {
-    float v[WM], lam[WM];
+  float u[WM - 1], inc[WM - 1], dne = 0.0f;
 #pragma unroll
-    for (int r = 0; r < WM; ++r) {
-      v[r] = v6[r];
-      lam[r] = lam6[r];
+  for (int r = 0; r < WM - 1; ++r) {
+    u[r] = v6[r];
+    inc[r] = 0.0f;
+  }
+#pragma unroll 1
+  for (int k = 1; k <= terms; ++k) {
+    const float ck = x > __shfl_sync(kFull, thr_lane, k - 1) ? kInvFactF32[k] : 0.0f;
+#pragma unroll
+    for (int i = WM - 2; i >= 0; --i) {
+      u[i] = fmaf(-lam6[i], u[i], i > 0 ? lam6[i - 1] * u[i - 1] : 0.0f);
+      inc[i] = fmaf(u[i], ck, inc[i]);
     }
-    dne = taylor_propagate<float, WM>(v, lam, w, lmax);
-    window_after_step<float, WM>(J, a.pol, v, w, nlo, nhi);
-    float* q = N + (int64_t)lo * J.ld + c;
+  }
+  if (w < 1) return;
+  // the window's top by conservation, whatever the bound WM
+  float v[WM], cum = 0.0f;
+#pragma unroll
+  for (int r = 0; r < WM; ++r) {
+    v[r] = v6[r];
+    if (r < w - 1) {
+      v[r] += inc[r];
+      cum -= inc[r];  // population that left states <= r
+      dne += cum;
+    } else if (r == w - 1) {
+      v[r] += cum;
+    }
+  }
+  if (w >= 2) {
+    float* __restrict__ q = static_cast<float*>(J.N) + (int64_t)lo * J.ld + c;
 #pragma unroll
     for (int r = 0; r < WM; ++r) {
       if (r < w) __stcs(q, v[r]);
@@ -287,9 +335,13 @@ __device__ __forceinline__ void taylor_cell(const StepArgs& a, int c, int lo, in
   }
   const float* __restrict__ G = static_cast<const float*>(J.n_gas);
   __stcs(static_cast<float*>(J.dne) + c, G ? dne * G[c] : dne);
-  if (nlo != lo || nhi != hi) {
-    J.lo[c] = (uint8_t)nlo;
-    J.hi[c] = (uint8_t)nhi;
+  if (w >= 2) {
+    int nlo = lo, nhi = lo + w - 1;
+    window_after_step<float, WM>(J, a.pol, v, w, nlo, nhi);
+    if (nlo != lo || nhi != lo + w - 1) {
+      J.lo[c] = (uint8_t)nlo;
+      J.hi[c] = (uint8_t)nhi;
+    }
   }
 }
 
@@ -313,44 +365,53 @@ __device__ __forceinline__ void eq1_rates(const StagedF32& tab, int lo, int w, f
     if (lam[r] > 1.0f / 64.0f) lam[r] = rate_ff_f32(tab, lo + r, f);
 }
 
-// Counts the lanes with `take` set into *counter (one atomic per warp).
-__device__ __forceinline__ void warp_count(uint32_t* counter, bool take) {
-  const unsigned m = __ballot_sync(kFull, take);
-  if ((threadIdx.x & 31) == 0 && m) atomicAdd(counter, (unsigned)__popc(m));
-}
-
+// The network for tiles of 128 cells.  A CTA is two groups of four warps:
+// the network warps (thread t: row t) evaluate the layers of tile i + 1
+// while the cell warps (thread 128 + t: cell t) finish tile i, loads and all;
+// Y, the outputs between them, is handed over by two named barriers.  Per
+// cell the two groups have about as many instructions (770 in the layers, as
+// packed pairs of units); as one group of 128 threads doing one after the other,
+// a CTA's tile took 15,000 cycles, most of them the cell part's latency, and
+// neither packed arithmetic nor two threads per row changed that.  12.8M cells
+// of an 18-state ladder: 1.34 ms as one group, 1.25 with two threads per row, 0.96 now.
 template <bool Step, int KP>
-__global__ void __launch_bounds__(kM) surrogate_kernel(const Dev* __restrict__ dev,
-                                                       const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(kCta, 4) surrogate_kernel(const Dev* __restrict__ dev,
+                                                            const __grid_constant__ StepArgs a) {
   extern __shared__ unsigned char smem_raw[];
   constexpr Plan P = plan_of(KP);
   // align the base to 1024 bytes (the swizzle atoms)
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char* base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-  float* Y = reinterpret_cast<float*>(base);  // output staging Y[k][128]
+  float* Y = reinterpret_cast<float*>(base);  // the accumulators of layer 3, Y[k][128]
   Consts& K = *reinterpret_cast<Consts*>(base + P.consts);
   StagedF32& tab = *reinterpret_cast<StagedF32*>(base + P.tab);
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + P.bar);
   uint32_t* slot = reinterpret_cast<uint32_t*>(base + P.slot);
+  volatile uint32_t* gave_up = slot + 1;  // the network warps' own
+  // what the cell warps see of it: written between YFree and YFull only, so
+  // that all of them see it in the same tile
+  volatile uint32_t* y_bad = slot + 2;
   const int t = threadIdx.x;
   const int warp = t >> 5;
+  const int row = t & (kM - 1);
 
   // stage the operands and constants
   {
     for (int h = 0; h < 2; ++h) {
       const uint4* s2 = reinterpret_cast<const uint4*>(dev->W2img[h]);
       uint4* d2 = reinterpret_cast<uint4*>(base + P.w2 + h * 8192);
-      for (int i = t; i < 8192 / 16; i += kM) d2[i] = s2[i];
+      for (int i = t; i < 8192 / 16; i += kCta) d2[i] = s2[i];
       const uint4* s3 = reinterpret_cast<const uint4*>(dev->W3img[h]);
       uint4* d3 = reinterpret_cast<uint4*>(base + P.w3 + h * KP * 128);
-      for (int i = t; i < KP * 128 / 16; i += kM) d3[i] = s3[i];
+      for (int i = t; i < KP * 128 / 16; i += kCta) d3[i] = s3[i];
     }
     const uint32_t* sc = reinterpret_cast<const uint32_t*>(&dev->k);
     uint32_t* dc = reinterpret_cast<uint32_t*>(&K);
-    for (int i = t; i < (int)(sizeof(Consts) / 4); i += kM) dc[i] = sc[i];
+    for (int i = t; i < (int)(sizeof(Consts) / 4); i += kCta) dc[i] = sc[i];
     stage_f32(&dev->tab, a.pol.log2dt, &tab);
   }
   if (t == 0) {
+    *gave_up = 0u;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(1)
                  : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar + 1)), "r"(1)
@@ -369,196 +430,256 @@ __global__ void __launch_bounds__(kM) surrogate_kernel(const Dev* __restrict__ d
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *slot;
-  const uint32_t tlane = tmem + ((uint32_t)(warp * 32) << 16);
-  const uint32_t sW2 = smem_u32(base + P.w2), sW3 = smem_u32(base + P.w3);
   const uint32_t sbar = smem_u32(bar);
-  // Test hook: the first wait of a tile polls, 64 times, a second barrier
-  // that nothing arrives at, so that it gives up while the layer-2 MMAs are
-  // in flight and the timeout path below runs (the drain at the end then
-  // waits, with the full limit, for the commit it skipped).
-  const uint32_t sdead = smem_u32(bar + 1);
-  const bool dead_wait = K.dead_wait != 0;
   const int Z = K.Z;
-  const float log2dt = (float)a.pol.log2dt;
-
   uint32_t phase = 0;
-  bool failed = false;
-  const int64_t ntiles = (a.ncells + kM - 1) / kM;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t c = tile * kM + t;
-    const bool on = c < a.ncells;
-    if (failed) {  // after a timeout: no tensor-core work, mark the outputs
-      if (!Step && on)
-        for (int k = 0; k < Z; ++k) a.W_out[(int64_t)k * a.ldw + c] = __int_as_float(0x7fc00000);
-      continue;
-    }
-    __syncthreads();  // every thread is done with the previous tile's Y
-    const float Eabs = on ? fabsf(a.E[c]) : 1.0f;
-    // the step's window populations, loaded now so that the loads are in
-    // flight while the network is evaluated
-    int clo = 0, chi = 0;
-    bool valid = false;
-    float v[ION_MAX_WINDOW];
+  bool failed = false;  // uniform in each group; the cell warps follow a tile later
+  const int64_t ncells = Step && a.list ? (int64_t)a.ws.hdr[kHdrNet] : a.ncells;
+  const int64_t ntiles = (ncells + kM - 1) / kM;
+  // cell `row` of a tile (its place in the list)
+  auto cell_of = [&](int64_t tile) -> int64_t {
+    const int64_t i = tile * kM + row;
+    return Step && a.list && i < ncells ? (int64_t)a.list[i] : i;
+  };
+  // log2|E|, and whether E has one
+  auto log2_field = [&](float Eabs, bool& pos) {
+    pos = Eabs > (float)kEmin && Eabs < INFINITY;
+    return log2f(pos ? Eabs : 1.0f);
+  };
+  // Whether the network could serve a cell at all: field in the trained range, a
+  // rate in the window.  Without a list both groups skip a tile none of
+  // whose cells it could serve.
+  auto servable = [&](bool pos, float l2, bool valid, int lo, int hi) {
+    return valid && hi > lo && pos && l2 >= K.l2lo && l2 <= K.l2hi && !a.pol.zero_dt &&
+           a.pop_tol > 0.0f;
+  };
+
+  if (t < kM) {
+    // ---- network warps
+    const uint32_t tlane = tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t sW2 = smem_u32(base + P.w2), sW3 = smem_u32(base + P.w3);
+    // Test hook: the first wait of a tile polls, 64 times, a second barrier
+    // that nothing arrives at, so that it gives up while the layer-2 MMAs are
+    // in flight and the timeout path below runs (the drain at the end then
+    // waits, with the full limit, for the commit it skipped).
+    const uint32_t sdead = smem_u32(bar + 1);
+    const bool dead_wait = K.dead_wait != 0;
+    bool handed = false;  // some tile's Y has been handed over
+    float E = 1.0f;
+    if (blockIdx.x * (int64_t)kM + row < ncells) E = a.E[cell_of(blockIdx.x)];
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      const int64_t next = tile + gridDim.x;
+      const bool more = next * kM + row < ncells;
+      const int64_t cnext = more ? cell_of(next) : 0;  // in flight during layer 1
+      bool pos;
+      const float l2 = log2_field(fabsf(E), pos);
+      bool use_net = true;
+      if constexpr (Step) {
+        if (!a.list && !failed) {
+          const int64_t c = tile * kM + row;
+          bool mine = false;
+          if (c < ncells) {
+            const int lo = a.J.lo[c], hi = a.J.hi[c];
+            mine = servable(pos, l2, window_ok(lo, hi, a.J.Z), lo, hi);
+          }
+          use_net = __syncthreads_or(mine) != 0;
+        }
+      }
+      if (failed) continue;
+      const float x = fminf(fmaxf(fmaf(K.xa, l2, K.xb), -1.0f), 1.0f);
+      if (use_net) {
+        const f32x2 x2 = pack2(x, x);
+        // layer 1 -> this thread's row of the A operand in tensor memory, as
+        // bf16 pairs (hi parts from column kColAhi, lo parts from kColAlo), 8
+        // columns (16 activations) at a time
 #pragma unroll
-    for (int r = 0; r < ION_MAX_WINDOW; ++r) v[r] = 0.0f;
-    if constexpr (Step) {
-      if (on) {
-        clo = a.J.lo[c];
-        chi = a.J.hi[c];
-        valid = window_ok(clo, chi, a.J.Z);
-        if (valid) {
-          const float* p = static_cast<const float*>(a.J.N) + (int64_t)clo * a.J.ld + c;
+        for (int q = 0; q < 4; ++q) {
+          uint32_t hi[8], lo[8];
+#pragma unroll
+          for (int j = 0; j < 8; j += 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&K.W1h[16 * q + 2 * j]);
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&K.b1h[16 * q + 2 * j]);
+            split2(mlp::gelu_half2(fma2(w.x, x2, b.x)), hi[j], lo[j]);
+            split2(mlp::gelu_half2(fma2(w.y, x2, b.y)), hi[j + 1], lo[j + 1]);
+          }
+          tmem_st8(tlane + kColAhi + 8 * q, hi);
+          tmem_st8(tlane + kColAlo + 8 * q, lo);
+        }
+      }
+      if (more) E = a.E[cnext];
+      if (!use_net) continue;
+      failed = !layer_products(tmem, sW2, sW2 + 8192, idesc_bf16(kM, H), t, sbar, phase,
+                               dead_wait, sdead, gave_up);
+      if (!failed) {
+        // layer 2 epilogue: h2 = g(acc + b2) -> the A operand (layer 2 has read
+        // it), 16 accumulator columns at a time
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          float v[16];
+          tmem_ld16(tlane + ch * 16, v);
+          uint32_t hi[8], lo[8];
+#pragma unroll
+          for (int j = 0; j < 8; j += 2) {
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&K.b2h[16 * ch + 2 * j]);
+            split2(mlp::gelu_half2(add2(pack2(v[2 * j], v[2 * j + 1]), b.x)), hi[j], lo[j]);
+            split2(mlp::gelu_half2(add2(pack2(v[2 * j + 2], v[2 * j + 3]), b.y)), hi[j + 1],
+                   lo[j + 1]);
+          }
+          tmem_st8(tlane + kColAhi + 8 * ch, hi);
+          tmem_st8(tlane + kColAlo + 8 * ch, lo);
+        }
+        failed = !layer_products(tmem, sW3, sW3 + KP * 128, idesc_bf16(kM, KP), t, sbar, phase,
+                                 false, sdead, gave_up);
+      }
+      if (handed) bar_sync<kBarYFree, kCta>();  // the cell warps have read the last Y
+      if (!failed) {
+        // layer 3 epilogue: the accumulators -> Y[k][row]; the readers, who need a
+        // window's states only, scale them
+#pragma unroll
+        for (int ch = 0; ch < KP / 16; ++ch) {
+          float v[16];
+          tmem_ld16(tlane + ch * 16, v);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int k = ch * 16 + j;
+            if (k < Z) Y[k * kM + row] = v[j];
+          }
+        }
+        tc_fence_before();
+      }
+      if (t == 0) *y_bad = failed ? 1u : 0u;
+      handed = true;
+      bar_arrive<kBarYFull, kCta>();
+    }
+    if (handed && !failed) bar_sync<kBarYFree, kCta>();  // the last tile's arrivals
+  } else {
+    // ---- cell warps
+    // log2 W_k of this thread's cell: ymean + yscale (acc + b3)
+    auto network_log2 = [&](int k) { return fmaf(K.yscale[k], Y[k * kM + row], K.yoff[k]); };
+    const float log2dt = (float)a.pol.log2dt;
+    const float wfloor = exp2f(K.yfloor + log2dt);
+    const int lane = t & 31;
+    // the cell waits for the network's outputs; false after a timeout
+    auto wait_outputs = [&]() {
+      bar_sync<kBarYFull, kCta>();
+      return *y_bad == 0u;
+    };
+    if constexpr (!Step) {
+      for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t c = tile * kM + row;
+        if (!failed) failed = !wait_outputs();
+        if (c < ncells)
+          for (int k = 0; k < Z; ++k) {
+            float W = __int_as_float(0x7fc00000);  // NaN after a timeout
+            if (!failed) {
+              const float s = network_log2(k);
+              W = s < K.yfloor ? 0.0f : exp2f(s);
+            }
+            a.W_out[(int64_t)k * a.ldw + c] = W;
+          }
+        if (!failed) bar_arrive<kBarYFree, kCta>();
+      }
+    } else {
+      const float thr_lane =
+          lane < DDParams<float>::PMAX ? kThrF32[lane] : __int_as_float(0x7f800000);
+      // cells of this thread on the network's rates and on Eq. 1's, added to
+      // the header once at the end
+      uint32_t n_net = 0, n_plain = 0;
+      for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const bool on = tile * kM + row < ncells;
+        const int c = on ? (int)cell_of(tile) : 0;
+        float Ec = 1.0f;
+        int lo = 0, hi = 0;
+        if (on) {
+          Ec = a.E[c];
+          lo = a.J.lo[c];
+          hi = a.J.hi[c];
+        }
+        const bool valid = on && window_ok(lo, hi, a.J.Z);
+        const int w = valid ? hi - lo + 1 : 0;
+        float v[ION_MAX_WINDOW];
+        {
+          const float* p = static_cast<const float*>(a.J.N) + (int64_t)lo * a.J.ld + c;
 #pragma unroll
           for (int r = 0; r < ION_MAX_WINDOW; ++r) {
-            if (r < chi - clo + 1) v[r] = __ldcs(p);
+            v[r] = r < w ? __ldcs(p) : 0.0f;
             p += a.J.ld;
           }
         }
-      }
-    }
-    const bool pos = Eabs > (float)kEmin && Eabs < INFINITY;
-    const float l2 = log2f(pos ? Eabs : 1.0f);
-    const float x = fminf(fmaxf(fmaf(K.xa, l2, K.xb), -1.0f), 1.0f);
-    // the step skips the network for a tile none of whose cells could use
-    // it (field outside the trained range, no rate in the window, or the
-    // network never trusted); the decision is uniform over the CTA
-    bool use_net = true;
-    // the validation bounds of the window's states, loaded now (like the
-    // populations) so that the loads are in flight during the network
-    float beta[ION_MAX_WINDOW - 1];
+        bool pos;
+        const float l2 = log2_field(fabsf(Ec), pos);
+        const bool mine = servable(pos, l2, valid, lo, hi);
+        float beta[ION_MAX_WINDOW - 1];
 #pragma unroll
-    for (int r = 0; r < ION_MAX_WINDOW - 1; ++r) beta[r] = 0.0f;
-    if constexpr (Step) {
-      const bool mine = valid && chi > clo && pos && l2 >= K.l2lo && l2 <= K.l2hi &&
-                        !a.pol.zero_dt && a.pop_tol > 0.0f;
-      use_net = __syncthreads_or(mine) != 0;
-      if (mine && a.bound) {
-        int bin = (int)floorf(fmaf(K.bin_a, l2, K.bin_b));
-        bin = min(max(bin, 0), K.nbins - 1);
-        const float* bb = a.bound + bin * Z + clo;
+        for (int r = 0; r < ION_MAX_WINDOW - 1; ++r) beta[r] = 0.0f;
+        if (mine && a.bound) {
+          int bin = (int)floorf(fmaf(K.bin_a, l2, K.bin_b));
+          bin = min(max(bin, 0), K.nbins - 1);
+          const float* bb = a.bound + bin * Z + lo;
 #pragma unroll
-        for (int r = 0; r < ION_MAX_WINDOW - 1; ++r)
-          if (r < chi - clo) beta[r] = __ldg(bb + r);
-      }
-    }
-    if (use_net) {
-    // layer 1 -> this thread's row of the A operand in tensor memory, as
-    // bf16 pairs (hi parts from column kColAhi, lo parts from kColAlo), 8
-    // columns (16 activations) at a time
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int u = 16 * q + 2 * j;
-        split2(mlp::gelu_half(fmaf(K.W1h[u], x, K.b1h[u])),
-               mlp::gelu_half(fmaf(K.W1h[u + 1], x, K.b1h[u + 1])), hi[j], lo[j]);
-      }
-      tmem_st8(tlane + kColAhi + 8 * q, hi);
-      tmem_st8(tlane + kColAlo + 8 * q, lo);
-    }
-    if (!layer_products(tmem, sW2, sW2 + 8192, idesc_bf16(kM, H), t, sbar, phase, dead_wait,
-                        sdead)) {
-      failed = true;
-      if (!Step && on)
-        for (int k = 0; k < Z; ++k) a.W_out[(int64_t)k * a.ldw + c] = __int_as_float(0x7fc00000);
-      continue;
-    }
-    // layer 2 epilogue: h2 = g(acc + b2) -> the A operand (layer 2 has read
-    // it), 16 accumulator columns at a time
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-      float v[16];
-      tmem_ld16(tlane + ch * 16, v);
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int u = ch * 16 + 2 * j;
-        split2(mlp::gelu_half(v[2 * j] + K.b2h[u]), mlp::gelu_half(v[2 * j + 1] + K.b2h[u + 1]),
-               hi[j], lo[j]);
-      }
-      tmem_st8(tlane + kColAhi + 8 * ch, hi);
-      tmem_st8(tlane + kColAlo + 8 * ch, lo);
-    }
-    if (!layer_products(tmem, sW3, sW3 + KP * 128, idesc_bf16(kM, KP), t, sbar, phase, false,
-                        sdead)) {
-      failed = true;
-      if (!Step && on)
-        for (int k = 0; k < Z; ++k) a.W_out[(int64_t)k * a.ldw + c] = __int_as_float(0x7fc00000);
-      continue;
-    }
-    // layer 3 epilogue: log2 W_k = ymean + yscale (acc + b3) -> Y[k][t]
-#pragma unroll
-    for (int ch = 0; ch < KP / 16; ++ch) {
-      float v[16];
-      tmem_ld16(tlane + ch * 16, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int k = ch * 16 + j;
-        if (k < Z) Y[k * kM + t] = fmaf(K.yscale[k], v[j], K.yoff[k]);
-      }
-    }
-    tc_fence_before();
-    }  // use_net
-    if constexpr (!Step) {
-      if (on)
-        for (int k = 0; k < Z; ++k) {
-          const float s = Y[k * kM + t];
-          a.W_out[(int64_t)k * a.ldw + c] = s < K.yfloor ? 0.0f : exp2f(s);
+          for (int r = 0; r < ION_MAX_WINDOW - 1; ++r)
+            if (r < hi - lo) beta[r] = __ldg(bb + r);
         }
-    } else {
-      const int lo = clo, hi = chi;
-      if (on && !valid) atomicAdd(&a.ws.hdr[kHdrInvalid], 1u);
-      const int w = hi - lo + 1;
-      float lam[ION_MAX_WINDOW];
+        if (failed) continue;
+        bool use_net = true;
+        if (!a.list) use_net = __syncthreads_or(mine) != 0;
+        float lam[ION_MAX_WINDOW];
 #pragma unroll
-      for (int r = 0; r < ION_MAX_WINDOW; ++r) lam[r] = 0.0f;
-      bool net = false, plain = false;
-      if (valid && w >= 2 && !a.pol.zero_dt) {
-        const bool in_range = use_net && pos && l2 >= K.l2lo && l2 <= K.l2hi;
-        const float wfloor = exp2f(K.yfloor + log2dt);
-        float err = 0.0f;
-#pragma unroll
-        for (int r = 0; r < ION_MAX_WINDOW - 1; ++r) {
-          if (in_range && r < w - 1) {
-            const int k = lo + r;
-            const float s = Y[k * kM + t];
-            lam[r] = s < K.yfloor ? 0.0f : ex2_approx(s + log2dt);
-            err += 2.0f * fmaf(fmaxf(lam[r], wfloor), beta[r], wfloor);
+        for (int r = 0; r < ION_MAX_WINDOW; ++r) lam[r] = 0.0f;
+        bool net = false;
+        if (use_net) {
+          if (!wait_outputs()) {
+            failed = true;  // the results of the call are invalid
+            continue;
           }
+          if (mine) {
+            float err = 0.0f;
+#pragma unroll
+            for (int r = 0; r < ION_MAX_WINDOW - 1; ++r) {
+              if (r < w - 1) {
+                const float s = network_log2(lo + r);
+                lam[r] = s < K.yfloor ? 0.0f : ex2_approx(s + log2dt);
+                err += 2.0f * fmaf(fmaxf(lam[r], wfloor), beta[r], wfloor);
+              }
+            }
+            net = err < a.pop_tol;  // pop_tol 0: never the network
+          }
+          bar_arrive<kBarYFree, kCta>();
         }
-        net = in_range && err < a.pop_tol;  // pop_tol 0: never the network
-        if (!net) {
-          plain = true;
+        if (on && !valid) atomicAdd(&a.ws.hdr[kHdrInvalid], 1u);
+        const bool rates = w >= 2 && !a.pol.zero_dt;
+        if (rates && !net) {
 #pragma unroll
           for (int r = 0; r < ION_MAX_WINDOW; ++r) lam[r] = 0.0f;
-          eq1_rates(tab, lo, w, a.E[c], lam);
+          eq1_rates(tab, lo, w, Ec, lam);
         }
-      }
-      // cells with some W dt > 1 take the Bateman form in the record kernel,
-      // with the rates of Eq. 1 (their error bound is far above any useful
-      // tolerance, so the network could not serve them)
-      float lmax = 0.0f;
+        // cells with some W dt > 1 take the Bateman form in the record kernel,
+        // with the rates of Eq. 1 (their error bound is far above any useful
+        // tolerance, so the network could not serve them)
+        float lmax = 0.0f;
 #pragma unroll
-      for (int r = 0; r < ION_MAX_WINDOW; ++r) lmax = fmaxf(lmax, lam[r]);
-      const bool stiff = valid && lmax > DDParams<float>::prop_max;
-      net = net && !stiff;
-      plain = plain || stiff;
-      warp_count(&a.ws.hdr[kHdrSurrogate], net);
-      warp_count(&a.ws.hdr[kHdrPlain], plain);
-      if (__ballot_sync(kFull, stiff))
-        append_record(a.ws, stiff, 0, (int)c, on ? a.E[c] : 0.0f, lo, hi, v);
-      // the warp's widest window bounds the series for all its lanes
-      const int wt = (valid && !stiff) ? w : 0;
-      const int Wm = __reduce_max_sync(kFull, wt);
-      if (wt > 0) {
+        for (int r = 0; r < ION_MAX_WINDOW; ++r) lmax = fmaxf(lmax, lam[r]);
+        const bool stiff = lmax > DDParams<float>::prop_max;
+        net = net && !stiff;
+        n_net += net ? 1u : 0u;
+        n_plain += rates && !net ? 1u : 0u;
+        if (__ballot_sync(kFull, stiff)) append_record(a.ws, stiff, 0, c, Ec, lo, hi, v);
+        // the warp's widest window and largest rate bound the series for all its lanes
+        const int wt = stiff ? 0 : w;
+        const int Wm = __reduce_max_sync(kFull, wt);
+        const float x = stiff ? 0.0f : 2.0f * lmax;
+        const float xw = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(x)));
+        const int terms = __popc(__ballot_sync(kFull, xw > thr_lane));
         if (Wm <= 2)
-          taylor_cell<2>(a, (int)c, lo, hi, v, lam, lmax);
+          taylor_cells<2>(a, c, lo, wt, v, lam, terms, x, thr_lane);
         else if (Wm <= 4)
-          taylor_cell<4>(a, (int)c, lo, hi, v, lam, lmax);
+          taylor_cells<4>(a, c, lo, wt, v, lam, terms, x, thr_lane);
         else
-          taylor_cell<ION_MAX_WINDOW>(a, (int)c, lo, hi, v, lam, lmax);
+          taylor_cells<ION_MAX_WINDOW>(a, c, lo, wt, v, lam, terms, x, thr_lane);
       }
+      const uint32_t wn = __reduce_add_sync(kFull, n_net), wp = __reduce_add_sync(kFull, n_plain);
+      if (lane == 0 && wn) atomicAdd(&a.ws.hdr[kHdrSurrogate], wn);
+      if (lane == 0 && wp) atomicAdd(&a.ws.hdr[kHdrPlain], wp);
     }
   }
   // leave: tensor memory is freed by the warp that allocated it once every
@@ -627,7 +748,11 @@ struct ion_surrogate {
   int device, num_sms, Z, KP, nbins;
   int fit_rates, fit_step;  // resident CTAs per SM of the two kernels
   ion::sg::Dev* dev;
-  float* bound;  // device [nbins][Z] of 2^bound - 1, or nullptr
+  // device [2][nbins][Z], or nullptr: beta = 2^bound - 1, and the gates
+  // beta (1 + beta)^-2 of NetSelect
+  float* bound;
+  float gate_min;
+  float bin_a, bin_b;
   ion_surrogate_norm norm;
 };
 
@@ -684,12 +809,12 @@ cudaError_t prepare(const void* fn, int KP, int* fit) {
       (e = cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev)) ||
       (e = cudaDeviceGetAttribute(&blk_sm, cudaDevAttrMaxBlocksPerMultiprocessor, dev)))
     return e;
-  const int warps = ion::sg::kM / 32;
+  const int warps = ion::sg::kCta / 32;
   const int regs_warp = ((fa.numRegs + 7) / 8 * 8 * 32 + 255) / 256 * 256;
   int f = regs_sm / (regs_warp * warps);
   const int per_block_smem = (int)smem + (int)fa.sharedSizeBytes + smem_rsv;
   f = std::min(f, smem_sm / per_block_smem);
-  f = std::min(f, thr_sm / ion::sg::kM);
+  f = std::min(f, thr_sm / ion::sg::kCta);
   f = std::min(f, blk_sm);
   // tensor memory: the resident CTAs' columns must fit the SM's 512, so that
   // no allocation ever waits
@@ -708,7 +833,7 @@ cudaError_t launch(const ion_surrogate* s, bool step, const StepArgs& a, cudaStr
   const void* fn = step ? kernel_of<true>(s->KP) : kernel_of<false>(s->KP);
   const Dev* dev = s->dev;
   void* args[] = {(void*)&dev, (void*)&a};
-  return cudaLaunchKernel(fn, blocks, ion::sg::kM, args, ion::sg::plan_of(s->KP).total, st);
+  return cudaLaunchKernel(fn, blocks, ion::sg::kCta, args, ion::sg::plan_of(s->KP).total, st);
 }
 
 int check_surrogate(const ion_surrogate* s) {
@@ -722,6 +847,20 @@ int check_surrogate(const ion_surrogate* s) {
 
 bool al4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 
+// Appends the gates of the bounds beta[0..m) (NetSelect) and returns the
+// smallest.
+float append_gates(std::vector<float>& beta) {
+  const size_t m = beta.size();
+  float least = INFINITY;
+  beta.resize(2 * m);
+  for (size_t i = 0; i < m; ++i) {
+    const double b = beta[i];
+    beta[m + i] = (float)(b / ((1.0 + b) * (1.0 + b)));
+    least = std::min(least, beta[m + i]);
+  }
+  return least;
+}
+
 // Replaces the surrogate's bound by the host array b [nbins*Z] (log2 units):
 // the device copy holds 2^b - 1, and the bin mapping of the kernels' Consts
 // follows nbins.  Synchronous.
@@ -733,9 +872,11 @@ int install_bound(ion_surrogate* s, const float* b, int nbins) {
       return ion::set_error(ION_EINVAL, "bound[%zu] must be finite and >= 0", i);
     beta[i] = (float)(std::exp2((double)b[i]) - 1.0);
   }
+  const float gate_min = append_gates(beta);
   float* dst = nullptr;
-  cudaError_t e = cudaMalloc(&dst, sizeof(float) * m);
-  if (e == cudaSuccess) e = cudaMemcpy(dst, beta.data(), sizeof(float) * m, cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMalloc(&dst, sizeof(float) * 2 * m);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(dst, beta.data(), sizeof(float) * 2 * m, cudaMemcpyHostToDevice);
   const double span = s->norm.log2E_max - s->norm.log2E_min;
   const float bin_a = (float)(nbins / span);
   const float bin_b = (float)(-s->norm.log2E_min * nbins / span);
@@ -757,6 +898,9 @@ int install_bound(ion_surrogate* s, const float* b, int nbins) {
   if (s->bound) cudaFree(s->bound);
   s->bound = dst;
   s->nbins = nbins;
+  s->gate_min = gate_min;
+  s->bin_a = bin_a;
+  s->bin_b = bin_b;
   return ION_OK;
 }
 
@@ -852,6 +996,9 @@ int ion_surrogate_create(const ion_species* sp, const float* P, const ion_surrog
   s->Z = Z;
   s->KP = KP;
   s->nbins = nbins;
+  s->gate_min = append_gates(beta);
+  s->bin_a = img->k.bin_a;
+  s->bin_b = img->k.bin_b;
   s->dev = nullptr;
   s->bound = nullptr;
   s->norm = *norm;
@@ -1026,14 +1173,38 @@ int ion_step_surrogate(const ion_surrogate* s, const float* E, float* N, int64_t
   a.E = E;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemsetAsync(a.ws.hdr, 0, kHdrWords * sizeof(uint32_t), st);
+  BatchArgs b;
+  std::memset(&b, 0, sizeof b);
+  b.njobs = 1;
+  b.job[0] = J;
+  b.pol = a.pol;
+  b.ws = a.ws;
+  // With validation bounds, the cells the network could not serve are
+  // stepped by the streaming kernel, and the network kernel takes the others from a
+  // list (in the FP64 queue's place, which the record kernel fills after it).
+  // Otherwise, or for arrays and policies the streaming kernel does not
+  // take, the network kernel walks all cells.
+  if (e == cudaSuccess && ncells > 0 && s->bound && !a.pol.adaptive && !a.pol.zero_dt &&
+      a.pop_tol > 0.0f) {
+    const uintptr_t al = reinterpret_cast<uintptr_t>(E) | reinterpret_cast<uintptr_t>(N) |
+                         reinterpret_cast<uintptr_t>(dne);
+    b.job[0].vec = (al & 7u) == 0 && ld % 2 == 0;
+    NetSelect sel;
+    sel.gate = s->bound + (size_t)s->nbins * s->Z;
+    sel.gate_min = s->gate_min;
+    sel.nbins = s->nbins;
+    sel.bin_a = s->bin_a;
+    sel.bin_b = s->bin_b;
+    sel.l2lo = (float)s->norm.log2E_min;
+    sel.l2hi = (float)s->norm.log2E_max;
+    sel.pop_tol = a.pop_tol;
+    sel.list = a.ws.queue;
+    bool fits = false;
+    e = launch_net_select_f32(b, sel, s->num_sms, &fits, st);
+    if (fits) a.list = sel.list;
+  }
   if (e == cudaSuccess) e = launch(s, true, a, st);
   if (e == cudaSuccess && ncells > 0) {
-    BatchArgs b;
-    std::memset(&b, 0, sizeof b);
-    b.njobs = 1;
-    b.job[0] = J;
-    b.pol = a.pol;
-    b.ws = a.ws;
     e = launch_stiff_f32(b, s->num_sms, st);
     if (e == cudaSuccess) e = launch_fb_f32(b, s->num_sms, st);
   }
