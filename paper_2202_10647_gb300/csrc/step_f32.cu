@@ -30,6 +30,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "f32x2.cuh"
 #include "ion_cell.cuh"
 #include "ion_step.cuh"
 
@@ -277,24 +278,65 @@ __device__ __forceinline__ void easy_cells(const JobIO& J, const Policy& pol,
   // the stage holds there: their rates and the rate into them are zero, so
   // their u is zero after one term and their inc stays zero.  Stiff cells
   // run with rates above lam_easy; their inc is never read.
-  float u[Q][WM], inc[Q][WM];
+  float inc[Q][WM];
+  if constexpr (Q % 2 == 0) {
+    // Two cells per instruction (f32x2; the loop's issue slots halve: PAIRUS).
+    // U_i = (-1)^i u_i, so that both of the recurrence's rates carry one sign:
+    // u_i' = -lam_i u_i + lam_{i-1} u_{i-1}, U_i' = -lam_i U_i - lam_{i-1} U_{i-1}
+    f32x2 L[Q / 2][WM - 1], U[Q / 2][WM - 1], I[Q / 2][WM - 1];
 #pragma unroll
-  for (int j = 0; j < Q; ++j) {
+    for (int j = 0; j < Q / 2; ++j) {
 #pragma unroll
-    for (int i = 0; i < WM; ++i) {
-      u[j][i] = v[j][i];
-      inc[j][i] = 0.0f;
+      for (int i = 0; i < WM - 1; ++i) {
+        const float s = i % 2 ? -1.0f : 1.0f;
+        L[j][i] = pack2(-lam[2 * j][i], -lam[2 * j + 1][i]);
+        U[j][i] = pack2(s * v[2 * j][i], s * v[2 * j + 1][i]);
+        I[j][i] = 0ull;
+      }
     }
-  }
 #pragma unroll 1
-  for (int k = 1; k <= Rw; ++k) {
-    const float ck = kInvFactF32[k];
+    for (int k = 1; k <= Rw; ++k) {
+      const f32x2 ck = pack2(kInvFactF32[k], kInvFactF32[k]);
+#pragma unroll
+      for (int j = 0; j < Q / 2; ++j) {
+#pragma unroll
+        for (int i = WM - 2; i >= 0; --i) {
+          U[j][i] = i > 0 ? fma2(L[j][i], U[j][i], mul2(L[j][i - 1], U[j][i - 1]))
+                          : mul2(L[j][0], U[j][0]);
+          I[j][i] = fma2(U[j][i], ck, I[j][i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < Q / 2; ++j) {
+#pragma unroll
+      for (int i = 0; i < WM - 1; ++i) {
+        const float s = i % 2 ? -1.0f : 1.0f;
+        unpack2(I[j][i], inc[2 * j][i], inc[2 * j + 1][i]);
+        inc[2 * j][i] *= s;
+        inc[2 * j + 1][i] *= s;
+      }
+    }
+  } else {
+    float u[Q][WM];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
 #pragma unroll
-      for (int i = WM - 2; i >= 0; --i) {
-        u[j][i] = fmaf(-lam[j][i], u[j][i], i > 0 ? lam[j][i - 1] * u[j][i - 1] : 0.0f);
-        inc[j][i] = fmaf(u[j][i], ck, inc[j][i]);
+      for (int i = 0; i < WM; ++i) {
+        u[j][i] = v[j][i];
+        inc[j][i] = 0.0f;
+      }
+    }
+#pragma unroll 1
+    for (int k = 1; k <= Rw; ++k) {
+      const float ck = kInvFactF32[k];
+#pragma unroll
+      for (int j = 0; j < Q; ++j) {
+#pragma unroll
+        for (int i = WM - 2; i >= 0; --i) {
+          u[j][i] = fmaf(-lam[j][i], u[j][i], i > 0 ? lam[j][i - 1] * u[j][i - 1] : 0.0f);
+          inc[j][i] = fmaf(u[j][i], ck, inc[j][i]);
+        }
       }
     }
   }
