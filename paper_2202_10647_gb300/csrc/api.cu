@@ -1,11 +1,13 @@
 // api.cu -- the C ABI of ionize.h: species tables, argument checking, the
 // ion_rates kernel, and dispatch of ion_step to the FP32 or FP64 kernels.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
 #include <string>
 
+#include "f32x2.cuh"
 #include "ion_device.cuh"
 #include "ion_step.cuh"
 #include "ionize.h"
@@ -89,19 +91,149 @@ void build_table(const double* U, const int* l, const int* m, int Z,
 }
 
 // ---------------------------------------------------------------------------
-// ion_rates kernels: one thread per cell, rates of states k_lo..k_hi-1.
+// ion_rates in FP32: the exponent y = a - b log2|E| - C/|E| in float-float
+// arithmetic, as rate_ff_f32 forms it but from the accurate log2 and reciprocal
+// of the field, two cells per instruction (f32x2) and kPairs pairs per
+// thread, a block's width apart so that every store is contiguous whatever the
+// row length.  2^y is one SFU exponential: y's integer part n, exact to take from
+// the leading sum, scales the result.  Bound by the FMA pipe (15 packed
+// instructions per rate, 107 us of the case below) and by issue; species whose rates
+// need no clamp and no cutoff test in FP32 (all but absurd ones: RateRow) take
+// a loop without them.  4,000,001 fields x 36 states: 217 us as scalars with two
+// exponentials, 213 packed with predicated stores, clamp and test, 177 now (200 as a
+// persistent grid, whose seventh round of tiles is half empty); 88 us at the HBM rate.
 // ---------------------------------------------------------------------------
-__global__ void rates_f32_kernel(const ion::SpeciesTable* t, const float* E,
-                                 int ncells, int k_lo, int k_hi, float* W,
-                                 int64_t ldw) {
-  __shared__ ion::StagedF32 tab;
-  ion::stage_f32(t, 0.0, &tab);
-  __syncthreads();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncells) return;
-  const ion::FieldF32 f = ion::field_f32<true>(E[c]);
-  for (int k = k_lo; k < k_hi; ++k)
-    W[(int64_t)(k - k_lo) * ldw + c] = ion::rate_dt_f32<true>(tab, k, f);
+constexpr int kRateThreads = 256;
+constexpr int kPairs = 2;
+
+struct alignas(16) RateRow {
+  ion::f32x2 b_neg, b, C, a, C_lo, b_lo, a_lo, C_neg;  // each value twice
+};
+
+// Whether a state's rate is 0 in FP32 wherever the cutoff makes it 0, and
+// below the clamp at 2^99 at every field: at the cutoff C/E = kCutoffLog2 y is
+// below -160 and still rising with E (b < C/E ln 2), and its maximum over E (at E =
+// C ln 2 / b, or the largest float) is below 98.
+__device__ __forceinline__ bool tame_state(double a, double b, double C) {
+  const float af = (float)a, bf = (float)b, Cf = (float)C;
+  if (!(Cf > 1e-30f && Cf < 1e30f && fabsf(af) < 1e30f && fabsf(bf) < 600.0f)) return false;
+  const float at_cutoff = af - bf * log2f(Cf / (float)ion::kCutoffLog2) - (float)ion::kCutoffLog2;
+  const float peak = bf > 1e-3f ? af - bf * log2f(Cf * 0.6931472f / bf) - bf * 1.442695f
+                                : af - fminf(bf, 0.0f) * 128.0f + 1.0f;
+  return at_cutoff < -160.0f && peak < 98.0f;
+}
+
+// The rates of the block's cells.  Full: all of them exist.  Tame: all states
+// of the species are (tame_state).
+template <bool Full, bool Tame>
+__device__ __forceinline__ void rates_f32_rows(const RateRow* rows, int nk, float* __restrict__ w,
+                                               int64_t ldw, const ion::f32x2 (&Ef)[kPairs],
+                                               const ion::f32x2 (&rE)[kPairs],
+                                               const ion::f32x2 (&ex)[kPairs],
+                                               const ion::f32x2 (&lm)[kPairs],
+                                               const ion::f32x2 (&lg)[kPairs], int left) {
+  using namespace ion;
+  const f32x2 one_neg = pack2(-1.0f, -1.0f);
+  // s + e = a + b exactly (Knuth)
+  auto two_sum2 = [&](f32x2 a, f32x2 b, f32x2& s, f32x2& e) {
+    s = add2(a, b);
+    const f32x2 bb = fma2(a, one_neg, s);
+    const f32x2 r = fma2(bb, one_neg, s);
+    e = add2(fma2(r, one_neg, a), fma2(bb, one_neg, b));
+  };
+#pragma unroll 1
+  for (int k = 0; k < nk; ++k, w += ldw) {
+    const RateRow& h = rows[k];
+#pragma unroll
+    for (int j = 0; j < kPairs; ++j) {
+      const f32x2 qn = mul2(h.C_neg, rE[j]);                             // -C/E, leading part
+      const f32x2 ql = mul2(add2(fma2(qn, Ef[j], h.C), h.C_lo), rE[j]);  // C/E = -qn + ql
+      const f32x2 pn = mul2(h.b_neg, ex[j]);
+      const f32x2 pe = fma2(h.b, ex[j], pn);  // b ex = -pn + pe exactly
+      f32x2 s1, e1, s2, e2;
+      two_sum2(h.a, pn, s1, e1);
+      two_sum2(s1, qn, s2, e2);
+      const f32x2 lo = fma2(h.b, lm[j], mul2(h.b_lo, lg[j]));
+      const f32x2 small = fma2(lo, one_neg, fma2(ql, one_neg, fma2(pe, one_neg, h.a_lo)));
+      const f32x2 tail = add2(add2(e1, e2), small);
+      // n = the integer nearest y; s2 - n is exact, so is the rest up to 2^-25
+      const f32x2 magic = pack2(12582912.0f, 12582912.0f);
+      const f32x2 m = add2(add2(s2, tail), magic);
+      const f32x2 n = fma2(magic, one_neg, m);
+      const f32x2 fr = add2(fma2(n, one_neg, s2), tail);
+      float fv[2], mv[2], qv[2];
+      unpack2(fr, fv[0], fv[1]);
+      unpack2(m, mv[0], mv[1]);
+      unpack2(qn, qv[0], qv[1]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        // 2^n as two normal factors (n below -200: 0 after rounding)
+        const float mc = Tame ? mv[i] : fminf(mv[i], 12582912.0f + 100.0f);
+        const int ni = (int)(__float_as_uint(fmaxf(mc, 12582912.0f - 200.0f)) - 0x4b400000u);
+        const int n1 = ni >> 1;
+        // (|rest| <= 1/2 unless y is past 2^22 in size, where n alone makes r 0)
+        float r = ex2_approx(fminf(fv[i], 1.0f)) * __int_as_float((n1 << 23) + 0x3f800000) *
+                  __int_as_float(((ni - n1) << 23) + 0x3f800000);
+        if (!Tame) {
+          r = mv[i] > 12582912.0f + 98.0f ? fminf(r, 0x1p99f) : r;
+          r = -qv[i] <= (float)kCutoffLog2 ? r : 0.0f;
+        }
+        const int o = (2 * j + i) * kRateThreads;
+        if (Full || o < left) __stcs(w + o, r);
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kRateThreads, 4)
+    rates_f32_kernel(const ion::SpeciesTable* __restrict__ t, const float* __restrict__ E,
+                     int64_t ncells, int k_lo, int k_hi, float* __restrict__ W, int64_t ldw) {
+  __shared__ RateRow rows[ION_MAX_Z];
+  using namespace ion;
+  constexpr int kCells = 2 * kPairs * kRateThreads;
+  bool tame = true;
+  for (int k = k_lo + threadIdx.x; k < k_hi; k += kRateThreads) {
+    const double a = t->a2[k], b = t->b[k], C = t->C[k];
+    float ah, al, bh, bl, ch, cl;
+    split_f64(a, ah, al);
+    split_f64(b, bh, bl);
+    split_f64(C, ch, cl);
+    rows[k - k_lo] = {pack2(-bh, -bh), pack2(bh, bh), pack2(ch, ch), pack2(ah, ah),
+                      pack2(cl, cl),   pack2(bl, bl), pack2(al, al), pack2(-ch, -ch)};
+    tame = tame_state(a, b, C);
+  }
+  tame = __syncthreads_and(tame);
+  const int nk = k_hi - k_lo;
+  // the block's cells are a block's width apart in each thread
+  const int64_t c0 = blockIdx.x * (int64_t)kCells + threadIdx.x;
+  // those from this thread's first on
+  const int left = (int)min(ncells - c0, (int64_t)kCells);
+  f32x2 Ef[kPairs], rE[kPairs], ex[kPairs], lm[kPairs], lg[kPairs];
+  unsigned zeros = 0;  // cells of zero field: their rates are overwritten with 0
+#pragma unroll
+  for (int j = 0; j < kPairs; ++j) {
+    FieldF32 f[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int o = (2 * j + h) * kRateThreads;
+      f[h] = field_f32<true>(o < left ? E[c0 + o] : 1.0f);
+      zeros |= f[h].zero ? 1u << (2 * j + h) : 0u;
+    }
+    Ef[j] = pack2(f[0].E, f[1].E);
+    rE[j] = pack2(f[0].rE, f[1].rE);
+    ex[j] = pack2(f[0].ex, f[1].ex);
+    lm[j] = pack2(f[0].lm, f[1].lm);
+    lg[j] = pack2(f[0].lg, f[1].lg);
+  }
+  float* w = W + c0;
+  if (left > (2 * kPairs - 1) * kRateThreads && tame)
+    rates_f32_rows<true, true>(rows, nk, w, ldw, Ef, rE, ex, lm, lg, left);
+  else
+    rates_f32_rows<false, false>(rows, nk, w, ldw, Ef, rE, ex, lm, lg, left);
+#pragma unroll
+  for (int j = 0; j < 2 * kPairs; ++j)
+    if ((zeros >> j & 1u) && j * kRateThreads < left)
+      for (int k = 0; k < nk; ++k) w[j * kRateThreads + k * ldw] = 0.0f;
 }
 
 __global__ void rates_f64_kernel(const ion::SpeciesTable* t, const double* E,
@@ -267,10 +399,11 @@ int ion_rates(const ion_species* sp, const void* E, int64_t ncells, int k_lo,
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int threads = 256;
   const int blocks = (int)((ncells + threads - 1) / threads);
+  constexpr int kPerBlock = 2 * kPairs * kRateThreads;
   if (dtype == ION_DTYPE_F32)
-    rates_f32_kernel<<<blocks, threads, 0, s>>>(sp->dev, static_cast<const float*>(E),
-                                                (int)ncells, k_lo, k_hi,
-                                                static_cast<float*>(W_out), ldw);
+    rates_f32_kernel<<<(unsigned)((ncells + kPerBlock - 1) / kPerBlock), kRateThreads, 0, s>>>(
+        sp->dev, static_cast<const float*>(E), ncells, k_lo, k_hi, static_cast<float*>(W_out),
+        ldw);
   else
     rates_f64_kernel<<<blocks, threads, 0, s>>>(sp->dev, static_cast<const double*>(E),
                                                 (int)ncells, k_lo, k_hi,

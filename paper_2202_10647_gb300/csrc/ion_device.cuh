@@ -192,35 +192,15 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // where it says W dt < 2^-12 its error (below 2^-10 relative for terms up
 // to 10^3) moves W dt by less than 3e-7 and no population can see it, so
 // only larger rates take the float-float evaluation.
-template <bool Precise = false>
-__device__ __forceinline__ float rate_dt_f32(const StagedF32& t, int k,
-                                             const FieldF32& f) {
+__device__ __forceinline__ float rate_ff_f32(const StagedF32& t, int k, const FieldF32& f);
+
+__device__ __forceinline__ float rate_dt_f32(const StagedF32& t, int k, const FieldF32& f) {
   if (f.zero) return 0.0f;
   const float4 h = t.hi[k];  // a_hi, b_hi, C_hi, a_lo
   const float q = h.z * f.rE;
   if (q > (float)kCutoffLog2) return 0.0f;
-  if (!Precise) {
-    const float y0 = fmaf(-h.y, f.lg, h.x) - q;
-    if (y0 < -12.0f) return ex2_approx(y0);
-  }
-  const float2 l = t.lo[k];  // b_lo, C_lo
-  const float ql = (fmaf(-q, f.E, h.z) + l.y) * f.rE;  // C/E = q + ql
-  const float p = h.y * f.ex;
-  const float pe = fmaf(h.y, f.ex, -p);  // b_hi*ex = p + pe exactly
-  float s1, e1, s2, e2;
-  two_sum(h.x, -p, s1, e1);
-  two_sum(s1, -q, s2, e2);
-  const float small = ((h.w - pe) - ql) - fmaf(h.y, f.lm, l.x * f.lg);
-  const float tail = (e1 + e2) + small;
-  if (Precise) {
-    // 2^(s2 + tail) as 2^s2 2^tail keeps the relative error at a few ulp for
-    // any size of the exponent (rounding s2 + tail to one float would cost
-    // up to |y| 2^-24 relative).
-    return s2 > 99.0f ? exp2f(99.0f) : exp2f(s2) * exp2f(tail);
-  }
-  float y = s2 + tail;
-  y = fminf(y, 99.0f);  // W dt <= 2^99: keeps every later product finite
-  return ex2_approx(y);
+  const float y0 = fmaf(-h.y, f.lg, h.x) - q;
+  return y0 < -12.0f ? ex2_approx(y0) : rate_ff_f32(t, k, f);
 }
 
 // The float-float branch of rate_dt_f32 alone, for a rate its plain FP32
