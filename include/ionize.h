@@ -250,7 +250,8 @@ typedef struct {
 
 /* Launch shape of the FP32 streaming kernels: cells per lane (1, 2 or 4),
  * warps per block (2, 4 or 8), resident blocks per SM (0: as many as fit).
- * NULL selects {2, 8, 0}, which ion_step uses too. */
+ * NULL selects {2, 8, 0}, which ion_step uses too; without a shape a call of
+ * at most 400,000 cells runs one cell per lane in a single kernel instead. */
 typedef struct {
   int cells_per_lane;
   int warps_per_block;

@@ -607,7 +607,7 @@ int run_batch(const ion_batch_job* jobs, int njobs, double dt_fs, const ion_step
   if (rc) return rc;
   ion::LaunchShape sh = ion::default_shape();
   if (shape) {
-    sh = {shape->cells_per_lane, shape->warps_per_block, shape->blocks_per_sm};
+    sh = {shape->cells_per_lane, shape->warps_per_block, shape->blocks_per_sm, false};
     if (!ion::valid_shape(sh))
       return fail(ION_EINVAL,
                   "launch shape (%d cells/lane, %d warps/block, %d blocks/SM) is not built",

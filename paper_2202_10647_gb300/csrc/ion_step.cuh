@@ -122,6 +122,7 @@ struct LaunchShape {
   int cells_per_lane;   // 1, 2 or 4
   int warps_per_block;  // 2, 4 or 8
   int blocks_per_sm;    // 0: as many as fit
+  bool direct;          // small grids may take ion_direct_kernel (no shape was asked for)
 };
 
 // Workspace layout of the FP32 form (bound by bind_workspace, step_f32.cu):

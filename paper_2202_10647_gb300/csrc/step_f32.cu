@@ -1214,6 +1214,85 @@ __global__ void __launch_bounds__(128) ion_fb_kernel(const __grid_constant__ Bat
 }
 
 // ---------------------------------------------------------------------------
+// Small grids: one cell per lane from its rates to its stores, with the FP64
+// coefficients of a nearly degenerate cell taken in place: one launch, no
+// records and no queue.  On a grid of a few warps per SM the streaming kernel's
+// ring is mostly its own filling, and the two launches behind it find next to
+// nothing.  Steps of n nitrogen (Kr-like) cells in a graph, direct against
+// streaming, us: 16,384 6.4 against 25 (8.4, 29); 160,000 12 against 27 (19, 35);
+// 320,000 19 against 30 (31, 38); 500,000 25 against 31 (45, 42); 1,000,000 42 against
+// 31 (82, 52).  The line is where the heavier gas's crossing lies.
+// ---------------------------------------------------------------------------
+constexpr int kDirectThreads = 64;
+constexpr int kDirectCells = 400000;
+
+// One cell of at most W states; `stiff`: some rate has W dt > 1, `fb`: FP64
+// coefficients.  Returns |change of sum_k N_k| (ION_CONSERVATION_CHECK).
+template <int W>
+__device__ __forceinline__ float direct_cell(const JobIO& J, const Policy& pol,
+                                             const StagedF32& tab, int c, float Ec, int lo, int hi,
+                                             bool& stiff, bool& fb) {
+  const int w = hi - lo + 1;
+  const float* p = static_cast<const float*>(J.N) + (int64_t)lo * J.ld + c;
+  float v[W], lam[W], lmax = 0.0f;
+#pragma unroll
+  for (int r = 0; r < W; ++r) {
+    v[r] = r < w ? p[(int64_t)r * J.ld] : 0.0f;
+    lam[r] = 0.0f;
+  }
+  if (!pol.zero_dt) {
+    const FieldF32 f = field_f32(Ec);
+#pragma unroll
+    for (int r = 0; r < W - 1; ++r) {
+      if (r < w - 1) lam[r] = rate_dt_f32(tab, lo + r, f);
+      lmax = fmaxf(lmax, lam[r]);
+    }
+  }
+  stiff = lmax > DDParams<float>::prop_max;
+  float d = 0.0f;
+  fb = update_cell<float, W>(J, pol, c, lo, hi, v, lam, true,
+                             (pol.flags & ION_CONSERVATION_CHECK) ? &d : nullptr);
+  if (fb) d = fb_cell<W>(J, pol, tab, c, lo, hi);
+  return d;
+}
+
+__global__ void __launch_bounds__(kDirectThreads)
+    ion_direct_kernel(const __grid_constant__ BatchArgs a) {
+  __shared__ StagedF32 tabs[kMaxJobs];
+  // the jobs' cells one after another: job j's first is chunk0
+  const int i = blockIdx.x * kDirectThreads + threadIdx.x;
+  const int jid = job_of(a, i);
+  const JobIO& J = a.job[jid];
+  const int c = i - J.chunk0;
+  const bool on = c < J.ncells;
+  // the cell's inputs travel while the tables are staged
+  const float Ec = on ? static_cast<const float*>(J.E)[c] : 0.0f;
+  const int lo = on ? J.lo[c] : 0, hi = on ? J.hi[c] : 0;
+  for (int j = 0; j < a.njobs; ++j) stage_f32(a.job[j].tab, a.pol.log2dt, &tabs[j]);
+  __syncthreads();
+  const bool ok = on && window_ok(lo, hi, J.Z);
+  if (on && !ok) atomicAdd(&a.ws.hdr[kHdrInvalid], 1u);
+  const int w = ok ? hi - lo + 1 : 0;
+  const int Wm = __reduce_max_sync(kFull, w);
+  bool stiff = false, fb = false;
+  float d = 0.0f;
+  if (w >= 1) {
+    if (Wm <= 2)
+      d = direct_cell<2>(J, a.pol, tabs[jid], c, Ec, lo, hi, stiff, fb);
+    else if (Wm <= 4)
+      d = direct_cell<4>(J, a.pol, tabs[jid], c, Ec, lo, hi, stiff, fb);
+    else
+      d = direct_cell<6>(J, a.pol, tabs[jid], c, Ec, lo, hi, stiff, fb);
+  }
+  const unsigned ms = __ballot_sync(kFull, stiff), mf = __ballot_sync(kFull, fb);
+  if ((threadIdx.x & 31) == 0) {
+    if (ms) atomicAdd(&a.ws.hdr[kHdrStiff], (unsigned)__popc(ms));
+    if (mf) atomicAdd(&a.ws.hdr[kHdrFallback], (unsigned)__popc(mf));
+  }
+  if (a.pol.flags & ION_CONSERVATION_CHECK) warp_max_into(&a.ws.hdr[kHdrCons], abs_bits(d));
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 // One instantiation of the streaming kernel: its function and smem needs.
@@ -1321,7 +1400,7 @@ cudaError_t resident_blocks(const StreamVariant& v, int njobs, size_t smem, int*
 
 }  // namespace
 
-LaunchShape default_shape() { return {2, 8, 0}; }
+LaunchShape default_shape() { return {2, 8, 0, true}; }
 
 bool valid_shape(const LaunchShape& s) {
   return find_variant(s.cells_per_lane, s.warps_per_block) != nullptr &&
@@ -1365,12 +1444,22 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
   const int chunk = 32 * v->Q;
   int total = 0, cells = 0;
   for (int j = 0; j < a.njobs; ++j) {
+    a.job[j].chunk0 = cells;
+    cells += a.job[j].ncells;
+  }
+  if (cells == 0) return cudaSuccess;
+  if (shape.direct && cells <= kDirectCells) {
+    a.nchunks = cells;
+    ion_direct_kernel<<<(cells + kDirectThreads - 1) / kDirectThreads, kDirectThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
+  cells = 0;
+  for (int j = 0; j < a.njobs; ++j) {
     a.job[j].chunk0 = total;
     total += a.job[j].ncells / chunk;
     cells += a.job[j].ncells;
   }
   a.nchunks = total;
-  if (cells == 0) return cudaSuccess;
   const size_t smem = v->smem(a.njobs);
   int fit = 0;
   if ((e = resident_blocks(*v, a.njobs, smem, &fit)) != cudaSuccess) return e;
