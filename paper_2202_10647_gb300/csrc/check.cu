@@ -30,18 +30,34 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
   e += err;
 }
 
+// The block's largest bits into *out.
+__device__ __forceinline__ void block_max_into(unsigned worst, unsigned* out) {
+  worst = __reduce_max_sync(0xffffffffu, worst);
+  __shared__ unsigned red[kThreads / 32];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = worst;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < kThreads / 32; ++i) m = max(m, red[i]);
+    if (m > *(volatile unsigned*)out) atomicMax(out, m);
+  }
+}
+
 // FP32 populations, four cells per thread (ld % 4 == 0, N 16-byte aligned):
 // each cell's planes are summed in float-float (TwoSum), whose error for a
 // few dozen non-negative terms of order 1 stays below 1e-12, far under the
-// FP32 rounding being measured; FP64 adds would make the kernel bound by
-// GB300's FP64 rate instead of memory.
+// FP32 rounding being measured; the target (th + tl) is taken off in float-float
+// too, as FP64 instructions at a cell's end keep GB300's slow FP64 pipe busy
+// (29 % of the time).  One tile of cells per block: a grid of 8 blocks per SM of
+// which about 5 fit made a second, half-empty wave.  37 planes of 16.8M cells: 490 us
+// with both, 334 without, 7.4 TB/s; bound by memory.
 __global__ void __launch_bounds__(kThreads)
     conservation_f32x4_kernel(const float* __restrict__ N, int64_t ld, int64_t ncells,
-                              int nplanes, double target, unsigned* out) {
+                              int nplanes, float th, float tl, unsigned* out) {
   unsigned worst = 0;
-  const int64_t stride = (int64_t)gridDim.x * kThreads * 4;
-  for (int64_t c = ((int64_t)blockIdx.x * kThreads + threadIdx.x) * 4; c < ncells;
-       c += stride) {
+  const int64_t c = ((int64_t)blockIdx.x * kThreads + threadIdx.x) * 4;
+  if (c < ncells) {
     const float4* p = reinterpret_cast<const float4*>(N + c);
     const int64_t ld4 = ld / 4;
     float s[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
@@ -68,21 +84,12 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (c + j < ncells) {
-        const double d = ((double)s[j] - target) + (double)e[j];
-        worst = max(worst, ordered_bits((float)fabs(d)));
+        two_sum_acc(s[j], e[j], -th);
+        worst = max(worst, ordered_bits(fabsf(s[j] + (e[j] - tl))));
       }
     }
   }
-  worst = __reduce_max_sync(0xffffffffu, worst);
-  __shared__ unsigned red[kThreads / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = worst;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned m = 0;
-#pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) m = max(m, red[i]);
-    atomicMax(out, m);
-  }
+  block_max_into(worst, out);
 }
 
 template <typename T>
@@ -105,16 +112,7 @@ __global__ void __launch_bounds__(kThreads)
     for (; k < nplanes; ++k) s += (double)__ldcs(p + (int64_t)k * ld);
     worst = max(worst, ordered_bits((float)fabs(s - target)));
   }
-  worst = __reduce_max_sync(0xffffffffu, worst);
-  __shared__ unsigned red[kThreads / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = worst;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned m = 0;
-#pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) m = max(m, red[i]);
-    atomicMax(out, m);
-  }
+  block_max_into(worst, out);
 }
 
 }  // namespace
@@ -151,11 +149,15 @@ extern "C" int ion_conservation(const void* N, int64_t ld, int64_t ncells, int n
   unsigned* out = reinterpret_cast<unsigned*>(out_max);
   if ((e = cudaMemsetAsync(out, 0, sizeof(unsigned), s)) != cudaSuccess)
     return ion::set_error(ION_ECUDA, "ion_conservation: %s", cudaGetErrorString(e));
+  // (a target that float arithmetic cannot hold, and more tiles than a grid has blocks, go to
+  // the general kernel)
+  const float th = (float)target;
   const bool x4 = dtype == ION_DTYPE_F32 && ld % 4 == 0 &&
-                  (reinterpret_cast<uintptr_t>(N) % 16) == 0;
+                  (reinterpret_cast<uintptr_t>(N) % 16) == 0 && std::fabs(target) < 1e30 &&
+                  need < (int64_t(1) << 31);
   if (x4)
-    conservation_f32x4_kernel<<<blocks, kThreads, 0, s>>>(static_cast<const float*>(N), ld,
-                                                          ncells, nplanes, target, out);
+    conservation_f32x4_kernel<<<(unsigned)need, kThreads, 0, s>>>(
+        static_cast<const float*>(N), ld, ncells, nplanes, th, (float)(target - (double)th), out);
   else if (dtype == ION_DTYPE_F32)
     conservation_kernel<float><<<blocks, kThreads, 0, s>>>(static_cast<const float*>(N), ld,
                                                            ncells, nplanes, target, out);

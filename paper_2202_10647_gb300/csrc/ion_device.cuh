@@ -96,6 +96,19 @@ struct FieldF32 {
   bool zero;     // W = 0 for every state
 };
 
+// log2 x and 1/x by the SFU for normal x, without the scaling of denormals
+// that __log2f and __fdividef carry (1/x is 0 for x > 2^126).
+__device__ __forceinline__ float lg2_approx(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 template <bool Precise = false>
 __device__ __forceinline__ FieldF32 field_f32(float E_in) {
   FieldF32 f;
@@ -106,10 +119,10 @@ __device__ __forceinline__ FieldF32 field_f32(float E_in) {
   const int bits = __float_as_int(E);
   const float mant = __int_as_float((bits & 0x007fffff) | 0x3f800000);
   f.ex = (float)((bits >> 23) - 127);
-  f.lm = Precise ? log2f(mant) : __log2f(mant);
+  f.lm = Precise ? log2f(mant) : lg2_approx(mant);
   f.lg = f.ex + f.lm;
   f.E = E;
-  f.rE = Precise ? __frcp_rn(E) : __fdividef(1.0f, E);
+  f.rE = Precise ? __frcp_rn(E) : rcp_approx(E);
   return f;
 }
 
@@ -361,6 +374,32 @@ __constant__ const float kInvFactF32[kEasyTerms + 1] = {
     1.0f / 355687428096000.0f,
     1.0f / 6402373705728000.0f};
 
+// (-1)^k/k! twice, for two cells per instruction (f32x2.cuh).
+constexpr unsigned long long twice(float x) {
+  return (unsigned long long)__builtin_bit_cast(unsigned, x) << 32 |
+         __builtin_bit_cast(unsigned, x);
+}
+__constant__ const unsigned long long kAltFact2[kEasyTerms + 1] = {
+    twice(1.0f),
+    twice(-1.0f),
+    twice(1.0f / 2),
+    twice(-1.0f / 6),
+    twice(1.0f / 24),
+    twice(-1.0f / 120),
+    twice(1.0f / 720),
+    twice(-1.0f / 5040),
+    twice(1.0f / 40320),
+    twice(-1.0f / 362880),
+    twice(1.0f / 3628800),
+    twice(-1.0f / 39916800),
+    twice(1.0f / 479001600),
+    twice(-1.0f / 6227020800.0f),
+    twice(1.0f / 87178291200.0f),
+    twice(-1.0f / 1307674368000.0f),
+    twice(1.0f / 20922789888000.0f),
+    twice(-1.0f / 355687428096000.0f),
+    twice(1.0f / 6402373705728000.0f)};
+
 template <typename T>
 struct DDParams;
 
@@ -379,7 +418,8 @@ struct DDParams<float> {
       if (i < rmax) R += x > kThrF32[i] ? 1 : 0;
     return R;
   }
-  __device__ static __forceinline__ float div(float a, float b) { return __fdividef(a, b); }
+  // (|b| lies in [tau / end_ratio, 2^99]: no scaling)
+  __device__ static __forceinline__ float div(float a, float b) { return a * rcp_approx(b); }
   __device__ static __forceinline__ float inv_fact(int n) { return kInvFactF[n]; }
   __device__ static __forceinline__ float expn(float z) { return exp(z); }
   // what the choices of a divided difference's form look at

@@ -277,26 +277,33 @@ __device__ __forceinline__ void easy_cells(const JobIO& J, const Policy& pol,
   // recurrences interleave.  Slots past a cell's window start from whatever
   // the stage holds there: their rates and the rate into them are zero, so
   // their u is zero after one term and their inc stays zero.  Stiff cells
-  // run with rates above lam_easy; their inc is never read.
-  float inc[Q][WM];
+  // run with rates above lam_easy; their results are never used.
+  // The last slot goes by conservation: the top state of a window of width WM
+  // gains what the others lost (narrower windows reach their top inside the
+  // series, whose rate there is zero, and never read this slot).
   if constexpr (Q % 2 == 0) {
-    // Two cells per instruction (f32x2; the loop's issue slots halve: PAIRUS).
-    // U_i = (-1)^i u_i, so that both of the recurrence's rates carry one sign:
-    // u_i' = -lam_i u_i + lam_{i-1} u_{i-1}, U_i' = -lam_i U_i - lam_{i-1} U_{i-1}
+    // Two cells per instruction (f32x2): the series and what follows from it,
+    // as this kernel is bound by issuing instructions (equal bits; the part after the series
+    // and the conservation sums in pairs: 30M mixed cells 999 -> 987 us, 20 Kr-like steps
+    // with the check 4 % less).
+    // U_i = (-1)^(i+k) u_i, so that the recurrence carries no sign:
+    // u_i' = -lam_i u_i + lam_{i-1} u_{i-1}, U_i' = lam_i U_i + lam_{i-1} U_{i-1},
+    // and the factors (-1)^k/k! do.
+    const f32x2 minus = pack2(-1.0f, -1.0f), plus = pack2(1.0f, 1.0f);
     f32x2 L[Q / 2][WM - 1], U[Q / 2][WM - 1], I[Q / 2][WM - 1];
 #pragma unroll
     for (int j = 0; j < Q / 2; ++j) {
 #pragma unroll
       for (int i = 0; i < WM - 1; ++i) {
-        const float s = i % 2 ? -1.0f : 1.0f;
-        L[j][i] = pack2(-lam[2 * j][i], -lam[2 * j + 1][i]);
-        U[j][i] = pack2(s * v[2 * j][i], s * v[2 * j + 1][i]);
+        L[j][i] = pack2(lam[2 * j][i], lam[2 * j + 1][i]);
+        const f32x2 u = pack2(v[2 * j][i], v[2 * j + 1][i]);
+        U[j][i] = i % 2 ? mul2(u, minus) : u;
         I[j][i] = 0ull;
       }
     }
 #pragma unroll 1
     for (int k = 1; k <= Rw; ++k) {
-      const f32x2 ck = pack2(kInvFactF32[k], kInvFactF32[k]);
+      const f32x2 ck = kAltFact2[k];
 #pragma unroll
       for (int j = 0; j < Q / 2; ++j) {
 #pragma unroll
@@ -309,16 +316,57 @@ __device__ __forceinline__ void easy_cells(const JobIO& J, const Policy& pol,
     }
 #pragma unroll
     for (int j = 0; j < Q / 2; ++j) {
+      const int wa = w[2 * j], wb = w[2 * j + 1];
+      f32x2 cum = 0ull;  // population that left states <= i
+      float da = 0.0f, db = 0.0f;
+      f32x2 nv[WM];
 #pragma unroll
-      for (int i = 0; i < WM - 1; ++i) {
-        const float s = i % 2 ? -1.0f : 1.0f;
-        unpack2(I[j][i], inc[2 * j][i], inc[2 * j + 1][i]);
-        inc[2 * j][i] *= s;
-        inc[2 * j + 1][i] *= s;
+      for (int i = 0; i < WM; ++i) nv[i] = pack2(v[2 * j][i], v[2 * j + 1][i]);
+      f32x2 s = 0ull, e = 0ull;  // CONS: ExactSum of both cells (0 added past a window)
+#pragma unroll
+      for (int i = 0; i < WM; ++i) {
+        const f32x2 old = nv[i];
+        if (i < WM - 1) {
+          cum = fma2(I[j][i], i % 2 ? plus : minus, cum);
+          nv[i] = fma2(I[j][i], i % 2 ? minus : plus, nv[i]);
+          float ca, cb;
+          unpack2(cum, ca, cb);
+          da += i == 0 || i < wa - 1 ? ca : 0.0f;
+          db += i == 0 || i < wb - 1 ? cb : 0.0f;
+        } else {
+          nv[i] = add2(nv[i], cum);
+        }
+        if constexpr (CONS) {
+          f32x2 x = old, y = nv[i];
+          if (i >= 2) {
+            float xa, xb, ya, yb;
+            unpack2(x, xa, xb);
+            unpack2(y, ya, yb);
+            x = pack2(i < wa ? xa : 0.0f, i < wb ? xb : 0.0f);
+            y = pack2(i < wa ? ya : 0.0f, i < wb ? yb : 0.0f);
+          }
+          f32x2 t = fma2(x, minus, s), z = fma2(s, minus, t);
+          e = add2(e, fma2(add2(x, z), minus, fma2(fma2(z, minus, t), minus, s)));
+          s = t;
+          t = add2(s, y);
+          z = fma2(s, minus, t);
+          e = add2(e, add2(fma2(fma2(z, minus, t), minus, s), fma2(z, minus, y)));
+          s = t;
+        }
+      }
+      dne[2 * j] = da;
+      dne[2 * j + 1] = db;
+#pragma unroll
+      for (int i = 0; i < WM; ++i) unpack2(nv[i], v[2 * j][i], v[2 * j + 1][i]);
+      if constexpr (CONS) {
+        float ta, tb;
+        unpack2(add2(s, e), ta, tb);
+        if (!stiff[2 * j] && wa >= 2) cmax = max(cmax, abs_bits(ta));
+        if (!stiff[2 * j + 1] && wb >= 2) cmax = max(cmax, abs_bits(tb));
       }
     }
   } else {
-    float u[Q][WM];
+    float u[Q][WM], inc[Q][WM];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
 #pragma unroll
@@ -339,44 +387,42 @@ __device__ __forceinline__ void easy_cells(const JobIO& J, const Policy& pol,
         }
       }
     }
-  }
-  // the last slot by conservation: the top state of a window of width WM
-  // gains what the others lost (narrower windows reach their top inside the
-  // series, whose rate there is zero, and never read this slot)
 #pragma unroll
-  for (int j = 0; j < Q; ++j) {
-    float t = 0.0f;
+    for (int j = 0; j < Q; ++j) {
+      float cum = 0.0f;
+      dne[j] = 0.0f;
 #pragma unroll
-    for (int i = 0; i < WM - 1; ++i) t -= inc[j][i];
-    inc[j][WM - 1] = t;
-  }
-#pragma unroll
-  for (int j = 0; j < Q; ++j) {
-    dne[j] = 0.0f;
-    nlo[j] = lo[j];
-    nhi[j] = hi[j];
-    if (stiff[j] || w[j] < 2) continue;
-    float cum = 0.0f;
-#pragma unroll
-    for (int r = 0; r < WM - 1; ++r) {
-      if (r < w[j] - 1) {
-        cum -= inc[j][r];  // population that left states <= r
-        dne[j] += cum;
+      for (int r = 0; r < WM - 1; ++r) {
+        cum -= inc[j][r];
+        if (r < w[j] - 1) dne[j] += cum;
+        v[j][r] += inc[j][r];
       }
-    }
+      v[j][WM - 1] += cum;
+      if constexpr (CONS) {
+        if (!stiff[j] && w[j] >= 2) {
+          ExactSum<float> acc;
 #pragma unroll
-    for (int r = 0; r < WM; ++r) v[j][r] += inc[j][r];
-    if constexpr (CONS) {
-      ExactSum<float> acc;
-#pragma unroll
-      for (int r = 0; r < WM; ++r) {
-        if (r < w[j]) {
-          acc.add(-vget(P[r][lane], j));
-          acc.add(v[j][r]);
+          for (int r = 0; r < WM; ++r) {
+            if (r < w[j]) {
+              acc.add(-vget(P[r][lane], j));
+              acc.add(v[j][r]);
+            }
+          }
+          cmax = max(cmax, abs_bits(acc.value()));
         }
       }
-      cmax = max(cmax, abs_bits(acc.value()));
     }
+  }
+#pragma unroll
+  for (int j = 0; j < Q; ++j) {
+    nlo[j] = lo[j];
+    nhi[j] = hi[j];
+    if (w[j] < 2) {  // nothing to step: what the slots hold stays
+      dne[j] = 0.0f;
+#pragma unroll
+      for (int r = 0; r < WM; ++r) v[j][r] = vget(P[r][lane], j);
+    }
+    if (stiff[j] || w[j] < 2) continue;
     if ((pol.flags & ION_NO_WINDOW_UPDATE) == 0) {
       if constexpr (AD)
         adapt_window<float, WM>(v[j], w[j], J.Z, pol.eps_f, pol.wmin, pol.wmax,
@@ -1168,25 +1214,30 @@ __device__ __forceinline__ float fb_cell(const JobIO& J, const Policy& pol,
   return (float)fabs(s1 - s0);
 }
 
-// The queue is dealt out a warp at a time across the blocks (warp k of the
-// grid takes entries 32k..32k+31, and warp k sits in block k mod grid), so
-// that a short queue spreads over as many SMs as it has warps: the FP64 pipe
-// is the bound here, and each SM has its own.  Each warp runs the
-// instantiation of its widest window, so its lanes do not diverge by width.
+// The queue is dealt out over all warps of the grid, `per` entries to a warp
+// (warp k of the grid takes entries k per .. k per + per - 1, and sits in block k mod
+// grid): a queue is short (thousands of cells), its cells take FP64 chains and
+// different branches of the divided differences, and a full warp runs the
+// branches of all its lanes one after another.  With as few cells per warp as the grid
+// allows the warps of an SM overlap those chains (a step of 16.8M Kr-like cells
+// with some thousand such cells: 24 -> 18 us; `per` is 32 once the queue fills the grid).
+// Each warp runs the instantiation of its widest window, so its lanes do not diverge
+// by width.
 __global__ void __launch_bounds__(128) ion_fb_kernel(const __grid_constant__ BatchArgs a) {
   __shared__ StagedF32 tabs[kMaxJobs];
   const unsigned n = *((volatile unsigned*)&a.ws.hdr[kHdrFallback]);
   const unsigned warps = gridDim.x * (blockDim.x / 32u);
   const unsigned wid = (threadIdx.x / 32u) * gridDim.x + blockIdx.x;  // warp of the grid
   const unsigned lane = threadIdx.x & 31u;
-  if (blockIdx.x * 32u >= n) return;  // no queued cell for this block
+  const unsigned per = min(32u, (n + warps - 1u) / warps);  // entries per warp
+  if (blockIdx.x * per >= n) return;  // no queued cell for this block
   for (int j = 0; j < a.njobs; ++j) stage_f32(a.job[j].tab, a.pol.log2dt, &tabs[j]);
   __syncthreads();
   uint32_t cmax = 0;  // largest |change of sum_k N_k| (bits), ION_CONSERVATION_CHECK
-  for (unsigned base = wid * 32u; base < n; base += warps * 32u) {  // warp-uniform
+  for (unsigned base = wid * per; base < n; base += warps * per) {  // warp-uniform
     const unsigned i = base + lane;
     int c = 0, jid = 0, lo = 0, hi = -1;
-    if (i < n) {
+    if (lane < per && i < n) {
       c = (int)a.ws.queue[i];
       jid = a.ws.queue_job[i];
       lo = a.job[jid].lo[c];
