@@ -7,12 +7,16 @@
 // "... of the logarithm function ...", ACM TOMS 16, 1990): a table entry picked
 // by the leading bits, and a short polynomial in what is left.  Exponents,
 // table indices, comparisons and conversions are integer and FP32 work.
-//   log2_rcp_f64   9 FP64 instructions for log2 E and 3 for 1/E
-//   exp2_f64       8
-// against some 25, 10 and 15 of log2(), a division and exp2().  Errors (measured over
-// 2^-20..2^60 and -1000..1000, against 113-bit arithmetic): log2 0.69 ulp of
-// max(|log2 E|, 1), 1/E 0.50 ulp, exp2 1.03 ulp.
-// The tables are nearest doubles of 40-digit values; the polynomials
+//   log2_f64   1 FP64 instruction
+//   rcp_f64, exp2_f64   none
+// against some 25, 10 and 15 of log2(), a division and exp2(), and 9, 3 and 8 of the same
+// method with the polynomials in FP64: everything else is 64-bit fixed point, 20 to 60
+// integer instructions each, whose issue time is that of one FP64 instruction at most.  A
+// rate of Eq. 1 keeps the two fused multiply-adds of its exponent.  FP64 step, 33.5M nitrogen
+// cells: 2,347 us with the polynomials in FP64, 1,922 so.
+// Errors (measured over 2^-20..2^60 and -1000..1000, against 113-bit arithmetic): log2
+// 0.57 ulp of max(|log2 E|, 1), 1/E 0.56 ulp, exp2 0.96 ulp.
+// The tables are nearest values of 40-digit ones; the polynomials
 // interpolate at Chebyshev nodes.
 #pragma once
 
@@ -20,160 +24,132 @@
 
 namespace ion {
 
-// log2(1 + r) / r for |r| <= 1/257, lowest degree first (error of the product below 2^-55)
-constexpr double kLog1 = 0x1.71547652b82fep+0, kLog2 = -0x1.71547652924f5p-1,
-                 kLog3 = 0x1.ec709dc35f513p-2, kLog4 = -0x1.7155a7b607d21p-2,
-                 kLog5 = 0x1.2777cad1d781ep-2;
-// (2^r - 1) / r for |r| <= 1/512
-constexpr double kExp1 = 0x1.62e42fefa39d9p-1, kExp2 = 0x1.ebfbdff82c585p-3,
-                 kExp3 = 0x1.c6b0902b5a621p-5, kExp4 = 0x1.3b2ab83eae236p-7;
+// log2(1 + rho/64) 64/rho for rho in [0, 1/2] in units of 2^-51, lowest degree first, every
+// other sign a minus (error of the product below 2^-60)
+constexpr uint64_t kLog1 = 0xb8aa3b295c17full, kLog2 = 0x171547652b7cull,
+                   kLog3 = 0x3d8e13b7caull;
+constexpr uint32_t kLog4 = 0xb8aa3580u, kLog5 = 0x24ed7a7u, kLog6 = 0x78ab1u;
+// 256 (2^(rho/256) - 1) / rho for rho in [0, 1] in units of 2^-52, lowest degree first (error
+// 2^-56.6 of 1)
+constexpr uint64_t kExp1 = 0xb17217f7d1cedull, kExp2 = 0x3d7f7bff1b7ull;
+constexpr uint32_t kExp3 = 0xe3583fe3u, kExp4 = 0x277045u;
 
-// Interval j of the mantissa, [1 + j/128, 1 + (j+1)/128): c = 1/(its middle),
-// and -log2 c = hi + lo, hi a multiple of 2^-12 (so that exponent + hi is
-// exact in FP32).
+// Interval j of the mantissa, [1 + j/128, 1 + (j+1)/128): c, the reciprocal of its lower end
+// rounded up, in units of 2^-31, and -log2 c in units of 2^-57.
 struct LogRow {
-  double c, lo;
+  unsigned long long log;
+  uint32_t c;
 };
 static __device__ const LogRow kLogTab[128] = {
-    {0x1.fe01fe01fe020p-1, 0x1.388daf558c06bp-17}, {0x1.fa11caa01fa12p-1, -0x1.39dd0ad09fae3p-15},
-    {0x1.f6310aca0dbb5p-1, 0x1.363ba850f9bdcp-14}, {0x1.f25f644230ab5p-1, 0x1.a6128d0b44e98p-14},
-    {0x1.ee9c7f8458e02p-1, 0x1.6ff0d25464b05p-15}, {0x1.eae807aba01ebp-1, -0x1.8ecf99b58c53fp-14},
-    {0x1.e741aa59750e4p-1, -0x1.29207b296fa60p-14}, {0x1.e3a9179dc1a73p-1, 0x1.ee0d80ceee769p-14},
-    {0x1.e01e01e01e01ep-1, -0x1.1169475d7eacbp-16}, {0x1.dca01dca01dcap-1, 0x1.11df348494026p-16},
-    {0x1.d92f2231e7f8ap-1, -0x1.cb1ca47d29656p-16}, {0x1.d5cac807572b2p-1, 0x1.9a83c2c02929ep-14},
-    {0x1.d272ca3fc5b1ap-1, -0x1.8f25bb7ce7abfp-14}, {0x1.cf26e5c44bfc6p-1, -0x1.eb5a7c2cdfe2bp-14},
-    {0x1.cbe6d9601cbe7p-1, 0x1.146d9a8a62f7ep-15}, {0x1.c8b265afb8a42p-1, 0x1.d5c83d2e452a2p-14},
-    {0x1.c5894d10d4986p-1, 0x1.fb7d64898a747p-14}, {0x1.c26b5392ea01cp-1, 0x1.fec7d05ddfef7p-15},
-    {0x1.bf583ee868d8bp-1, -0x1.1a8be56a4a677p-14}, {0x1.bc4fd65883e7bp-1, -0x1.39b9be8f27664p-16},
-    {0x1.b951e2b18ff23p-1, -0x1.30e8a06a144d4p-15}, {0x1.b65e2e3beee05p-1, -0x1.f4e1c4791b3e5p-14},
-    {0x1.b37484ad806cep-1, -0x1.80389d6fe4abcp-16}, {0x1.b094b31d922a4p-1, 0x1.4ce4823c9a978p-17},
-    {0x1.adbe87f94905ep-1, -0x1.5176cbe670fc9p-16}, {0x1.aaf1d2f87ebfdp-1, -0x1.d68aabd572843p-14},
-    {0x1.a82e65130e159p-1, -0x1.662513dc07841p-16}, {0x1.a574107688a4ap-1, 0x1.2fb6c4709bb77p-17},
-    {0x1.a2c2a87c51ca0p-1, -0x1.53293365ee1ffp-16}, {0x1.a01a01a01a01ap-1, -0x1.c69c94d7ca5f5p-14},
-    {0x1.9d79f176b682dp-1, -0x1.62faf11824ed0p-17}, {0x1.9ae24ea5510dap-1, 0x1.f3fb753f12621p-16},
-    {0x1.9852f0d8ec0ffp-1, 0x1.c40747db55ba5p-17}, {0x1.95cbb0be377aep-1, -0x1.edc9990e6dba5p-15},
-    {0x1.934c67f9b2ce6p-1, 0x1.e36852915b397p-15}, {0x1.90d4f120190d5p-1, 0x1.f5248cd4b831fp-14},
-    {0x1.8e6527af1373fp-1, -0x1.e9c8343e7d51dp-14}, {0x1.8bfce8062ff3ap-1, 0x1.57ac51aac45d3p-14},
-    {0x1.899c0f601899cp-1, -0x1.0f309e79c7fa3p-16}, {0x1.87427bcc092b9p-1, 0x1.4673b5c37168ep-14},
-    {0x1.84f00c2780614p-1, 0x1.f90527409a9a9p-14}, {0x1.82a4a0182a4a0p-1, 0x1.d6759b25dfe53p-14},
-    {0x1.8060180601806p-1, 0x1.c28def7de8b09p-15}, {0x1.7e225515a4f1dp-1, -0x1.c8203f37965dcp-15},
-    {0x1.7beb3922e017cp-1, 0x1.11b7f10cf28cdp-15}, {0x1.79baa6bb6398bp-1, 0x1.2a6c24cae773dp-14},
-    {0x1.77908119ac60dp-1, 0x1.02f6ca47b4a06p-14}, {0x1.756cac201756dp-1, 0x1.4c80bf27c0644p-18},
-    {0x1.734f0c541fe8dp-1, -0x1.9dddf9b048396p-14}, {0x1.713786d9c7c09p-1, -0x1.2c2f68d6954f5p-18},
-    {0x1.6f26016f26017p-1, 0x1.708fa2b79c3a2p-15}, {0x1.6d1a62681c861p-1, 0x1.8acf798a81799p-15},
-    {0x1.6b1490aa31a3dp-1, 0x1.6b902680a153cp-18}, {0x1.691473a88d0c0p-1, -0x1.51b11b3640d44p-14},
-    {0x1.6719f3601671ap-1, 0x1.1c67c93ac8928p-15}, {0x1.6524f853b4aa3p-1, 0x1.b869f1c3f86f9p-14},
-    {0x1.63356b88ac0dep-1, -0x1.d1156507ddd2ep-14}, {0x1.614b36831ae94p-1, 0x1.f3a73c300cf4dp-14},
-    {0x1.5f66434292dfcp-1, 0x1.08892bc00b902p-14}, {0x1.5d867c3ece2a5p-1, -0x1.211c336f787e2p-15},
-    {0x1.5babcc647fa91p-1, 0x1.2a3b39774d885p-14}, {0x1.59d61f123ccaap-1, -0x1.c5489254cab0cp-14},
-    {0x1.5805601580560p-1, -0x1.5d4e9185f6f6ap-14}, {0x1.56397ba7c52e2p-1, -0x1.9c130dd53fb2bp-14},
-    {0x1.54725e6bb82fep-1, 0x1.8026a02700cf1p-14}, {0x1.52aff56a8054bp-1, -0x1.baf2648728ff6p-20},
-    {0x1.50f22e111c4c5p-1, 0x1.d064ae0fb3b2bp-14}, {0x1.4f38f62dd4c9bp-1, -0x1.f07f428bdfa24p-15},
-    {0x1.4d843bedc2c4cp-1, -0x1.7cdb7a8f76aacp-16}, {0x1.4bd3edda68fe1p-1, -0x1.8b96385a2290ep-16},
-    {0x1.4a27fad76014ap-1, -0x1.01b66fbd35f1bp-14}, {0x1.4880522014880p-1, 0x1.c5e5a04b0f37ep-14},
-    {0x1.46dce34596066p-1, -0x1.5106da1a8bfeap-19}, {0x1.453d9e2c776cap-1, 0x1.8e8353e67cf46p-14},
-    {0x1.43a2730abee4dp-1, -0x1.6d7a370decda8p-14}, {0x1.420b5265e5951p-1, -0x1.fa11e53f4ccabp-15},
-    {0x1.40782d10e6566p-1, -0x1.1eb680e5478bap-14}, {0x1.3ee8f42a5af07p-1, -0x1.d115ef7d881c8p-14},
-    {0x1.3d5d991aa75c6p-1, 0x1.da80c6c41fec7p-15}, {0x1.3bd60d9232955p-1, -0x1.c4a2399046319p-15},
-    {0x1.3a524387ac822p-1, 0x1.8325bdbe206dfp-15}, {0x1.38d22d366088ep-1, 0x1.da44a19b5ae54p-14},
-    {0x1.3755bd1c945eep-1, -0x1.96e87473d1d94p-14}, {0x1.35dce5f9f2af8p-1, -0x1.90a5d6749fc73p-14},
-    {0x1.34679ace01346p-1, 0x1.ee564c7bdde2ap-14}, {0x1.32f5ced6a1dfap-1, 0x1.cea240187f1ecp-15},
-    {0x1.3187758e9ebb6p-1, -0x1.48e97e1d6ef37p-15}, {0x1.301c82ac40260p-1, 0x1.4c40d29bf2a72p-14},
-    {0x1.2eb4ea1fed14bp-1, -0x1.45566b911825ap-14}, {0x1.2d50a012d50a0p-1, -0x1.601c2624789b9p-16},
-    {0x1.2bef98e5a3711p-1, 0x1.55e2da951b46cp-18}, {0x1.2a91c92f3c105p-1, 0x1.0111eb309295ep-20},
-    {0x1.293725bb804a5p-1, -0x1.15db83a3de8d4p-15}, {0x1.27dfa38a1ce4dp-1, -0x1.9654f63a37048p-14},
-    {0x1.268b37cd60127p-1, 0x1.c5db68e0b581cp-15}, {0x1.2539d7e9177b2p-1, -0x1.1e0a946366676p-14},
-    {0x1.23eb79717605bp-1, 0x1.9f66474ab71c2p-16}, {0x1.22a0122a0122ap-1, 0x1.75adcff6ed5b9p-14},
-    {0x1.21579804855e6p-1, -0x1.f37dd9d537ae7p-14}, {0x1.2012012012012p-1, -0x1.d29d03b17694dp-14},
-    {0x1.1ecf43c7fb84cp-1, 0x1.d95932267742ep-14}, {0x1.1d8f5672e4abdp-1, 0x1.116a2f25a8d38p-14},
-    {0x1.1c522fc1ce059p-1, -0x1.4b4070f761cb5p-17}, {0x1.1b17c67f2bae3p-1, -0x1.d61ee0d335c9dp-14},
-    {0x1.19e0119e0119ep-1, 0x1.88221cc248074p-19}, {0x1.18ab083902bdbp-1, 0x1.7eafe46c09af7p-14},
-    {0x1.1778a191bd684p-1, -0x1.7ddd7736b2075p-14}, {0x1.1648d50fc3201p-1, -0x1.d0ea66df5c657p-15},
-    {0x1.151b9a3fdd5c9p-1, -0x1.80512926a2eb2p-15}, {0x1.13f0e8d344724p-1, -0x1.040be494e45b9p-14},
-    {0x1.12c8b89edc0acp-1, -0x1.b336660616083p-14}, {0x1.11a3019a74826p-1, 0x1.333db8a408927p-14},
-    {0x1.107fbbe011080p-1, -0x1.3f3259e07f7c2p-16}, {0x1.0f5edfab325a2p-1, 0x1.c48acb8c5386cp-14},
-    {0x1.0e40655826011p-1, -0x1.1dbd93565013ap-15}, {0x1.0d24456359e3ap-1, 0x1.6da28bed90aebp-15},
-    {0x1.0c0a7868b4171p-1, 0x1.9672e671465afp-14}, {0x1.0af2f722eecb5p-1, -0x1.ef24a116d13a0p-14},
-    {0x1.09ddba6af8360p-1, -0x1.d922a355856dep-14}, {0x1.08cabb37565e2p-1, 0x1.d948fdf0ddd22p-14},
-    {0x1.07b9f29b8eae2p-1, 0x1.28ebdc7871acbp-14}, {0x1.06ab59c7912fbp-1, 0x1.69117d848d53cp-18},
-    {0x1.059eea0727586p-1, -0x1.5cfea0583643ap-14}, {0x1.04949cc1664c5p-1, 0x1.9e05fae11982bp-15},
-    {0x1.038c6b78247fcp-1, -0x1.64a621928396bp-14}, {0x1.02864fc7729e9p-1, 0x1.18f3a319fa1a3p-19},
-    {0x1.0182436517a37p-1, 0x1.180b8a89c05b7p-14}, {0x1.0080402010080p-1, 0x1.c9e2b7a341bd1p-14},};
-static __device__ const float kLogHi[128] = {
-    23, 69, 114, 159, 204, 249, 293, 336, 380, 423, 466, 508, 551, 593, 634, 675,
-    716, 757, 798, 838, 878, 918, 957, 996, 1035, 1074, 1112, 1150, 1188, 1226, 1263, 1300,
-    1337, 1374, 1410, 1446, 1483, 1518, 1554, 1589, 1624, 1659, 1694, 1729, 1763, 1797, 1831, 1865,
-    1899, 1932, 1965, 1998, 2031, 2064, 2096, 2128, 2161, 2192, 2224, 2256, 2287, 2319, 2350, 2381,
-    2411, 2442, 2472, 2503, 2533, 2563, 2593, 2622, 2652, 2681, 2711, 2740, 2769, 2798, 2826, 2855,
-    2883, 2911, 2940, 2968, 2995, 3023, 3051, 3078, 3106, 3133, 3160, 3187, 3214, 3241, 3267, 3294,
-    3320, 3346, 3373, 3399, 3424, 3450, 3476, 3502, 3527, 3552, 3578, 3603, 3628, 3653, 3678, 3702,
-    3727, 3751, 3776, 3800, 3824, 3849, 3873, 3896, 3920, 3944, 3968, 3991, 4015, 4038, 4061, 4084,};  // in units of 2^-12
-// 2^(j/256)
-static __device__ const double kExpTab[256] = {
-    0x1.0000000000000p+0, 0x1.00b1afa5abcbfp+0, 0x1.0163da9fb3335p+0, 0x1.02168143b0281p+0,
-    0x1.02c9a3e778061p+0, 0x1.037d42e11bbccp+0, 0x1.04315e86e7f85p+0, 0x1.04e5f72f654b1p+0,
-    0x1.059b0d3158574p+0, 0x1.0650a0e3c1f89p+0, 0x1.0706b29ddf6dep+0, 0x1.07bd42b72a836p+0,
-    0x1.0874518759bc8p+0, 0x1.092bdf66607e0p+0, 0x1.09e3ecac6f383p+0, 0x1.0a9c79b1f3919p+0,
-    0x1.0b5586cf9890fp+0, 0x1.0c0f145e46c85p+0, 0x1.0cc922b7247f7p+0, 0x1.0d83b23395decp+0,
-    0x1.0e3ec32d3d1a2p+0, 0x1.0efa55fdfa9c5p+0, 0x1.0fb66affed31bp+0, 0x1.1073028d7233ep+0,
-    0x1.11301d0125b51p+0, 0x1.11edbab5e2ab6p+0, 0x1.12abdc06c31ccp+0, 0x1.136a814f204abp+0,
-    0x1.1429aaea92de0p+0, 0x1.14e95934f312ep+0, 0x1.15a98c8a58e51p+0, 0x1.166a45471c3c2p+0,
-    0x1.172b83c7d517bp+0, 0x1.17ed48695bbc0p+0, 0x1.18af9388c8deap+0, 0x1.1972658375d2fp+0,
-    0x1.1a35beb6fcb75p+0, 0x1.1af99f8138a1cp+0, 0x1.1bbe084045cd4p+0, 0x1.1c82f95281c6bp+0,
-    0x1.1d4873168b9aap+0, 0x1.1e0e75eb44027p+0, 0x1.1ed5022fcd91dp+0, 0x1.1f9c18438ce4dp+0,
-    0x1.2063b88628cd6p+0, 0x1.212be3578a819p+0, 0x1.21f49917ddc96p+0, 0x1.22bdda27912d1p+0,
-    0x1.2387a6e756238p+0, 0x1.2451ffb82140ap+0, 0x1.251ce4fb2a63fp+0, 0x1.25e85711ece75p+0,
-    0x1.26b4565e27cddp+0, 0x1.2780e341ddf29p+0, 0x1.284dfe1f56381p+0, 0x1.291ba7591bb70p+0,
-    0x1.29e9df51fdee1p+0, 0x1.2ab8a66d10f13p+0, 0x1.2b87fd0dad990p+0, 0x1.2c57e39771b2fp+0,
-    0x1.2d285a6e4030bp+0, 0x1.2df961f641589p+0, 0x1.2ecafa93e2f56p+0, 0x1.2f9d24abd886bp+0,
-    0x1.306fe0a31b715p+0, 0x1.31432edeeb2fdp+0, 0x1.32170fc4cd831p+0, 0x1.32eb83ba8ea32p+0,
-    0x1.33c08b26416ffp+0, 0x1.3496266e3fa2dp+0, 0x1.356c55f929ff1p+0, 0x1.36431a2de883bp+0,
-    0x1.371a7373aa9cbp+0, 0x1.37f26231e754ap+0, 0x1.38cae6d05d866p+0, 0x1.39a401b7140efp+0,
-    0x1.3a7db34e59ff7p+0, 0x1.3b57fbfec6cf4p+0, 0x1.3c32dc313a8e5p+0, 0x1.3d0e544ede173p+0,
-    0x1.3dea64c123422p+0, 0x1.3ec70df1c5175p+0, 0x1.3fa4504ac801cp+0, 0x1.40822c367a024p+0,
-    0x1.4160a21f72e2ap+0, 0x1.423fb2709468ap+0, 0x1.431f5d950a897p+0, 0x1.43ffa3f84b9d4p+0,
-    0x1.44e086061892dp+0, 0x1.45c2042a7d232p+0, 0x1.46a41ed1d0057p+0, 0x1.4786d668b3237p+0,
-    0x1.486a2b5c13cd0p+0, 0x1.494e1e192aed2p+0, 0x1.4a32af0d7d3dep+0, 0x1.4b17dea6db7d7p+0,
-    0x1.4bfdad5362a27p+0, 0x1.4ce41b817c114p+0, 0x1.4dcb299fddd0dp+0, 0x1.4eb2d81d8abffp+0,
-    0x1.4f9b2769d2ca7p+0, 0x1.508417f4531eep+0, 0x1.516daa2cf6642p+0, 0x1.5257de83f4eefp+0,
-    0x1.5342b569d4f82p+0, 0x1.542e2f4f6ad27p+0, 0x1.551a4ca5d920fp+0, 0x1.56070dde910d2p+0,
-    0x1.56f4736b527dap+0, 0x1.57e27dbe2c4cfp+0, 0x1.58d12d497c7fdp+0, 0x1.59c0827ff07ccp+0,
-    0x1.5ab07dd485429p+0, 0x1.5ba11fba87a03p+0, 0x1.5c9268a5946b7p+0, 0x1.5d84590998b93p+0,
-    0x1.5e76f15ad2148p+0, 0x1.5f6a320dceb71p+0, 0x1.605e1b976dc09p+0, 0x1.6152ae6cdf6f4p+0,
-    0x1.6247eb03a5585p+0, 0x1.633dd1d1929fdp+0, 0x1.6434634ccc320p+0, 0x1.652b9febc8fb7p+0,
-    0x1.6623882552225p+0, 0x1.671c1c70833f6p+0, 0x1.68155d44ca973p+0, 0x1.690f4b19e9538p+0,
-    0x1.6a09e667f3bcdp+0, 0x1.6b052fa75173ep+0, 0x1.6c012750bdabfp+0, 0x1.6cfdcddd47645p+0,
-    0x1.6dfb23c651a2fp+0, 0x1.6ef9298593ae5p+0, 0x1.6ff7df9519484p+0, 0x1.70f7466f42e87p+0,
-    0x1.71f75e8ec5f74p+0, 0x1.72f8286ead08ap+0, 0x1.73f9a48a58174p+0, 0x1.74fbd35d7cbfdp+0,
-    0x1.75feb564267c9p+0, 0x1.77024b1ab6e09p+0, 0x1.780694fde5d3fp+0, 0x1.790b938ac1cf6p+0,
-    0x1.7a11473eb0187p+0, 0x1.7b17b0976cfdbp+0, 0x1.7c1ed0130c132p+0, 0x1.7d26a62ff86f0p+0,
-    0x1.7e2f336cf4e62p+0, 0x1.7f3878491c491p+0, 0x1.80427543e1a12p+0, 0x1.814d2add106d9p+0,
-    0x1.82589994cce13p+0, 0x1.8364c1eb941f7p+0, 0x1.8471a4623c7adp+0, 0x1.857f4179f5b21p+0,
-    0x1.868d99b4492edp+0, 0x1.879cad931a436p+0, 0x1.88ac7d98a6699p+0, 0x1.89bd0a478580fp+0,
-    0x1.8ace5422aa0dbp+0, 0x1.8be05bad61778p+0, 0x1.8cf3216b5448cp+0, 0x1.8e06a5e0866d9p+0,
-    0x1.8f1ae99157736p+0, 0x1.902fed0282c8ap+0, 0x1.9145b0b91ffc6p+0, 0x1.925c353aa2fe2p+0,
-    0x1.93737b0cdc5e5p+0, 0x1.948b82b5f98e5p+0, 0x1.95a44cbc8520fp+0, 0x1.96bdd9a7670b3p+0,
-    0x1.97d829fde4e50p+0, 0x1.98f33e47a22a2p+0, 0x1.9a0f170ca07bap+0, 0x1.9b2bb4d53fe0dp+0,
-    0x1.9c49182a3f090p+0, 0x1.9d674194bb8d5p+0, 0x1.9e86319e32323p+0, 0x1.9fa5e8d07f29ep+0,
-    0x1.a0c667b5de565p+0, 0x1.a1e7aed8eb8bbp+0, 0x1.a309bec4a2d33p+0, 0x1.a42c980460ad8p+0,
-    0x1.a5503b23e255dp+0, 0x1.a674a8af46052p+0, 0x1.a799e1330b358p+0, 0x1.a8bfe53c12e59p+0,
-    0x1.a9e6b5579fdbfp+0, 0x1.ab0e521356ebap+0, 0x1.ac36bbfd3f37ap+0, 0x1.ad5ff3a3c2774p+0,
-    0x1.ae89f995ad3adp+0, 0x1.afb4ce622f2ffp+0, 0x1.b0e07298db666p+0, 0x1.b20ce6c9a8952p+0,
-    0x1.b33a2b84f15fbp+0, 0x1.b468415b749b1p+0, 0x1.b59728de5593ap+0, 0x1.b6c6e29f1c52ap+0,
-    0x1.b7f76f2fb5e47p+0, 0x1.b928cf22749e4p+0, 0x1.ba5b030a1064ap+0, 0x1.bb8e0b79a6f1fp+0,
-    0x1.bcc1e904bc1d2p+0, 0x1.bdf69c3f3a207p+0, 0x1.bf2c25bd71e09p+0, 0x1.c06286141b33dp+0,
-    0x1.c199bdd85529cp+0, 0x1.c2d1cd9fa652cp+0, 0x1.c40ab5fffd07ap+0, 0x1.c544778fafb22p+0,
-    0x1.c67f12e57d14bp+0, 0x1.c7ba88988c933p+0, 0x1.c8f6d9406e7b5p+0, 0x1.ca3405751c4dbp+0,
-    0x1.cb720dcef9069p+0, 0x1.ccb0f2e6d1675p+0, 0x1.cdf0b555dc3fap+0, 0x1.cf3155b5bab74p+0,
-    0x1.d072d4a07897cp+0, 0x1.d1b532b08c968p+0, 0x1.d2f87080d89f2p+0, 0x1.d43c8eacaa1d6p+0,
-    0x1.d5818dcfba487p+0, 0x1.d6c76e862e6d3p+0, 0x1.d80e316c98398p+0, 0x1.d955d71ff6075p+0,
-    0x1.da9e603db3285p+0, 0x1.dbe7cd63a8315p+0, 0x1.dd321f301b460p+0, 0x1.de7d5641c0658p+0,
-    0x1.dfc97337b9b5fp+0, 0x1.e11676b197d17p+0, 0x1.e264614f5a129p+0, 0x1.e3b333b16ee12p+0,
-    0x1.e502ee78b3ff6p+0, 0x1.e653924676d76p+0, 0x1.e7a51fbc74c83p+0, 0x1.e8f7977cdb740p+0,
-    0x1.ea4afa2a490dap+0, 0x1.eb9f4867cca6ep+0, 0x1.ecf482d8e67f1p+0, 0x1.ee4aaa2188510p+0,
-    0x1.efa1bee615a27p+0, 0x1.f0f9c1cb6412ap+0, 0x1.f252b376bba97p+0, 0x1.f3ac948dd7274p+0,
-    0x1.f50765b6e4540p+0, 0x1.f6632798844f8p+0, 0x1.f7bfdad9cbe14p+0, 0x1.f91d802243c89p+0,
-    0x1.fa7c1819e90d8p+0, 0x1.fbdba3692d514p+0, 0x1.fd3c22b8f71f1p+0, 0x1.fe9d96b2a23d9p+0,};
+    {0x000000000000000ull, 0x80000000u}, {0x005bf942d5f6cf7ull, 0x7f01fc08u}, {0x00b73cb3d332c83ull, 0x7e07e07fu},
+    {0x0111cd1d01da1bcull, 0x7d11967au}, {0x016bad37532a86aull, 0x7c1f07c2u}, {0x01c4dfab339cee2ull, 0x7b301ecdu},
+    {0x021d6713dd3eabfull, 0x7a44c6b0u}, {0x027545fb467f1c1ull, 0x795ceb25u}, {0x02cc7edf2532823ull, 0x78787879u},
+    {0x0323142dbd3bc7aull, 0x77975b90u}, {0x037908480b9c281ull, 0x76b981dbu}, {0x03ce5d8223b1685ull, 0x75ded953u},
+    {0x04231622d484097ull, 0x75075076u}, {0x04773465b9e19a1ull, 0x7432d63eu}, {0x04caba783d826b9ull, 0x73615a25u},
+    {0x051daa7e2b9c9e3ull, 0x7292cc16u}, {0x0570068e67e05a8ull, 0x71c71c72u}, {0x05c1d0b4d9a6306ull, 0x70fe3c08u},
+    {0x06130af3a5527ffull, 0x70381c0fu}, {0x0663b74196c10e7ull, 0x6f74ae27u}, {0x06b3d78b055b63bull, 0x6eb3e454u},
+    {0x07036db336d8f74ull, 0x6df5b0f8u}, {0x07527b92e4311f0ull, 0x6d3a06d4u}, {0x07a102f9b26bfc9ull, 0x6c80d902u},
+    {0x07ef05ae0caa21eull, 0x6bca1af3u}, {0x083c856d731aec6ull, 0x6b15c06cu}, {0x088983ed440326eull, 0x6a63bd82u},
+    {0x08d602d8f54b156ull, 0x69b4069cu}, {0x092203d5195e89aull, 0x6906906au}, {0x096d887e1cb4088ull, 0x685b4fe6u},
+    {0x09b89266fd487f3ull, 0x67b23a55u}, {0x0a03231d5c74ed0ull, 0x670b453cu}, {0x0a4d3c25a14def5ull, 0x66666667u},
+    {0x0a96defdc93d91full, 0x65c393e1u}, {0x0ae00d1cb2e61bcull, 0x6522c3f4u}, {0x0b28c7f1dd2e07bull, 0x6483ed28u},
+    {0x0b7110e68c2941full, 0x63e7063fu}, {0x0bb8e95d21ea5a8ull, 0x634c0635u}, {0x0c0052b1658b961ull, 0x62b2e43eu},
+    {0x0c474e394a1dd49ull, 0x621b97c3u}, {0x0c8ddd4455d651eull, 0x61861862u}, {0x0cd4011c75d2518ull, 0x60f25debu},
+    {0x0d19bb04f339abdull, 0x60606061u}, {0x0d5f0c3c471897eull, 0x5fd017f5u}, {0x0da3f5fb967bfe8ull, 0x5f417d06u},
+    {0x0de87974b7303cfull, 0x5eb48824u}, {0x0e2c97d686405eaull, 0x5e293206u}, {0x0e70524906cfa14ull, 0x5d9f7391u},
+    {0x0eb3a9efd435315ull, 0x5d1745d2u}, {0x0ef69fe9af2215aull, 0x5c90a1feu}, {0x0f3935508a59535ull, 0x5c0b8171u},
+    {0x0f7b6b3919d004full, 0x5b87ddaeu}, {0x0fbd42b3e68e5ecull, 0x5b05b05cu}, {0x0ffebccce71c044ull, 0x5a84f346u},
+    {0x103fda8b1733221ull, 0x5a05a05bu}, {0x10809cf21ec7226ull, 0x5987b1aau}, {0x10c105006895934ull, 0x590b2165u},
+    {0x110113b0d1388eaull, 0x588fe9ddu}, {0x1140c9fa4e3820dull, 0x58160582u}, {0x118028cf0d9a51full, 0x579d6ee4u},
+    {0x11bf311e3698476ull, 0x572620afu}, {0x11fde3d2890e218ull, 0x56b015adu}, {0x123c41d3a0fc191ull, 0x563b48c3u},
+    {0x127a4c051f5d8b3ull, 0x55c7b4f2u}, {0x12b80346e325b36ull, 0x55555556u}, {0x12f56875d14735cull, 0x54e42524u},
+    {0x13327c6a7522227ull, 0x54741facu}, {0x136f3ffae3ca602ull, 0x54054055u}, {0x13abb3fa7a9ed2dull, 0x5397829du},
+    {0x13e7d937650239bull, 0x532ae21du}, {0x1423b07e336d911ull, 0x52bf5a82u}, {0x145f3a988473f53ull, 0x5254e78fu},
+    {0x149a784ba4b64e1ull, 0x51eb851fu}, {0x14d56a5b1cb97ceull, 0x51832f20u}, {0x15101186c64bcbaull, 0x511be196u},
+    {0x154a6e8c43291e4ull, 0x50b59898u}, {0x1584822633a01b7ull, 0x50505051u}, {0x15be4d0c904a4aeull, 0x4fec04ffu},
+    {0x15f7cff3de8f2a6ull, 0x4f88b2f4u}, {0x16310b8f4b16f90ull, 0x4f265692u}, {0x166a008e24e8e0bull, 0x4ec4ec4fu},
+    {0x16a2af9dfd01424ull, 0x4e6470b1u}, {0x16db1969e1804e4ull, 0x4e04e04fu}, {0x17133e9ac4a2020ull, 0x4da637d0u},
+    {0x174b1fd61cfa1c1ull, 0x4d4873edu}, {0x1782bdbf7cfd3c8ull, 0x4ceb916eu}, {0x17ba18f9028457eull, 0x4c8f8d29u},
+    {0x17f132215e052c1ull, 0x4c346405u}, {0x182809d5736b4adull, 0x4bda12f7u}, {0x185ea0b03214c8full, 0x4b809702u},
+    {0x1894f74a6c913ddull, 0x4b27ed37u}, {0x18cb0e3ab024c60ull, 0x4ad012b5u}, {0x1900e615bac2f6dull, 0x4a7904a8u},
+    {0x19367f6d16e42c8ull, 0x4a22c04bu}, {0x196bdad20f74ff9ull, 0x49cd42e3u}, {0x19a0f8d311755adull, 0x497889c3u},
+    {0x19d5d9fcc591071ull, 0x4924924au}, {0x1a0a7ed9ed9210aull, 0x48d159e3u}, {0x1a3ee7f341a1a25ull, 0x487ede05u},
+    {0x1a7315cff11797eull, 0x482d1c32u}, {0x1aa708f4de7fdfcull, 0x47dc11f8u}, {0x1adac1e7110f889ull, 0x478bbcedu},
+    {0x1b0e41267051ef6ull, 0x473c1ab7u}, {0x1b4187341467904ull, 0x46ed2902u}, {0x1b74948ef3186aeull, 0x469ee585u},
+    {0x1ba769b317650aeull, 0x46514e03u}, {0x1bda071c20957c9ull, 0x46046047u}, {0x1c0c6d43d9578b3ull, 0x45b81a26u},
+    {0x1c3e9ca2c4c5bbfull, 0x456c797eu}, {0x1c7095ae03c6c7eull, 0x45217c39u}, {0x1ca258dc8dc9d17ull, 0x44d72045u},
+    {0x1cd3e6a06cc294bull, 0x448d639eu}, {0x1d053f6ca7138dcull, 0x44444445u}, {0x1d3663b27c4f2c4ull, 0x43fbc044u},
+    {0x1d6753dfedaa38dull, 0x43b3d5b0u}, {0x1d981063b7f3100ull, 0x436c82a3u}, {0x1dc899ab374d71aull, 0x4325c53fu},
+    {0x1df8f0203dd402full, 0x42df9bb1u}, {0x1e29142dcba412eull, 0x429a042au}, {0x1e59063bd8d9383ull, 0x4254fce5u},
+    {0x1e88c6b2b54adb3ull, 0x42108422u}, {0x1eb855f82d4804bull, 0x41cc982au}, {0x1ee7b4718b44139ull, 0x4189374cu},
+    {0x1f16e281680bcb4ull, 0x41465fe0u}, {0x1f45e08b1c216c0ull, 0x41041042u}, {0x1f74aef092a1e61ull, 0x40c246d5u},
+    {0x1fa34e10c64e9e9ull, 0x40810205u}, {0x1fd1be4bf563f72ull, 0x40404041u}};
+// 2^(i/256), in units of 2^-62.
+static __device__ const unsigned long long kExpTab[256] = {
+    0x4000000000000000ull, 0x402c6be96af2fb58ull, 0x4058f6a7ecccd5b6ull, 0x4085a050ec0a036aull,
+    0x40b268f9de0183baull, 0x40df50b846ef302bull, 0x410c57a1b9fe12f6ull, 0x41397dcbd952c4a6ull,
+    0x4166c34c5615d0ecull, 0x41942838f07e22a3ull, 0x41c1aca777db771bull, 0x41ef50adcaa0d899ull,
+    0x421d1461d66f2023ull, 0x424af7d9981f7e98ull, 0x4278fb2b1bce0d15ull, 0x42a71e6c7ce464afull,
+    0x42d561b3e6243d8aull, 0x4303c51791b21550ull, 0x433248adc91fdd02ull, 0x4360ec8ce577ae44ull,
+    0x438fb0cb4f468808ull, 0x43be957f7ea712b6ull, 0x43ed9abffb4c6bc9ull, 0x441cc0a35c8cf8eaull,
+    0x444c0740496d4294ull, 0x447b6ead78aad636ull, 0x44aaf701b0c72feeull, 0x44daa053c812abd2ull,
+    0x450a6abaa4b77ecdull, 0x453a564d3cc4b723ull, 0x456a632296394492ull, 0x459a9151c70f0819ull,
+    0x45cae0f1f545eb73ull, 0x45fb521a56ef0042ull, 0x462be4e23237a6efull, 0x465c9960dd74bd4bull,
+    0x468d6fadbf2dd4f3ull, 0x46be67e04e28717cull, 0x46ef821011734e6bull, 0x4720be54a071ad01ull,
+    0x47521cc5a2e6a9e0ull, 0x47839d7ad1009a90ull, 0x47b5408bf36472e2ull, 0x47e70610e3393241ull,
+    0x4818ee218a3358eeull, 0x484af8d5e2a06536ull, 0x487d2645f7725895ull, 0x48af7689e44b44eaull,
+    0x48e1e9b9d588e19bull, 0x49147fee085028d6ull, 0x4947393eca98fcd6ull, 0x497a15c47b39d53eull,
+    0x49ad159789f37496ull, 0x49e038d0777ca5e0ull, 0x4a137f87d58e025bull, 0x4a46e9d646edbf6aull,
+    0x4a7a77d47f7b84b1ull, 0x4aae299b443c4a6bull, 0x4ae1ff436b663ff7ull, 0x4b15f8e5dc6cbab0ull,
+    0x4b4a169b900c2d00ull, 0x4b7e587d905625d1ull, 0x4bb2bea4f8bd5847ull, 0x4be7492af621abd6ull,
+    0x4c1bf828c6dc54b8ull, 0x4c50cbb7bacbf4cbull, 0x4c85c3f13360c4d5ull, 0x4cbae0eea3a8c63cull,
+    0x4cf022c9905bfd32ull, 0x4d25899b8fe8b365ull, 0x4d5b157e4a7fc325ull, 0x4d90c68b7a20eb1eull,
+    0x4dc69cdceaa72a9cull, 0x4dfc988c79d52661ull, 0x4e32b9b417619617ull, 0x4e69006dc503ba65ull,
+    0x4e9f6cd3967fdba8ull, 0x4ed5feffb1b3d155ull, 0x4f0cb70c4ea39210ull, 0x4f439513b785cc80ull,
+    0x4f7a993048d088d7ull, 0x4fb1c37c7145d328ull, 0x4fe91412b2006e83ull, 0x50208b0d9e8090dfull,
+    0x50582887dcb8a7e1ull, 0x508fec9c251a267cull, 0x50c7d76542a25b72ull, 0x50ffe8fe12e750c4ull,
+    0x513821818624b40cull, 0x5170810a9f48c7cfull, 0x51a907b474015dc9ull, 0x51e1b59a2cc8da3eull,
+    0x521a8ad704f3404full, 0x525387864abb4762ull, 0x528cabc35f4f799dull, 0x52c5f7a9b6df5b77ull,
+    0x52ff6b54d8a89c75ull, 0x533906e05f045106ull, 0x5372ca67f774358full, 0x53acb60762affaaeull,
+    0x53e6c9da74b29ab5ull, 0x542105fd14c7b869ull, 0x545b6a8b3d990704ull, 0x5495f7a0fd3bbb8eull,
+    0x54d0ad5a753e077cull, 0x550b8bd3dab49cbdull, 0x5546932976483b15ull, 0x5581c377a44346f0ull,
+    0x55bd1cdad49f699cull, 0x55f89f6f8b133af4ull, 0x56344b525f1ff495ull, 0x5670209ffc1f2e82ull,
+    0x56ac1f752150a563ull, 0x56e847eea1e80a49ull, 0x57249a29651adc07ull, 0x57611642662e4a33ull,
+    0x579dbc56b48521baull, 0x57da8c8373adc331ull, 0x581786e5db7022c2ull, 0x5854ab9b37dbd1e5ull,
+    0x5891fac0e95612c8ull, 0x58cf747464a7f584ull, 0x590d18d3330c7f1eull, 0x594ae7faf23eda52ull,
+    0x5988e20954889245ull, 0x59c7071c20cfd70cull, 0x5a05575132a5cc20ull, 0x5a43d2c67a54e0c0ull,
+    0x5a827999fcef3242ull, 0x5ac14be9d45cf869ull, 0x5b0049d42f6afbb6ull, 0x5b3f737751d915c8ull,
+    0x5b7ec8f19468bbc9ull, 0x5bbe4a6164eb92f4ull, 0x5bfdf7e546520f3eull, 0x5c3dd19bd0ba1c1aull,
+    0x5c7dd7a3b17dcf75ull, 0x5cbe0a1bab4226dfull, 0x5cfe69229605cef5ull, 0x5d3ef4d75f2ff504ull,
+    0x5d7fad59099f22feull, 0x5dc092c6adb825b8ull, 0x5e01a53f7974fd86ull, 0x5e42e4e2b073d935ull,
+    0x5e8451cfac061b5full, 0x5ec5ec25db3f6a41ull, 0x5f07b404c304c9f1ull, 0x5f49a98bfe1bc11cull,
+    0x5f8bccdb3d398841ull, 0x5fce1e124712437cull, 0x60109d50f86846d8ull, 0x60534ab7441b6546ull,
+    0x6096266533384a2bull, 0x60d9307ae507dd9aull, 0x611c69188f1eb339ull, 0x615fd05e7d6c83e4ull,
+    0x61a3666d124bb204ull, 0x61e72b64c690d8afull, 0x622b1f66299a6599ull, 0x626f4291e1603dd5ull,
+    0x62b39508aa836d6full, 0x62f816eb585de1edull, 0x633cc85ad5122fbdull, 0x6381a978219b628full,
+    0x63c6ba6455dcd8aeull, 0x640bfb40a0b22959ull, 0x64516c2e47ff1623ull, 0x64970d4ea8bf8766ull,
+    0x64dcdec3371793d1ull, 0x6522e0ad7e639312ull, 0x6569132f21483ba7ull, 0x65af7669d9c2cbe4ull,
+    0x65f60a7f79393e2eull, 0x663ccf91e88a8873ull, 0x6683c5c3281ee6e9ull, 0x66caed354ff83222ull,
+    0x6712460a8fc24072ull, 0x6759d0652ee352afull, 0x67a18c678c8c8c61ull, 0x67e97a341fca775bull,
+    0x683199ed779592caull, 0x6879ebb63ae2edc6ull, 0x68c26fb128b4cd63ull, 0x690b2601182b5e56ull,
+    0x69540ec8f895722dull, 0x699d2a2bd181482aull, 0x69e6784cc2cd61bdull, 0x6a2ff94f04b962b0ull,
+    0x6a79ad55e7f6fd10ull, 0x6ac39484d5bae8c5ull, 0x6b0daeff4fcde703ull, 0x6b57fce8f09dd17full,
+    0x6ba27e656b4eb57aull, 0x6bed33988bcbfab5ull, 0x6c381ca636d99642ull, 0x6c8339b26a25494eull,
+    0x6cce8ae13c57ebdbull, 0x6d1a1056dd26c382ull, 0x6d65ca379564e639ull, 0x6db1b8a7c714a92bull,
+    0x6dfddbcbed791babull, 0x6e4a33c89d278e49ull, 0x6e96c0c284192610ull, 0x6ee382de69bc7bf8ull,
+    0x6f307a412f074892ull, 0x6f7da70fce881bf9ull, 0x6fcb096f5c782210ull, 0x7018a18506ccf314ull,
+    0x70666f76154a7089ull, 0x70b47367e994ae92ull, 0x7102ad7fff41e9b4ull, 0x71511de3ebec8913ull,
+    0x719fc4b95f452d29ull, 0x71eea2262324cb0cull, 0x723db6501b9ed447ull, 0x728d015d47136b40ull,
+    0x72dc8373be41a454ull, 0x732c3cb9b459d38bull, 0x737c2d55770fe711ull, 0x73cc556d6eadce5full,
+    0x741cb5281e25ee34ull, 0x746d4cac2325a155ull, 0x74be1c203627c62bull, 0x750f23ab2a87593eull,
+    0x75606373ee921c97ull, 0x75b1dba18b9b4c20ull, 0x76038c5b260e5eeeull, 0x765575c7fd81d5a0ull,
+    0x76a7980f6cca15c2ull, 0x76f9f358ea0c5249ull, 0x774c87cc06d1812eull, 0x779f559070195e36ull,
+    0x77f25ccdee6d7ae6ull, 0x78459dac65f45bb5ull, 0x78991853d684a285ull, 0x78ecccec5bb84661ull,
+    0x7940bb9e2cffd89dull, 0x7994e4919db5d74eull, 0x79e947ef1d320d2dull, 0x7a3de5df36dcfeefull,
+    0x7a92be8a92436616ull, 0x7ae7d219f329b948ull, 0x7b3d20b6399fc237ull, 0x7b92aa886214411cull,
+    0x7be86fb985689ddcull, 0x7c3e7072d904a6ceull, 0x7c94acddaeea5d3aull, 0x7ceb252375c9cf9bull,
+    0x7d41d96db915019dull, 0x7d98c9e62113e1faull, 0x7deff6b672f84e24ull, 0x7e47600890f223deull,
+    0x7e9f06067a4360baull, 0x7ef6e8da4b544f9aull, 0x7f4f08ae3dc7c426ull, 0x7fa765aca88f6453ull};
 
 __device__ __forceinline__ int hi_word(double x) { return __double2hiint(x); }
 __device__ __forceinline__ int lo_word(double x) { return __double2loint(x); }
@@ -200,34 +176,55 @@ __device__ __forceinline__ long long order_f64(double x) {
   return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-// log2 E of a positive, normal E.
-__device__ __forceinline__ double log2_f64(double E) {
-  const int h = hi_word(E);
-  const int j = (h >> 13) & 127;
-  const double m = __hiloint2double((h & 0x000fffff) | 0x3ff00000, lo_word(E));
-  const LogRow t = kLogTab[j];
-  const double r = fma(m, t.c, -1.0);  // exact up to its own last bit
-  // exponent - log2 c's leading part, exact in FP32
-  const float ehi = fmaf(kLogHi[j], 1.0f / 4096.0f, (float)((h >> 20) - 1023));
-  double p = fma(r, kLog5, kLog4);
-  p = fma(p, r, kLog3);
-  p = fma(p, r, kLog2);
-  p = fma(p, r, kLog1);
-  return f64_of_f32(ehi) + fma(p, r, t.lo);
+// The upper 64 bits of a b, at most 2 below (the product of the lower halves is left
+// out).
+__device__ __forceinline__ uint64_t mul_hi64(uint64_t a, uint64_t b) {
+  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32),
+                 bl = (uint32_t)b;
+  return (uint64_t)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh);
+}
+// The same for a of 32 + S bits: cheaper, and at most 2 below too.
+template <int S>
+__device__ __forceinline__ uint64_t mul_hi_short(uint64_t a, uint32_t bh, uint32_t bl) {
+  return (((uint64_t)(uint32_t)a * bh) >> 32) + (uint64_t)(uint32_t)(a >> 32) * bh +
+         (__umulhi((uint32_t)(a >> S), bl) >> (32 - S));
 }
 
-// 1/E of a positive, normal E (0 above 2^1020): the FP32 reciprocal of its
-// mantissa, one step of the cubic iteration s (1 + d + d^2), d = 1 - m s.
+// log2 E of a positive, normal E: exponent - log2 c + log2(m c), the last two in fixed
+// point, rounded to 2^-52 as the fraction of a number in [1, 2].
+__device__ __forceinline__ double log2_f64(double E) {
+  const uint32_t h = (uint32_t)hi_word(E), l = (uint32_t)lo_word(E);
+  const LogRow t = kLogTab[(h >> 13) & 127];
+  const uint64_t m = ((uint64_t)((h & 0xfffffu) | 0x100000u) << 32 | l) << 11;
+  // m c - 1 = rho/64, m c in units of 2^-62
+  const uint64_t mc = (uint64_t)(uint32_t)(m >> 32) * t.c + __umulhi((uint32_t)m, t.c);
+  const uint64_t rho = mc << 8;  // the 1 shifted out
+  const uint32_t rh = (uint32_t)(rho >> 32), rl = (uint32_t)rho;
+  const uint64_t B = kLog3 - __umulhi(kLog4 - __umulhi(kLog5 - __umulhi(kLog6, rh), rh), rh);
+  const uint64_t C = kLog2 - mul_hi_short<6>(B, rh, rl);
+  const uint64_t q = kLog1 - mul_hi_short<13>(C, rh, rl);
+  const uint64_t f = ((t.log + mul_hi64(rho, q) + 16u) >> 5) + 0x3ff0000000000000ull;
+  return f64_of_f32((float)((int)(h >> 20) - 1024)) + __longlong_as_double((long long)f);
+}
+
+// 1/E of a positive, normal E (0 above 2^1020): the FP32 reciprocal s of its
+// mantissa m, and s (1 + d + d^2), d = 1 - m s, in fixed point.
 __device__ __forceinline__ double rcp_f64(double E) {
-  const int h = hi_word(E), l = lo_word(E);
-  const double m = __hiloint2double((h & 0x000fffff) | 0x3ff00000, l);
-  const float mf = __uint_as_float(0x3f800000u | ((uint32_t)(h & 0x000fffff) << 3) |
-                                   ((uint32_t)l >> 29));
-  const double s = f64_of_f32(__fdividef(1.0f, mf));
-  const double d = fma(-m, s, 1.0);
-  const double q = fma(s, fma(d, d, d), s);
-  const int e = (h >> 20) - 1023;
-  return e > 1020 ? 0.0 : __hiloint2double(hi_word(q) - (e << 20), lo_word(q));
+  const uint32_t h = (uint32_t)hi_word(E), l = (uint32_t)lo_word(E);
+  const uint32_t sb = __float_as_uint(
+      fmaxf(__fdividef(1.0f, __uint_as_float(0x3f800000u | (h & 0xfffffu) << 3 | l >> 29)), 0.5f));
+  const uint32_t S = ((sb & 0x7fffffu) | 0x800000u) << ((sb >> 23) - 126u);  // units of 2^-24
+  // 1 - m s in units of 2^-76, below 2^-21: its low 64 bits are all of it
+  const long long d =
+      -(long long)((uint64_t)l * S + ((uint64_t)(((h & 0xfffffu) | 0x100000u) * S) << 32));
+  const int dq = (int)(d >> 40);
+  const long long t = (d >> 12) + ((uint32_t)(dq * dq) >> 8);  // d + d^2 in units of 2^-64
+  const uint64_t q = ((uint64_t)S << 36) + (uint64_t)(((long long)S * (t >> 4)) >> 24);
+  const uint64_t M = (q + 64u) >> 7;  // 53 bits, whose leading one adds 1 to the exponent field
+  const int e = (int)(h >> 20) - 1023;
+  return e > 1020 ? 0.0
+                  : __hiloint2double((int)((uint32_t)(M >> 32) + (uint32_t)((1021 - e) << 20)),
+                                     (int)(uint32_t)M);
 }
 
 // a / b for a normal b up to 2^1020.
@@ -236,24 +233,40 @@ __device__ __forceinline__ double div_f64(double a, double b) {
   return a * __hiloint2double(hi_word(r) ^ (hi_word(b) & (int)0x80000000), lo_word(r));
 }
 
-// 2^y; y is clamped to [-1200, 1000] (-1200: 0 after rounding).
+// 2^y in 64-bit integers; y is clamped to [-1200, 1000] (-1200: 0 after rounding).
+// With y in units of 2^-53, y = n + i/256 + rho/256 + ..: n the exponent, i the
+// table entry T = 2^(i/256), rho in [0, 1) the rest; 2^y = 2^n (T + T p), p =
+// 2^(rho/256) - 1 = rho/256 q(rho), q a cubic in units of 2^-52.
 __device__ __forceinline__ double exp2_f64(double y) {
-  const int yh = hi_word(y);
-  if (yh >= 0x408f4000) y = 1000.0;               // 2^1000 at most
-  if ((uint32_t)yh > 0xc092c000u) y = -1200.0;    // below -1200
-  constexpr double kMagic = 0x1.8p44;             // 8 fractional bits
-  const double t = y + kMagic;
-  const int n = lo_word(t);
-  const double r = y - (t - kMagic);
-  double p = fma(r, kExp4, kExp3);
-  p = fma(p, r, kExp2);
-  p = fma(p, r, kExp1);
-  const double T = kExpTab[n & 255];
-  const double v = fma(T, p * r, T);
-  const int e = n >> 8;
-  if (e >= -1021) return __hiloint2double(hi_word(v) + (e << 20), lo_word(v));
-  // below the normal range: scaled up by 2^256, then back with one rounding
-  return __hiloint2double(hi_word(v) + ((e + 256) << 20), lo_word(v)) * 0x1p-256;
+  uint32_t h = (uint32_t)hi_word(y), l = (uint32_t)lo_word(y);
+  const bool tiny = h >= 0xc08ff000u;  // y <= -1022: below the normal range
+  if (tiny) {
+    y = (h > 0xc092c000u ? -1200.0 : y) + 256.0;
+    h = (uint32_t)hi_word(y);
+    l = (uint32_t)lo_word(y);
+  }
+  if ((int)h >= 0x408f4000) {  // 2^1000 at most
+    h = 0x408f4000u;
+    l = 0;
+  }
+  // |y| in units of 2^-53, rounded where it has bits below
+  const uint32_t s = 1032u - ((h >> 20) & 0x7ffu);
+  uint64_t m = ((uint64_t)((h & 0xfffffu) | 0x100000u) << 32 | l) << 11;
+  m = s < 64u ? ((m >> s) + 1u) >> 1 : 0u;
+  const uint64_t Y = (int)h < 0 ? 0u - m : m;
+  const int yh = (int)(Y >> 32);
+  const uint64_t T = kExpTab[(yh >> 13) & 255];
+  const uint64_t rho = Y << 19;
+  const uint32_t rh = (uint32_t)(rho >> 32), rl = (uint32_t)rho;
+  const uint64_t B = kExp2 + __umulhi(kExp3 + __umulhi(kExp4, rh), rh);
+  const uint64_t q = kExp1 + mul_hi_short<10>(B, rh, rl);
+  const uint64_t p = mul_hi64(rho, q);              // units of 2^-60
+  const uint64_t S = T + (mul_hi64(T, p) << 4);     // units of 2^-62
+  // rounded to 53 bits, whose leading one adds 1 to the exponent field
+  const uint64_t M = (S + 512u) >> 10;
+  const double v = __hiloint2double((int)((uint32_t)(M >> 32) + (uint32_t)(((yh >> 21) + 1022) << 20)),
+                                    (int)(uint32_t)M);
+  return tiny ? v * 0x1p-256 : v;  // back with one rounding
 }
 
 // e^z for z <= 0: the product with log2 e rounds once, |z| 2^-53 relative to

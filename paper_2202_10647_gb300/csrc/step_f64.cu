@@ -146,7 +146,7 @@ __device__ __forceinline__ float estimate_f32(const StagedF32& tab, const Policy
   return lmax;
 }
 
-// 33.5M nitrogen cells: 2,340 us (5,573 with library functions, four FP64
+// 33.5M nitrogen cells: 1,922 us (5,573 with library functions, four FP64
 // instructions per slot and term, choices by FP64 comparisons and widths rounded up to
 // 2, 4, 6; 20 + 16 w bytes per cell take 381 us).
 __global__ void __launch_bounds__(kThreads, 2)
