@@ -79,7 +79,7 @@ __device__ __forceinline__ double f64_cell(const JobIO& J, const Policy& pol,
   }
   const double dne =
       lmax <= DDParams<double>::prop_max
-          ? taylor_flow_f64<W>(v, lam, DDParams<double>::terms(2.0f * lmax, DDParams<double>::PMAX))
+          ? taylor_flow_f64<W>(v, lam, flow_terms<W>(2.0f * lmax))
           : dd_update<double, W>(v, lam, W);
   if (check) {
 #pragma unroll
@@ -146,7 +146,7 @@ __device__ __forceinline__ float estimate_f32(const StagedF32& tab, const Policy
   return lmax;
 }
 
-// 33.5M nitrogen cells: 1,922 us (5,573 with library functions, four FP64
+// 33.5M nitrogen cells: 1,787 us (5,573 with library functions, four FP64
 // instructions per slot and term, choices by FP64 comparisons and widths rounded up to
 // 2, 4, 6; 20 + 16 w bytes per cell take 381 us).
 __global__ void __launch_bounds__(kThreads, 2)
