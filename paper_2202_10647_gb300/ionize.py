@@ -244,8 +244,13 @@ def _check(rc: int):
         raise IonError(rc, lib().ion_last_error().decode())
 
 
-def _stream(t: torch.Tensor):
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+# The host side of a call on a small patch costs more than its kernel, so
+# addresses and streams go to the library as integers (its declarations make them
+# pointers) and no device or stream object is made: step() of 16,384 cells takes
+# 10.7 us (16.7 with ctypes pointers, device and stream objects made on each call; its kernel
+# 6.4).
+def _stream(t: torch.Tensor) -> int:
+    return torch._C._cuda_getCurrentRawStream(t.get_device())
 
 
 def _stream_of(device):
@@ -255,18 +260,26 @@ def _stream_of(device):
 def _ptr(t, offset: int = 0):
     """Device address of element `offset` (along the last axis for the
     population planes, which keep their stride ld)."""
-    return None if t is None else ctypes.c_void_p(t.data_ptr() + offset * t.element_size())
+    if t is None:
+        return None
+    return t.data_ptr() + offset * t.element_size() if offset else t.data_ptr()
 
 
 def _need(t: torch.Tensor, name: str, dtype, device=None):
+    """Raises unless t is a contiguous CUDA tensor of dtype (on `device`, a torch.device or its
+    index)."""
+    index = device if device is None or type(device) is int else device.index
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype
+            and (index is None or t.get_device() == index) and t.is_contiguous()):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
-    if device is not None and t.device != device:
-        raise ValueError(f"{name} is on {t.device}, expected {device}")
+    if index is not None and t.get_device() != index:
+        raise ValueError(f"{name} is on {t.device}, expected cuda:{index}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
 
@@ -443,7 +456,7 @@ def step(sp: Species, E: torch.Tensor, N: torch.Tensor, k_lo: torch.Tensor,
     f64 = bool(flags & ION_F64_PLAIN)
     dt_ = torch.float64 if f64 else torch.float32
     _need(E, "E", dt_)
-    dev = E.device
+    dev = E.get_device()
     _need(N, "N", dt_, dev)
     _need(k_lo, "k_lo", torch.uint8, dev)
     _need(k_hi, "k_hi", torch.uint8, dev)
@@ -453,17 +466,18 @@ def step(sp: Species, E: torch.Tensor, N: torch.Tensor, k_lo: torch.Tensor,
     if N.dim() != 2 or N.shape[0] != sp.Z + 1:
         raise ValueError(f"N must have shape (Z+1, ld) = ({sp.Z + 1}, ld)")
     off = int(offset)
+    ld = N.shape[1]
     n = E.numel() - off if ncells is None else int(ncells)
     if off < 0 or n < 0 or off + n > min(E.numel(), k_lo.numel(), k_hi.numel(),
-                                         dne.numel(), N.shape[1]):
+                                         dne.numel(), ld):
         raise ValueError("offset/ncells outside the arrays")
     if n_gas is not None and off + n > n_gas.numel():
         raise ValueError("offset/ncells outside n_gas")
     if ws is None:
-        ws = workspace(n, flags, dev)
+        ws = workspace(n, flags, E.device)
     _need(ws, "ws", torch.uint8, dev)
     opts = _opts(eps_shift, degen_gap, window)
-    _check(lib().ion_step(sp.handle, _ptr(E, off), _ptr(N, off), N.shape[1], n,
+    _check(lib().ion_step(sp.handle, _ptr(E, off), _ptr(N, off), ld, n,
                           float(dt), _ptr(k_lo, off), _ptr(k_hi, off), _ptr(dne, off),
                           _ptr(n_gas, off), ctypes.byref(opts), int(flags), _ptr(ws),
                           ws.numel(), _stream(E)))
