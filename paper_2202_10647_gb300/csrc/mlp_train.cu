@@ -485,8 +485,8 @@ int check_common(const char* who, const float* P, int K, const float* x, int64_t
 // ---- training data ---------------------------------------------------------
 // x = clamp(2 (log2|E| - l2lo) / (l2hi - l2lo) - 1, -1, 1) in FP64, scale =
 // 2 / (l2hi - l2lo); the clamp after the rounding to float (rounding keeps
-// the order).  Bound by the FP64 pipe (a field's 12 instructions); 1,048,576
-// fields: 94 us with log2() and a division, 23 us now.
+// the order).  Bound by issue and the FP64 pipe; 1,048,576
+// fields: 94 us with log2() and a division, 11 us now.
 __global__ void mlp_inputs_kernel(const float* __restrict__ E, int64_t n, double l2lo,
                                   double scale, float* __restrict__ x) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -508,11 +508,15 @@ __global__ void mlp_inputs_kernel(const float* __restrict__ E, int64_t n, double
 // (T. F. Chan, G. H. Golub, R. J. LeVeque, "Algorithms for computing the
 // sample variance", Am. Stat. 37, 1983), in a fixed order.  The slices'
 // means and M2 wait in T, which the last kernel then overwrites.
-// Bound: 3 FP64 instructions per value for the moments (2 lanes per clock and
-// SM), memory for the scaling.  1,048,576 x 18 values: two passes of 18 blocks
-// took 2 x 918 us, scaling by an FP64 division 335 us; now 140 us (107 us of
-// FP64 issue) and 15 us to combine the slices, and 40 us (34 us of traffic;
-// 124 us with an FP64 product instead of the pairs).
+// A thread sums in 64-bit integers: its values in units of 2^-57 of the slice's largest
+// power of 2 in the column (finer than the ulps that FP64 sums of them round by), the
+// squared deviations in units of 2^-58 of the thread's largest; some 40 integer
+// instructions a value in the issue time of less than one of the three FP64 ones.  Columns
+// of slices with infinities or NaN, or of sizes beyond 2^400, take FP64.
+// 1,048,576 x 18 values: two passes of 18 blocks took 2 x 918 us, scaling by an FP64
+// division 335 us; moments by slices in FP64 140 us (107 us of FP64 issue), now 67 us
+// (23 us of traffic); 15 us to combine the slices, and 40 us to scale (34 us of
+// traffic; 124 us with an FP64 product instead of the pairs).
 constexpr int kStdThreads = 256;
 constexpr int kHold = 32;
 
@@ -548,33 +552,84 @@ __device__ __forceinline__ double get_f64(const float* p) {
   return __hiloint2double(__float_as_int(p[1]), __float_as_int(p[0]));
 }
 
+// x 2^(57 - E), towards 0, of a double x of at most 2^(E+1) in size, E + 1023 = e.
+__device__ __forceinline__ long long fixed_bits(long long x, int e) {
+  const uint32_t h = (uint32_t)(x >> 32), l = (uint32_t)x;
+  const uint64_t m = ((uint64_t)((h & 0xfffffu) | 0x100000u) << 32 | l) << 6;
+  const uint32_t s = (uint32_t)(e + 1) - ((h >> 20) & 0x7ffu);
+  const long long f = s < 64u ? (long long)(m >> s) : 0;
+  return (int)h < 0 ? -f : f;
+}
+__device__ __forceinline__ double power_of_2(int n) {
+  return __hiloint2double((1023 + n) << 20, 0);
+}
+
 // Slice blockIdx.x of the rows: its column means and M2 into
 // part_out[(2 slice + which) K + k].
 __global__ void __launch_bounds__(kStdThreads)
     mlp_moments_kernel(const double* __restrict__ Y, int64_t n, int K, float* part_out) {
   __shared__ double part[kStdThreads], means[kMaxOut];
+  __shared__ int top[kMaxOut];
   const int rows = kStdThreads / K;
   const int64_t r0 = blockIdx.x * (int64_t)rows * kHold;
   const int ns = (int)min((int64_t)rows * kHold, n - r0);  // rows of this slice
   const int row = threadIdx.x / K, k = threadIdx.x % K;
   const bool on = row < rows;
   const double* y = Y + r0 * K + threadIdx.x;
-  double v[kHold], s = 0.0;
+  long long v[kHold];  // the values' bits, then the fixed-point values
+  if (threadIdx.x < K) top[threadIdx.x] = 0;
+  int e = 0;  // the largest exponent field
 #pragma unroll
-  for (int i = 0; i < kHold; ++i)
-    v[i] = on && row + i * rows < ns ? __ldcs(y + (int64_t)i * rows * K) : 0.0;
+  for (int i = 0; i < kHold; ++i) {
+    v[i] = on && row + i * rows < ns ? __double_as_longlong(__ldcs(y + (int64_t)i * rows * K)) : 0;
+    e = max(e, (int)(v[i] >> 32) & 0x7ff00000);
+  }
+  __syncthreads();
+  if (on) atomicMax(&top[k], e >> 20);
+  __syncthreads();
+  e = top[k];
+  const bool fixed = e > 1023 - 400 && e < 1023 + 400;
+  double s = 0.0;
+  if (fixed) {
+    long long sum = 0;
 #pragma unroll
-  for (int i = 0; i < kHold; ++i) s += v[i];
+    for (int i = 0; i < kHold; ++i) {
+      v[i] = fixed_bits(v[i], e);
+      sum += v[i];
+    }
+    s = (double)sum * power_of_2(e - 1023 - 57);
+  } else {
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) s += __longlong_as_double(v[i]);
+  }
   const double sum = column_sum(s, part, K, rows);
   if (row == 0) means[k] = sum / (double)ns;
   __syncthreads();
   const double mean = means[k];
   double q = 0.0;
+  if (fixed) {
+    const long long m = fixed_bits(__double_as_longlong(mean), e);
+    unsigned long long all = 1, acc = 0;
 #pragma unroll
-  for (int i = 0; i < kHold; ++i) {
-    if (on && row + i * rows < ns) {
-      const double d = v[i] - mean;
-      q = fma(d, d, q);
+    for (int i = 0; i < kHold; ++i) {
+      const long long d = v[i] - m;
+      v[i] = on && row + i * rows < ns ? (d < 0 ? -d : d) : 0;
+      all |= (unsigned long long)v[i];
+    }
+    const int sh = __clzll((long long)all) - 3;  // |d| < 2^59: the largest to below 2^61
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) {
+      const uint64_t d = (uint64_t)v[i] << sh;
+      acc += mul_hi64(d, d);
+    }
+    q = (double)(long long)acc * power_of_2(64 - 2 * sh + 2 * (e - 1023 - 57));
+  } else {
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) {
+      if (on && row + i * rows < ns) {
+        const double d = __longlong_as_double(v[i]) - mean;
+        q = fma(d, d, q);
+      }
     }
   }
   const double m2 = column_sum(q, part, K, rows);
