@@ -928,7 +928,8 @@ def main():
         },
         "accuracy": acc,
         "peaks_measured": pk,
-        "gpu_launches": 3 * args.steps,
+        # the header's clearing, the streaming, record and queue kernels
+        "gpu_launches": 4 * args.steps,
         "clocks": clocks,
         "cpu_baseline": cpu,
         "e2e": e2e,

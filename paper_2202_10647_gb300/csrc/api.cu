@@ -638,9 +638,10 @@ int run_batch(const ion_batch_job* jobs, int njobs, double dt_fs, const ion_step
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e;
   if (f64) {
-    e = cudaMemsetAsync(a.ws.hdr, 0, ion::kHdrWords * sizeof(uint32_t), s);
+    bool dependent = false;
+    e = ion::launch_clear(a.ws.hdr, total, &dependent, s);
     for (int j = 0; j < njobs && e == cudaSuccess; ++j)
-      e = ion::launch_step_f64(a.job[j], a.pol, a.ws.hdr, j == 0, s);
+      e = ion::launch_step_f64(a.job[j], a.pol, a.ws.hdr, j == 0, dependent, s);
   } else {
     e = ion::launch_batch_f32(a, sh, jobs[0].species->num_sms, s);
   }

@@ -155,6 +155,27 @@ int job_from_args(const ion_species* sp, const void* E, void* N, int64_t ld, int
                   const char* who, JobIO* J);
 int workspace_ok(void* workspace, size_t have, size_t need);
 
+// Launches a kernel that follows another of the same call (programmatic dependent launch):
+// its blocks are set up while the last blocks of the one before finish, and what
+// that one writes is there after cudaGridDependencySynchronize, which every thread
+// calls.  Only inside a call: the first kernel of each is an ordinary launch, so that it
+// follows all that the stream held before.  `dependent` false: an ordinary launch.
+template <typename... P, typename... A>
+cudaError_t launch_after(bool dependent, void (*kernel)(P...), unsigned blocks, unsigned threads,
+                         size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Launchers.  They only enqueue; the caller has validated.  `a.job[j].chunk0`
 // and `a.nchunks` are filled in by launch_batch_f32.
 cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms,
@@ -169,9 +190,12 @@ cudaError_t launch_fb_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
 // otherwise).
 cudaError_t launch_net_select_f32(BatchArgs& a, const NetSelect& sel, int num_sms, bool* fits,
                                   cudaStream_t s);
-// `first`: nothing has run since the header was cleared.
+// `first`: nothing has run since the header was cleared (`dependent`: by a kernel).
 cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr, bool first,
-                            cudaStream_t s);
+                            bool dependent, cudaStream_t s);
+// Zeroes the workspace header for a step of `cells` cells; *dependent: by a kernel, which the
+// next one may follow as its dependent.
+cudaError_t launch_clear(uint32_t* hdr, int64_t cells, bool* dependent, cudaStream_t s);
 LaunchShape default_shape();
 bool valid_shape(const LaunchShape& s);
 

@@ -358,6 +358,7 @@ __global__ void __launch_bounds__(256)
     mlp_grad_sum(int np, int nparts, Parts in, float* __restrict__ grad,
                  float* __restrict__ loss, float inv_BK) {
   __shared__ float red[8][33];
+  cudaGridDependencySynchronize();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
   float g = 0.0f;
@@ -640,11 +641,14 @@ __global__ void __launch_bounds__(kStdThreads)
   }
 }
 
-// Block k: the mean and scale of column k from the slices' means and M2.
+// Block k: the mean and scale of column k from the slices' means and M2.  (What a dependent
+// kernel reads of the one before is not declared __restrict__: a read-only load may be taken
+// ahead of the wait.)
 __global__ void __launch_bounds__(kStdThreads)
-    mlp_moments_combine(const float* __restrict__ part_in, int64_t n, int K, int64_t slices,
+    mlp_moments_combine(const float* part_in, int64_t n, int K, int64_t slices,
                         double min_scale, double* mean_out, double* scale_out) {
   __shared__ double part[kStdThreads];
+  cudaGridDependencySynchronize();
   const int k = blockIdx.x;
   const int64_t per = (int64_t)(kStdThreads / K) * kHold;
   auto total = [&](double v) {
@@ -695,9 +699,9 @@ __device__ __forceinline__ void split_bits(double x, float& hi, float& lo, bool&
 // range, in FP64.  Every thread stays on one column.
 __global__ void __launch_bounds__(kStdThreads)
     mlp_normalize_kernel(const double* __restrict__ Y, int64_t n, int K,
-                         const double* __restrict__ mean, const double* __restrict__ scale,
-                         float* __restrict__ T) {
+                         const double* mean, const double* scale, float* __restrict__ T) {
   constexpr int kUnroll = 8;
+  cudaGridDependencySynchronize();
   const int rows = kStdThreads / K;
   if ((int)threadIdx.x >= rows * K) return;
   const int64_t step = (int64_t)rows * K;
@@ -821,9 +825,8 @@ int ion_mlp_loss_grad(const float* P, int K, const float* x, const float* t, int
   }
   if (e == cudaSuccess) {
     const int np = nparams(K);
-    mlp_grad_sum<<<(np + 31) / 32, 256, 0, s>>>(np, nparts, a, grad, loss,
-                                                (float)(1.0 / ((double)B * K)));
-    e = cudaGetLastError();
+    e = ion::launch_after(true, mlp_grad_sum, (np + 31) / 32, 256, 0, s, np, nparts, a, grad, loss,
+                          (float)(1.0 / ((double)B * K)));
   }
   if (e != cudaSuccess)
     return ion::set_error(ION_ECUDA, "ion_mlp_loss_grad launch: %s", cudaGetErrorString(e));
@@ -913,20 +916,24 @@ int ion_mlp_standardize(const double* Y, int64_t n, int K, double min_scale, dou
                           "ion_mlp_standardize: Y, mean_out, scale_out (8-byte aligned) and T "
                           "(4-byte aligned) must be non-NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaError_t e;
   const int64_t slices = (n + std_rows(K) - 1) / std_rows(K);
   // a slice's means and M2 take four floats per column of T: four rows
   if (n >= 4 * slices) {
     mlp_moments_kernel<<<(unsigned)slices, kStdThreads, 0, s>>>(Y, n, K, T);
-    mlp_moments_combine<<<K, kStdThreads, 0, s>>>(T, n, K, slices, min_scale, mean_out,
-                                                  scale_out);
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = ion::launch_after(true, mlp_moments_combine, K, kStdThreads, 0, s, T, n, K, slices, min_scale,
+                            mean_out, scale_out);
   } else {
     mlp_moments_small<<<K, kStdThreads, 0, s>>>(Y, n, K, min_scale, mean_out, scale_out);
+    e = cudaGetLastError();
   }
   const int64_t per = (int64_t)std_columns(K) * 8;
   const int64_t need = (n * K + per - 1) / per;
-  mlp_normalize_kernel<<<(unsigned)std::min<int64_t>(need, 4096), kStdThreads, 0, s>>>(
-      Y, n, K, mean_out, scale_out, T);
-  const cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = ion::launch_after(true, mlp_normalize_kernel, (unsigned)std::min<int64_t>(need, 4096),
+                          kStdThreads, 0, s, Y, n, K, mean_out, scale_out, T);
   if (e != cudaSuccess)
     return ion::set_error(ION_ECUDA, "ion_mlp_standardize launch: %s", cudaGetErrorString(e));
   return ion::set_error(ION_OK, "%s", "");

@@ -549,6 +549,7 @@ __global__ void __maxnreg__(stream_regs<Q>())
     for (int i = threadIdx.x; i < nz; i += blockDim.x) z[i] = 0.0f;
   }
   __syncthreads();
+  cudaGridDependencySynchronize();  // the header is zero
 
   constexpr int kChunk = 32 * Q;
   const int lane = threadIdx.x & 31;
@@ -834,6 +835,7 @@ __device__ __forceinline__ void lean_body(const BatchArgs& a, const NetSelect* s
     for (int i = threadIdx.x; i < nz; i += blockDim.x) z[i] = 0.0f;
   }
   __syncthreads();
+  cudaGridDependencySynchronize();  // the header is zero
 
   constexpr int kChunk = 32 * Q;
   constexpr uint32_t kStageBytes = sizeof(LStage<Q>);
@@ -1273,9 +1275,10 @@ __global__ void __launch_bounds__(128) ion_fb_kernel(const __grid_constant__ Bat
 // records and no queue.  On a grid of a few warps per SM the streaming kernel's
 // ring is mostly its own filling, and the two launches behind it find next to
 // nothing.  Steps of n nitrogen (Kr-like) cells in a graph, direct against
-// streaming, us: 16,384 6.4 against 25 (8.4, 29); 160,000 12 against 27 (19, 35);
-// 320,000 19 against 30 (31, 38); 500,000 25 against 31 (45, 42); 1,000,000 42 against
-// 31 (82, 52).  The line is where the heavier gas's crossing lies.
+// streaming, us: 16,384 4.3 against 15.5 (6.7, 24.6); 160,000 8.8 against 18.3 (15.5, 29.3);
+// 320,000 14.6 against 19.9 (27.4, 34.9); 400,000 17.1 against 20.2 (33.0, 35.9).  The line
+// is close to the heavier gas's crossing (before the launches of a call overlapped, 500,000
+// cells 25 against 31 and 45 against 42).
 // ---------------------------------------------------------------------------
 constexpr int kDirectThreads = 64;
 constexpr int kDirectCells = 400000;
@@ -1324,6 +1327,7 @@ __global__ void __launch_bounds__(kDirectThreads)
   const int lo = on ? J.lo[c] : 0, hi = on ? J.hi[c] : 0;
   for (int j = 0; j < a.njobs; ++j) stage_f32(a.job[j].tab, a.pol.log2dt, &tabs[j]);
   __syncthreads();
+  cudaGridDependencySynchronize();  // the header is zero
   const bool ok = on && window_ok(lo, hi, J.Z);
   if (on && !ok) atomicAdd(&a.ws.hdr[kHdrInvalid], 1u);
   const int w = ok ? hi - lo + 1 : 0;
@@ -1349,6 +1353,10 @@ __global__ void __launch_bounds__(kDirectThreads)
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
+__global__ void ion_clear_kernel(uint32_t* hdr) {
+  if (threadIdx.x < kHdrWords) hdr[threadIdx.x] = 0;
+}
+
 // One instantiation of the streaming kernel: its function and smem needs.
 struct StreamVariant {
   const void* fn;
@@ -1454,6 +1462,26 @@ cudaError_t resident_blocks(const StreamVariant& v, int njobs, size_t smem, int*
 
 }  // namespace
 
+// A call on a small patch waits for its host side, where a memset is 1.5 us
+// cheaper than a launch and an attribute (16,384 cells by step(): 10.7 against 12.3 us); in a
+// captured graph, and on more cells, the device waits for the memset and the launch
+// after it (200 captured FP64 steps of 128x128 cells: 3717 us with memsets, 3030 so).
+constexpr int64_t kHostBoundCells = 100000;
+
+cudaError_t launch_clear(uint32_t* hdr, int64_t cells, bool* dependent, cudaStream_t s) {
+  static_assert(kHdrWords <= 32, "one warp");
+  *dependent = true;
+  if (cells <= kHostBoundCells) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    if (e != cudaSuccess) return e;
+    *dependent = st != cudaStreamCaptureStatusNone;
+  }
+  if (!*dependent) return cudaMemsetAsync(hdr, 0, kHdrWords * sizeof(uint32_t), s);
+  ion_clear_kernel<<<1, 32, 0, s>>>(hdr);
+  return cudaGetLastError();
+}
+
 LaunchShape default_shape() { return {2, 8, 0, true}; }
 
 bool valid_shape(const LaunchShape& s) {
@@ -1493,19 +1521,20 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
                    lean_fits(a, shape.cells_per_lane),
                    (a.pol.flags & ION_CONSERVATION_CHECK) != 0);
   if (!v) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(a.ws.hdr, 0, kHdrWords * sizeof(uint32_t), s);
-  if (e != cudaSuccess) return e;
   const int chunk = 32 * v->Q;
   int total = 0, cells = 0;
   for (int j = 0; j < a.njobs; ++j) {
     a.job[j].chunk0 = cells;
     cells += a.job[j].ncells;
   }
+  bool dependent = false;
+  cudaError_t e = launch_clear(a.ws.hdr, cells, &dependent, s);
+  if (e != cudaSuccess) return e;
   if (cells == 0) return cudaSuccess;
   if (shape.direct && cells <= kDirectCells) {
     a.nchunks = cells;
-    ion_direct_kernel<<<(cells + kDirectThreads - 1) / kDirectThreads, kDirectThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(dependent, ion_direct_kernel, (cells + kDirectThreads - 1) / kDirectThreads,
+                        kDirectThreads, 0, s, a);
   }
   cells = 0;
   for (int j = 0; j < a.njobs; ++j) {
@@ -1523,8 +1552,9 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
   const int64_t need = ((int64_t)total + v->W - 1) / v->W;
   int blocks = (int)(need < (int64_t)per_sm * num_sms ? need : (int64_t)per_sm * num_sms);
   if (blocks < 1) blocks = 1;  // the tails still need a warp
-  void* args[] = {&a};
-  if ((e = cudaLaunchKernel(v->fn, blocks, v->W * 32, args, smem, s)) != cudaSuccess) return e;
+  if ((e = launch_after(dependent, reinterpret_cast<void (*)(BatchArgs)>(const_cast<void*>(v->fn)),
+                        blocks, v->W * 32, smem, s, a)) != cudaSuccess)
+    return e;
   if ((e = launch_stiff_f32(a, num_sms, s)) != cudaSuccess) return e;
   return launch_fb_f32(a, num_sms, s);
 }
@@ -1549,26 +1579,10 @@ cudaError_t launch_net_select_f32(BatchArgs& a, const NetSelect& sel, int num_sm
   return cudaLaunchKernel(v->fn, blocks, v->W * 32, args, smem, s);
 }
 
-// Launches a kernel that follows another of the same call (programmatic dependent launch):
-// its blocks are set up and stage their tables while the last blocks of the one before
-// finish, and wait there (cudaGridDependencySynchronize) until all of it is done and its
-// stores are seen.  The streaming kernels give no early trigger: record blocks
-// that come up beside them run under their shared-memory carveout, with next to no L1
-// (20 Kr-like steps 5 % slower).  One step, us: 33.5M nitrogen cells 318 -> 313, 4M
-// Kr-like adaptive 177 -> 173, 1M Ar-like field 80 -> 74, 30M mixed 987 -> 977.
-cudaError_t launch_after(void (*kernel)(BatchArgs), int blocks, int threads, const BatchArgs& a,
-                         cudaStream_t s) {
-  cudaLaunchAttribute at = {};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.stream = s;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
-}
+// The record and queue kernels follow the streaming kernel as its dependents, which gives no
+// early trigger: record blocks that come up beside it run under its shared-memory carveout,
+// with next to no L1 (20 Kr-like steps 5 % slower).  One step, us: 33.5M nitrogen cells 318 ->
+// 313, 4M Kr-like adaptive 177 -> 173, 1M Ar-like field 80 -> 74, 30M mixed 987 -> 977.
 
 // The record kernel's grid is one wave of resident blocks: a second, partial
 // wave would start its share of the records only after the first finished.
@@ -1590,14 +1604,14 @@ cudaError_t launch_stiff_f32(const BatchArgs& a, int num_sms, cudaStream_t s) {
       if (cache) g_stiff_fit[dev] = fit;
     }
   }
-  return launch_after(ion_stiff_kernel, fit * num_sms, 256, a, s);
+  return launch_after(true, ion_stiff_kernel, fit * num_sms, 256, 0, s, a);
 }
 
 cudaError_t launch_fb_f32(const BatchArgs& a, int num_sms, cudaStream_t s) {
   const bool need_fb = (a.pol.flags & ION_NO_FP64_FALLBACK) == 0 &&
                        ((a.pol.flags & ION_FORCE_FP64_COEF) != 0 || a.pol.gap > 0.0);
   if (!need_fb) return cudaSuccess;
-  return launch_after(ion_fb_kernel, 2 * num_sms, 128, a, s);
+  return launch_after(true, ion_fb_kernel, 2 * num_sms, 128, 0, s, a);
 }
 
 }  // namespace ion

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   if (lane < kClasses) sm.count[wib][lane] = 0;
   __syncthreads();
+  cudaGridDependencySynchronize();  // the header is zero
   uint32_t(*queue)[kQueueCap] = sm.queue[wib];
   int* count = sm.count[wib];
   const unsigned below = (1u << lane) - 1u;
@@ -238,10 +239,10 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // One cell per lane, for grids of at most kDirectGroups warps per SM: the
 // queues cost a batch per class and block at the end, and save nothing until
-// they fill.  Direct against queued, us, nitrogen (Kr-like) cells: 16,384 28 against 38
+// until they fill.  Direct against queued, us, nitrogen (Kr-like) cells: 16,384 28 against 38
 // (40, 110); 120,000 53 against 52 (123, 190); 160,000 67 against 54 (143, 198);
 // 320,000 109 against 58 (260, 235): the line lies between the two gases'
-// crossings.  Bound by latency: an FP64 instruction holds its scheduler 64
+// crossings (with log2 and exp2 still on the FP64 pipe).  Bound by latency: an FP64 instruction holds its scheduler 64
 // cycles whatever its lanes, and a warp with Taylor and Bateman lanes runs
 // both, some 400 of them.  A warp runs its lanes' widths one after another (cells
 // side by side mostly share theirs); a cell whose FP32 estimate is far below
@@ -262,6 +263,7 @@ __global__ void __launch_bounds__(kDirectThreads)
   stage_f64(J.tab, pol.log2dt, &tab);
   stage_f32(J.tab, pol.log2dt, &tab32);
   __syncthreads();
+  cudaGridDependencySynchronize();  // the header is zero
   const bool ok = window_ok(lo, hi, J.Z);
   if (on && !ok) atomicAdd(&hdr[kHdrInvalid], 1u);
   int w = on && ok ? hi - lo + 1 : 0;
@@ -286,7 +288,8 @@ int g_fit[kMaxDevices] = {};  // resident blocks per SM, per device (0: not yet)
 }  // namespace
 
 cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr, bool first,
-                            cudaStream_t s) {
+                            bool dependent, cudaStream_t s) {
+  dependent = dependent && first;
   if (job.ncells == 0) return cudaSuccess;
   int dev = 0, fit = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -295,9 +298,9 @@ cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr, 
     return e;
   const int64_t groups = ((int64_t)job.ncells + 31) / 32;
   if (groups <= (int64_t)kDirectGroups * sms) {
-    ion_step_f64_direct<<<(job.ncells + kDirectThreads - 1) / kDirectThreads, kDirectThreads, 0,
-                          s>>>(job, pol, hdr);
-    return cudaGetLastError();
+    const unsigned blocks = (job.ncells + kDirectThreads - 1) / kDirectThreads;
+    return launch_after(dependent, ion_step_f64_direct, blocks, kDirectThreads, 0, s, job, pol,
+                        hdr);
   }
   {
     std::lock_guard<std::mutex> lock(g_mu);
@@ -319,8 +322,7 @@ cudaError_t launch_step_f64(const JobIO& job, const Policy& pol, uint32_t* hdr, 
   const int64_t need = (groups + kWarps - 1) / kWarps;
   const int64_t cap = (int64_t)fit * sms;
   const int blocks = (int)(need < cap ? need : cap);
-  ion_step_f64_kernel<<<blocks, kThreads, 0, s>>>(job, pol, hdr);
-  return cudaGetLastError();
+  return launch_after(dependent, ion_step_f64_kernel, blocks, kThreads, 0, s, job, pol, hdr);
 }
 
 }  // namespace ion
