@@ -253,10 +253,10 @@ __global__ void rates_f64_kernel(const ion::SpeciesTable* t, const double* E,
 // evaluates log2|E| and 1/|E| once into shared memory, then the threads walk
 // the block's rows in the order of the output, each staying on one state (so
 // that its a, b, C sit in registers and a warp's stores are contiguous).  The
-// bound is the FP64 pipe: 12 instructions per field and 2 per rate, every
+// bound is the FP64 pipe: one instruction per field and 2 per rate (67 us below), every
 // comparison and clamp an integer one.  1,048,576 fields of an 18-state
-// ladder: 292 us as one thread per cell with rows stored K doubles apart,
-// 88 us here (output alone at the HBM rate: 23 us).
+// ladder: 292 us as one thread per cell with rows stored K doubles apart, 88 us
+// with 12 FP64 instructions per field, 72 us here (output alone at the HBM rate: 23 us).
 constexpr int kTargetCells = 256;
 
 __global__ void __launch_bounds__(kTargetCells)

@@ -239,12 +239,13 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // One cell per lane, for grids of at most kDirectGroups warps per SM: the
 // queues cost a batch per class and block at the end, and save nothing until
-// until they fill.  Direct against queued, us, nitrogen (Kr-like) cells: 16,384 28 against 38
-// (40, 110); 120,000 53 against 52 (123, 190); 160,000 67 against 54 (143, 198);
-// 320,000 109 against 58 (260, 235): the line lies between the two gases'
-// crossings (with log2 and exp2 still on the FP64 pipe).  Bound by latency: an FP64 instruction holds its scheduler 64
-// cycles whatever its lanes, and a warp with Taylor and Bateman lanes runs
-// both, some 400 of them.  A warp runs its lanes' widths one after another (cells
+// they fill.  Direct against queued, us a step in a graph, nitrogen (Kr-like) cells: 16,384
+// 21.6 against 34.2 (33.5, 93.3); 80,000 32.4 against 36.5 (68.6, 141); 120,000 35.9 against
+// 36.8 (97.8, 161); 160,000 44.7 against 39.0 (115, 183); 320,000 71.7 against 48.8 (209,
+// 235): the line lies between the two gases' crossings, where what the one loses is small
+// against what the other gains.  Bound by latency: an FP64 instruction holds its scheduler
+// 64 cycles whatever its lanes, and a warp with Taylor and Bateman lanes runs
+// both.  A warp runs its lanes' widths one after another (cells
 // side by side mostly share theirs); a cell whose FP32 estimate is far below
 // the first term's threshold keeps its populations.
 constexpr int kDirectThreads = 64;
