@@ -233,10 +233,15 @@ __device__ __forceinline__ double div_f64(double a, double b) {
   return a * __hiloint2double(hi_word(r) ^ (hi_word(b) & (int)0x80000000), lo_word(r));
 }
 
-// 2^y in 64-bit integers; y is clamped to [-1200, 1000] (-1200: 0 after rounding).
+// The upper words of 1000 and of 100, the largest exponents of exp2_f64.
+constexpr uint32_t kTop1000 = 0x408f4000u, kTopStep = 0x40590000u;
+
+// 2^y in 64-bit integers; y is clamped to [-1200, 1000] (-1200: 0 after rounding), or to the
+// number whose upper word is Top.
 // With y in units of 2^-53, y = n + i/256 + rho/256 + ..: n the exponent, i the
 // table entry T = 2^(i/256), rho in [0, 1) the rest; 2^y = 2^n (T + T p), p =
 // 2^(rho/256) - 1 = rho/256 q(rho), q a cubic in units of 2^-52.
+template <uint32_t Top = kTop1000>
 __device__ __forceinline__ double exp2_f64(double y) {
   uint32_t h = (uint32_t)hi_word(y), l = (uint32_t)lo_word(y);
   const bool tiny = h >= 0xc08ff000u;  // y <= -1022: below the normal range
@@ -245,8 +250,8 @@ __device__ __forceinline__ double exp2_f64(double y) {
     h = (uint32_t)hi_word(y);
     l = (uint32_t)lo_word(y);
   }
-  if ((int)h >= 0x408f4000) {  // 2^1000 at most
-    h = 0x408f4000u;
+  if ((int)h >= (int)Top) {
+    h = Top;
     l = 0;
   }
   // |y| in units of 2^-53, rounded where it has bits below

@@ -266,10 +266,15 @@ __device__ __forceinline__ bool past_cutoff(double rE, double rmax) {
   return __double_as_longlong(rE) > __double_as_longlong(rmax);
 }
 
-// W_k dt in FP64.
+// W_k dt in FP64, at most 2^1000, or at most 2^100 in a step (kTopStep): e^{-W dt} is long 0
+// there, and a rate that keeps anything (below 2^10) is nothing beside it, so that the step's
+// results are those of any larger rate.  The divided differences' keys then tell nodes apart
+// (floats end at 2^128), a series over nodes of equal keys (2^77 apart at most) stays
+// below 2^960, and so does a product of a window's rates.
+template <uint32_t Top = kTop1000>
 __device__ __forceinline__ double rate_dt_f64(const StagedF64& t, int k, const FieldF64& f) {
   if (f.zero || past_cutoff(f.rE, t.rmax[k])) return 0.0;
-  return exp2_f64(exponent_f64(t.a[k], t.b[k], t.C[k], f));
+  return exp2_f64<Top>(exponent_f64(t.a[k], t.b[k], t.C[k], f));
 }
 
 __device__ __forceinline__ double rate_dt_f64(const StagedF64& t, int k, double E_in) {
@@ -446,8 +451,8 @@ struct DDParams<double> {
   __device__ static __forceinline__ double expn(double z) { return exp_f64(z); }
   // the leading 24 bits choose: a form taken at a spread 2^-23 of the node's
   // size off its threshold is as accurate, and where that is large (a node
-  // below -2^20) every value is 0; equal nodes have equal keys, so that no
-  // difference divides by 0
+  // below -2^20) every value is 0 (times a series that kTopStep keeps finite);
+  // equal nodes have equal keys, so that no difference divides by 0
   __device__ static __forceinline__ float key(double z) { return f32_of_f64(z); }
 };
 

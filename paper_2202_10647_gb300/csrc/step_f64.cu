@@ -66,7 +66,7 @@ __device__ __forceinline__ double f64_cell(const JobIO& J, const Policy& pol,
   float lmax = 0.0f;
 #pragma unroll
   for (int r = 0; r < W - 1; ++r) {
-    lam[r] = pol.zero_dt ? 0.0 : rate_dt_f64(tab, lo + r, f);
+    lam[r] = pol.zero_dt ? 0.0 : rate_dt_f64<kTopStep>(tab, lo + r, f);
     lmax = fmaxf(lmax, f32_of_f64(lam[r]));
   }
   lam[W - 1] = 0.0;
