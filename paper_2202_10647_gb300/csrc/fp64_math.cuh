@@ -8,14 +8,15 @@
 // by the leading bits, and a short polynomial in what is left.  Exponents,
 // table indices, comparisons and conversions are integer and FP32 work.
 //   log2_f64   1 FP64 instruction
-//   rcp_f64, exp2_f64   none
+//   rcp_f64, exp2_f64, exp_f64   none
 // against some 25, 10 and 15 of log2(), a division and exp2(), and 9, 3 and 8 of the same
 // method with the polynomials in FP64: everything else is 64-bit fixed point, 20 to 60
 // integer instructions each, whose issue time is that of one FP64 instruction at most.  A
 // rate of Eq. 1 keeps the two fused multiply-adds of its exponent.  FP64 step, 33.5M nitrogen
 // cells: 2,347 us with the polynomials in FP64, 1,922 so.
 // Errors (measured over 2^-20..2^60 and -1000..1000, against 113-bit arithmetic): log2
-// 0.57 ulp of max(|log2 E|, 1), 1/E 0.56 ulp, exp2 0.96 ulp.
+// 0.57 ulp of max(|log2 E|, 1), 1/E 0.56 ulp, exp2 0.96 ulp, e^z 0.98 ulp down to z = -256 (1.2
+// to -512, 1.9 below).
 // The tables are nearest values of 40-digit ones; the polynomials
 // interpolate at Chebyshev nodes.
 #pragma once
@@ -33,6 +34,7 @@ constexpr uint32_t kLog4 = 0xb8aa3580u, kLog5 = 0x24ed7a7u, kLog6 = 0x78ab1u;
 // 2^-56.6 of 1)
 constexpr uint64_t kExp1 = 0xb17217f7d1cedull, kExp2 = 0x3d7f7bff1b7ull;
 constexpr uint32_t kExp3 = 0xe3583fe3u, kExp4 = 0x277045u;
+constexpr uint64_t kLog2E = 0xb8aa3b295c17f0bcull;  // log2 e in units of 2^-63
 
 // Interval j of the mantissa, [1 + j/128, 1 + (j+1)/128): c, the reciprocal of its lower end
 // rounded up, in units of 2^-31, and -log2 c in units of 2^-57.
@@ -233,14 +235,31 @@ __device__ __forceinline__ double div_f64(double a, double b) {
   return a * __hiloint2double(hi_word(r) ^ (hi_word(b) & (int)0x80000000), lo_word(r));
 }
 
+// 2^(Y 2^-53) in 64-bit integers, Y two's complement.  Y = n + i/256 + rho/256 (in those
+// units): n the exponent, i the table entry T = 2^(i/256), rho in [0, 1) the rest; the result is
+// 2^n (T + T p), p = 2^(rho/256) - 1 = rho/256 q(rho), q a cubic in units of 2^-52.
+// `tiny`: of an exponent 256 larger, scaled back with one rounding (below the normal range).
+__device__ __forceinline__ double exp2_fixed(uint64_t Y, bool tiny) {
+  const int yh = (int)(Y >> 32);
+  const uint64_t T = kExpTab[(yh >> 13) & 255];
+  const uint64_t rho = Y << 19;
+  const uint32_t rh = (uint32_t)(rho >> 32), rl = (uint32_t)rho;
+  const uint64_t B = kExp2 + __umulhi(kExp3 + __umulhi(kExp4, rh), rh);
+  const uint64_t q = kExp1 + mul_hi_short<10>(B, rh, rl);
+  const uint64_t p = mul_hi64(rho, q);              // units of 2^-60
+  const uint64_t S = T + (mul_hi64(T, p) << 4);     // units of 2^-62
+  // rounded to 53 bits, whose leading one adds 1 to the exponent field
+  const uint64_t M = (S + 512u) >> 10;
+  const double v = __hiloint2double((int)((uint32_t)(M >> 32) + (uint32_t)(((yh >> 21) + 1022) << 20)),
+                                    (int)(uint32_t)M);
+  return tiny ? v * 0x1p-256 : v;
+}
+
 // The upper words of 1000 and of 100, the largest exponents of exp2_f64.
 constexpr uint32_t kTop1000 = 0x408f4000u, kTopStep = 0x40590000u;
 
-// 2^y in 64-bit integers; y is clamped to [-1200, 1000] (-1200: 0 after rounding), or to the
-// number whose upper word is Top.
-// With y in units of 2^-53, y = n + i/256 + rho/256 + ..: n the exponent, i the
-// table entry T = 2^(i/256), rho in [0, 1) the rest; 2^y = 2^n (T + T p), p =
-// 2^(rho/256) - 1 = rho/256 q(rho), q a cubic in units of 2^-52.
+// 2^y; y is clamped to [-1200, 1000] (-1200: 0 after rounding), or to the number whose
+// upper word is Top.
 template <uint32_t Top = kTop1000>
 __device__ __forceinline__ double exp2_f64(double y) {
   uint32_t h = (uint32_t)hi_word(y), l = (uint32_t)lo_word(y);
@@ -258,24 +277,20 @@ __device__ __forceinline__ double exp2_f64(double y) {
   const uint32_t s = 1032u - ((h >> 20) & 0x7ffu);
   uint64_t m = ((uint64_t)((h & 0xfffffu) | 0x100000u) << 32 | l) << 11;
   m = s < 64u ? ((m >> s) + 1u) >> 1 : 0u;
-  const uint64_t Y = (int)h < 0 ? 0u - m : m;
-  const int yh = (int)(Y >> 32);
-  const uint64_t T = kExpTab[(yh >> 13) & 255];
-  const uint64_t rho = Y << 19;
-  const uint32_t rh = (uint32_t)(rho >> 32), rl = (uint32_t)rho;
-  const uint64_t B = kExp2 + __umulhi(kExp3 + __umulhi(kExp4, rh), rh);
-  const uint64_t q = kExp1 + mul_hi_short<10>(B, rh, rl);
-  const uint64_t p = mul_hi64(rho, q);              // units of 2^-60
-  const uint64_t S = T + (mul_hi64(T, p) << 4);     // units of 2^-62
-  // rounded to 53 bits, whose leading one adds 1 to the exponent field
-  const uint64_t M = (S + 512u) >> 10;
-  const double v = __hiloint2double((int)((uint32_t)(M >> 32) + (uint32_t)(((yh >> 21) + 1022) << 20)),
-                                    (int)(uint32_t)M);
-  return tiny ? v * 0x1p-256 : v;  // back with one rounding
+  return exp2_fixed((int)h < 0 ? 0u - m : m, tiny);
 }
 
-// e^z for z <= 0: the product with log2 e rounds once, |z| 2^-53 relative to
-// e^z, at most 0.37 2^-53 absolute.
-__device__ __forceinline__ double exp_f64(double z) { return exp2_f64(z * 0x1.71547652b82fep+0); }
+// e^z for z <= 0: |z| log2 e as a 64-bit product in units of 2^-53 (a product in FP64 would
+// round it by |z| 2^-53 of the result, and cost the FP64 pipe an instruction).
+__device__ __forceinline__ double exp_f64(double z) {
+  const uint32_t h = min((uint32_t)hi_word(z) & 0x7fffffffu, 0x40875000u);  // 0 from -746 on
+  const uint64_t m = ((uint64_t)((h & 0xfffffu) | 0x100000u) << 32 | (uint32_t)lo_word(z)) << 11;
+  uint64_t P = mul_hi64(m, kLog2E);
+  const uint32_t s = 1032u - (h >> 20);  // P is in units of 2^(-53 - s)
+  if (s) P = s < 65u ? ((P >> (s - 1u)) + 1u) >> 1 : 0u;
+  const bool tiny = P >= 1022ull << 53;
+  if (tiny) P -= 256ull << 53;
+  return exp2_fixed(0u - P, tiny);
+}
 
 }  // namespace ion
