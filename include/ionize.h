@@ -511,9 +511,10 @@ ION_API int ion_surrogate_rates(const ion_surrogate* s, const float* E, int64_t 
  * (a perturbation of the rate matrix by dA moves the solution of Eq. 3 by
  * at most |dA| in the 1-norm); if it is below pop_tol the network's rates
  * are used, otherwise (and outside the range) the rates of Eq. 1; pop_tol 0
- * never uses the network.  (Where the arrays allow the streaming kernel, a
- * cell whose rates of Eq. 1, lowered by twice their validation bound, already
- * exceed pop_tol takes Eq. 1 without asking the network.)  A cell
+ * never uses the network.  (In a call of more than 320,000 cells whose
+ * arrays allow the streaming kernel, a cell whose rates of Eq. 1, lowered by
+ * twice their validation bound, already exceed pop_tol takes Eq. 1 without
+ * asking the network.)  A cell
  * with some rate W dt > 1 always takes the rates of Eq. 1 (its bound would
  * exceed any useful tolerance) and is finished in the Bateman form by
  * ion_step's record kernel.  The update itself is ion_step's (Taylor or

@@ -836,6 +836,15 @@ cudaError_t launch(const ion_surrogate* s, bool step, const StepArgs& a, cudaStr
   return cudaLaunchKernel(fn, blocks, ion::sg::kCta, args, ion::sg::plan_of(s->KP).total, st);
 }
 
+// Steps of at most this many cells take the network kernel over all of them: on a few
+// tens of thousands the streaming kernel in front of it is mostly the filling of its own ring.
+// List against all cells, us a step in a graph with the copy of its windows, nitrogen (Ar-like,
+// Kr-like) cells: 20,000 38 against 23 (45, 25; 46, 27); 160,000 47 against 38 (57, 43; 54, 45);
+// 250,000 49 against 46 (61, 51; 61, 55); 300,000 51 against 51 (62, 58; 62, 62); 350,000 51
+// against 54 (65, 60; 63, 70); 450,000 54 against 64 (70, 74; 68, 82); 1,000,000 65 against 114
+// (99, 129; 94, 152).  The line lies between the gases' crossings.
+constexpr int64_t kListCells = 320000;
+
 int check_surrogate(const ion_surrogate* s) {
   if (!s || !s->dev) return ion::set_error(ION_EINVAL, "surrogate is NULL or destroyed");
   int d = -1;
@@ -1182,10 +1191,10 @@ int ion_step_surrogate(const ion_surrogate* s, const float* E, float* N, int64_t
   // With validation bounds, the cells the network could not serve are
   // stepped by the streaming kernel, and the network kernel takes the others from a
   // list (in the FP64 queue's place, which the record kernel fills after it).
-  // Otherwise, or for arrays and policies the streaming kernel does not
-  // take, the network kernel walks all cells.
-  if (e == cudaSuccess && ncells > 0 && s->bound && !a.pol.adaptive && !a.pol.zero_dt &&
-      a.pop_tol > 0.0f) {
+  // Otherwise, on small grids, or for arrays and policies the streaming kernel does
+  // not take, the network kernel walks all cells.
+  if (e == cudaSuccess && ncells > kListCells && s->bound && !a.pol.adaptive &&
+      !a.pol.zero_dt && a.pop_tol > 0.0f) {
     const uintptr_t al = reinterpret_cast<uintptr_t>(E) | reinterpret_cast<uintptr_t>(N) |
                          reinterpret_cast<uintptr_t>(dne);
     b.job[0].vec = (al & 7u) == 0 && ld % 2 == 0;
