@@ -202,10 +202,11 @@ __device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
       : "memory");
 }
 
-// Named barriers of a CTA (0 is __syncthreads): the network warps among
-// themselves; Y written (network warps arrive, cell warps wait); Y read (the
-// other way round).
-constexpr int kBarNet = 1, kBarYFull = 2, kBarYFree = 3;
+// Named barriers of a CTA (0 is __syncthreads, which the two groups, on different
+// branches, may not meet at): the network warps among themselves; Y written
+// (network warps arrive, cell warps wait); Y read (the other way round); a
+// tile's cells looked at by both.
+constexpr int kBarNet = 1, kBarYFull = 2, kBarYFree = 3, kBarTile = 4;
 template <int Id, int N>
 __device__ __forceinline__ void bar_sync() {
   asm volatile("bar.sync %0, %1;" ::"n"(Id), "n"(N) : "memory");
@@ -213,6 +214,22 @@ __device__ __forceinline__ void bar_sync() {
 template <int Id, int N>
 __device__ __forceinline__ void bar_arrive() {
   asm volatile("bar.arrive %0, %1;" ::"n"(Id), "n"(N) : "memory");
+}
+// bar_sync, and whether some thread's p is true.
+template <int Id, int N>
+__device__ __forceinline__ bool bar_or(bool p) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t"
+      ".reg .pred mine, any;\n\t"
+      "setp.ne.u32 mine, %1, 0;\n\t"
+      "bar.red.or.pred any, %2, %3, mine;\n\t"
+      "selp.u32 %0, 1, 0, any;\n\t"
+      "}"
+      : "=r"(any)
+      : "r"((uint32_t)p), "n"(Id), "n"(N)
+      : "memory");
+  return any != 0u;
 }
 
 // One layer's products for the 128-row tile once every network thread has stored its
@@ -482,7 +499,7 @@ __global__ void __launch_bounds__(kCta, 4) surrogate_kernel(const Dev* __restric
             const int lo = a.J.lo[c], hi = a.J.hi[c];
             mine = servable(pos, l2, window_ok(lo, hi, a.J.Z), lo, hi);
           }
-          use_net = __syncthreads_or(mine) != 0;
+          use_net = bar_or<kBarTile, kCta>(mine);
         }
       }
       if (failed) continue;
@@ -622,7 +639,7 @@ __global__ void __launch_bounds__(kCta, 4) surrogate_kernel(const Dev* __restric
         }
         if (failed) continue;
         bool use_net = true;
-        if (!a.list) use_net = __syncthreads_or(mine) != 0;
+        if (!a.list) use_net = bar_or<kBarTile, kCta>(mine);
         float lam[ION_MAX_WINDOW];
 #pragma unroll
         for (int r = 0; r < ION_MAX_WINDOW; ++r) lam[r] = 0.0f;
