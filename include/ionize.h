@@ -202,6 +202,10 @@ ION_API size_t ion_step_workspace_bytes(int64_t ncells, int flags);
  * Alignment: E, N, dne, n_gas aligned to their element size; with ION_F32
  * k_lo and k_hi 4-byte aligned (they are copied four cells at a time).
  * Calls that share a workspace must not overlap on the device.
+ * Ranges: a cell's results do not depend on the size of the call.  With
+ * ION_F32 they depend on its chunk, 64 cells from the call's first (those of
+ * a last, partial chunk take the record kernel's form): a grid stepped in
+ * ranges of whole chunks gets the bits of one call over all of it.
  * Errors: ION_EINVAL (checked before any launch), ION_ECUDA. */
 ION_API int ion_step(const ion_species* sp, const void* E, void* N, int64_t ld,
              int64_t ncells, double dt_fs, uint8_t* k_lo, uint8_t* k_hi,
@@ -251,7 +255,8 @@ typedef struct {
 /* Launch shape of the FP32 streaming kernels: cells per lane (1, 2 or 4),
  * warps per block (2, 4 or 8), resident blocks per SM (0: as many as fit).
  * NULL selects {2, 8, 0}, which ion_step uses too; without a shape a call of
- * at most 400,000 cells runs one cell per lane in a single kernel instead. */
+ * at most 400,000 cells runs one cell per lane in a single kernel instead,
+ * with the same results. */
 typedef struct {
   int cells_per_lane;
   int warps_per_block;

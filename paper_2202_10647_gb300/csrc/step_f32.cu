@@ -1274,34 +1274,128 @@ __global__ void __launch_bounds__(128) ion_fb_kernel(const __grid_constant__ Bat
 // coefficients of a nearly degenerate cell taken in place: one launch, no
 // records and no queue.  On a grid of a few warps per SM the streaming kernel's
 // ring is mostly its own filling, and the two launches behind it find next to
-// nothing.  Steps of n nitrogen (Kr-like) cells in a graph, direct against
-// streaming, us: 16,384 4.3 against 15.5 (6.7, 24.6); 160,000 8.8 against 18.3 (15.5, 29.3);
-// 320,000 14.6 against 19.9 (27.4, 34.9); 400,000 17.1 against 20.2 (33.0, 35.9).  The line
-// is close to the heavier gas's crossing (before the launches of a call overlapped, 500,000
-// cells 25 against 31 and 45 against 42).
+// nothing.  A block is one chunk of the streaming kernels (64 cells of one job)
+// and shares what their warp shares, the width bound and the number of terms, so that
+// every cell gets their bits: a caller may split a grid into ranges of whole chunks.
+// Steps of n nitrogen (Ar-like, Kr-like) cells in a graph, direct against streaming, us:
+// 16,384 4.7 against 19.3 (6.0, 24.0; 6.3, 24.5); 160,000 8.9 against 23.2 (13.3, 29.1; 15.3,
+// 30.2); 320,000 13.8 against 26.2 (22.1, 32.2; 27.0, 36.2); 400,000 16.4 against 26.9 (26.7,
+// 33.9; 32.3, 37.5): the line is where the heavier gas gains little more.  Without the chunk's
+// common terms and bound (other bits): 4.3, 9.7, 15.8, 18.6 us of nitrogen.  Eight blocks per
+// SM (128 registers; 168 and six when left to itself): 400,000 Kr-like cells 36.6 -> 32.5 us.
 // ---------------------------------------------------------------------------
 constexpr int kDirectThreads = 64;
 constexpr int kDirectCells = 400000;
 
-// One cell of at most W states; `stiff`: some rate has W dt > 1, `fb`: FP64
-// coefficients.  Returns |change of sum_k N_k| (ION_CONSERVATION_CHECK).
-template <int W>
-__device__ __forceinline__ float direct_cell(const JobIO& J, const Policy& pol,
-                                             const StagedF32& tab, int c, float Ec, int lo, int hi,
-                                             bool& stiff, bool& fb) {
-  const int w = hi - lo + 1;
-  const float* p = static_cast<const float*>(J.N) + (int64_t)lo * J.ld + c;
-  float v[W], lam[W], lmax = 0.0f;
+// The chunk's cells whose rates all have W dt <= 1 (easy_cells, one cell per
+// lane; a cold chunk's series has no term and leaves v as it is); stiff marks
+// the others, left untouched.  v6 holds zeros past w; lam becomes the window's rates.
+// Every thread of the block calls this; red: the two warps' maxima; thr_lane: kThrF32[lane].
+template <int WM>
+__device__ __forceinline__ void direct_easy(const JobIO& J, const Policy& pol,
+                                            const StagedF32& tab, unsigned* red, int c, float Ec,
+                                            int lo, int hi, int w, float (&v6)[ION_MAX_WINDOW],
+                                            float (&lam)[WM], bool& stiff, uint32_t& change,
+                                            float thr_lane) {
+  const int lane = threadIdx.x & 31;
+  float v[WM], lmax = 0.0f;
+  const FieldF32 f = field_f32(Ec);
+  const bool live = w >= 2 && !f.zero && !pol.zero_dt;
+  const int base = w > 0 ? lo : 0;
 #pragma unroll
-  for (int r = 0; r < W; ++r) {
-    v[r] = r < w ? p[(int64_t)r * J.ld] : 0.0f;
+  for (int r = 0; r < WM; ++r) {
+    v[r] = v6[r];
     lam[r] = 0.0f;
   }
+#pragma unroll
+  for (int r = 0; r < WM - 1; ++r) {
+    const float4 h = tab.hi[base + r];
+    const float y = fmaf(-h.z, f.rE, fmaf(-h.y, f.lg, h.x));
+    lam[r] = live && r < w - 1 ? ex2_approx(fminf(y, 99.0f)) : 0.0f;
+  }
+#pragma unroll
+  for (int r = 0; r < WM - 1; ++r) {
+    if (lam[r] > kLamPrecise) lam[r] = rate_ff_f32(tab, base + r, f);
+    lmax = fmaxf(lmax, lam[r]);
+  }
+  stiff = lmax > lam_easy<2>();
+  const unsigned xl = __reduce_max_sync(kFull, __float_as_uint(stiff ? 0.0f : 2.0f * lmax));
+  if (lane == 0) red[threadIdx.x >> 5] = xl;
+  __syncthreads();
+  const float xw = __uint_as_float(max(red[0], red[1]));
+  const int R = __popc(__ballot_sync(kFull, xw > thr_lane));
+  float u[WM - 1], inc[WM - 1];
+#pragma unroll
+  for (int i = 0; i < WM - 1; ++i) {
+    u[i] = v[i];
+    inc[i] = 0.0f;
+  }
+#pragma unroll 1
+  for (int k = 1; k <= R; ++k) {
+    const float ck = kInvFactF32[k];
+#pragma unroll
+    for (int i = WM - 2; i >= 0; --i) {
+      u[i] = fmaf(-lam[i], u[i], i > 0 ? lam[i - 1] * u[i - 1] : 0.0f);
+      inc[i] = fmaf(u[i], ck, inc[i]);
+    }
+  }
+  if (w == 0 || stiff) return;
+  float dne = 0.0f;
+  int nlo = lo, nhi = hi;
+  if (w >= 2) {
+    float cum = 0.0f;
+#pragma unroll
+    for (int r = 0; r < WM - 1; ++r) {
+      cum -= inc[r];  // population that left states <= r
+      if (r < w - 1) dne += cum;
+      v[r] += inc[r];
+    }
+    v[WM - 1] += cum;
+    if (pol.flags & ION_CONSERVATION_CHECK) {
+      ExactSum<float> acc;
+#pragma unroll
+      for (int r = 0; r < WM; ++r) {
+        if (r < w) {
+          acc.add(-v6[r]);
+          acc.add(v[r]);
+        }
+      }
+      change = abs_bits(acc.value());
+    }
+    window_after_step<float, WM>(J, pol, v, w, nlo, nhi);
+    float* p = static_cast<float*>(J.N) + (int64_t)lo * J.ld + c;
+#pragma unroll
+    for (int r = 0; r < WM; ++r) {
+      if (r < w) __stcs(p, v[r]);
+      p += J.ld;
+    }
+  }
+  const float* __restrict__ G = static_cast<const float*>(J.n_gas);
+  __stcs(static_cast<float*>(J.dne) + c, G ? dne * G[c] : dne);
+  if (nlo != lo || nhi != hi) {
+    J.lo[c] = (uint8_t)nlo;
+    J.hi[c] = (uint8_t)nhi;
+  }
+}
+
+// What the record kernel and the FP64-coefficient pass do with a cell of at most W
+// states.  lam: rates by direct_easy, of which those above kLamPrecise are rate_dt_f32's
+// too, or zeros.  `stiff`: some rate has W dt > 1, `fb`: FP64 coefficients.  Returns
+// |change of sum_k N_k| (ION_CONSERVATION_CHECK).
+template <int W>
+__device__ __forceinline__ float direct_record(const JobIO& J, const Policy& pol,
+                                               const StagedF32& tab, int c, float Ec, int lo,
+                                               int hi, const float (&v6)[ION_MAX_WINDOW],
+                                               float (&lam)[W], bool& stiff, bool& fb) {
+  const int w = hi - lo + 1;
+  float v[W], lmax = 0.0f;
+#pragma unroll
+  for (int r = 0; r < W; ++r) v[r] = v6[r];
   if (!pol.zero_dt) {
     const FieldF32 f = field_f32(Ec);
 #pragma unroll
     for (int r = 0; r < W - 1; ++r) {
-      if (r < w - 1) lam[r] = rate_dt_f32(tab, lo + r, f);
+      if (r < w - 1 && !(lam[r] > kLamPrecise)) lam[r] = rate_dt_f32(tab, lo + r, f);
       lmax = fmaxf(lmax, lam[r]);
     }
   }
@@ -1313,41 +1407,65 @@ __device__ __forceinline__ float direct_cell(const JobIO& J, const Policy& pol,
   return d;
 }
 
-__global__ void __launch_bounds__(kDirectThreads)
+template <int W>
+__device__ __forceinline__ void direct_chunk(const JobIO& J, const Policy& pol,
+                                             const StagedF32& tab, unsigned* red, bool tail,
+                                             int c, float Ec, int lo, int hi, int w,
+                                             float (&v)[ION_MAX_WINDOW], bool& stiff, bool& fb,
+                                             uint32_t& change, float thr_lane) {
+  bool rec = w > 0;
+  float lam[W];
+#pragma unroll
+  for (int r = 0; r < W; ++r) lam[r] = 0.0f;
+  if (!tail) {
+    direct_easy<W>(J, pol, tab, red, c, Ec, lo, hi, w, v, lam, stiff, change, thr_lane);
+    rec = stiff;
+  }
+  if (rec) change = abs_bits(direct_record<W>(J, pol, tab, c, Ec, lo, hi, v, lam, stiff, fb));
+}
+
+__global__ void __launch_bounds__(kDirectThreads, 8)
     ion_direct_kernel(const __grid_constant__ BatchArgs a) {
-  __shared__ StagedF32 tabs[kMaxJobs];
-  // the jobs' cells one after another: job j's first is chunk0
-  const int i = blockIdx.x * kDirectThreads + threadIdx.x;
-  const int jid = job_of(a, i);
+  __shared__ StagedF32 tab;
+  __shared__ unsigned red[4];
+  const int lane = threadIdx.x & 31;
+  const float thr_lane = lane < kEasyTerms ? kThrF32[lane] : __int_as_float(0x7f800000);
+  const int jid = job_of(a, blockIdx.x);
   const JobIO& J = a.job[jid];
-  const int c = i - J.chunk0;
+  const int c0 = ((int)blockIdx.x - J.chunk0) * kDirectThreads;
+  const int c = c0 + threadIdx.x;
   const bool on = c < J.ncells;
-  // the cell's inputs travel while the tables are staged
+  // the cell's inputs travel while the table is staged
   const float Ec = on ? static_cast<const float*>(J.E)[c] : 0.0f;
   const int lo = on ? J.lo[c] : 0, hi = on ? J.hi[c] : 0;
-  for (int j = 0; j < a.njobs; ++j) stage_f32(a.job[j].tab, a.pol.log2dt, &tabs[j]);
+  stage_f32(J.tab, a.pol.log2dt, &tab);
+  const bool ok = on && window_ok(lo, hi, J.Z);
+  const int w = ok ? hi - lo + 1 : 0;
+  float v[ION_MAX_WINDOW];
+  const float* p = static_cast<const float*>(J.N) + (int64_t)lo * J.ld + c;
+#pragma unroll
+  for (int r = 0; r < ION_MAX_WINDOW; ++r) v[r] = r < w ? p[(int64_t)r * J.ld] : 0.0f;
+  const int Ww = __reduce_max_sync(kFull, w);
+  if ((threadIdx.x & 31) == 0) red[2 + (threadIdx.x >> 5)] = Ww;
   __syncthreads();
   cudaGridDependencySynchronize();  // the header is zero
-  const bool ok = on && window_ok(lo, hi, J.Z);
   if (on && !ok) atomicAdd(&a.ws.hdr[kHdrInvalid], 1u);
-  const int w = ok ? hi - lo + 1 : 0;
-  const int Wm = __reduce_max_sync(kFull, w);
+  const int W = max(red[2], red[3]);
+  const bool tail = c0 + kDirectThreads > J.ncells;
   bool stiff = false, fb = false;
-  float d = 0.0f;
-  if (w >= 1) {
-    if (Wm <= 2)
-      d = direct_cell<2>(J, a.pol, tabs[jid], c, Ec, lo, hi, stiff, fb);
-    else if (Wm <= 4)
-      d = direct_cell<4>(J, a.pol, tabs[jid], c, Ec, lo, hi, stiff, fb);
-    else
-      d = direct_cell<6>(J, a.pol, tabs[jid], c, Ec, lo, hi, stiff, fb);
-  }
+  uint32_t change = 0;
+  if (W <= 2)
+    direct_chunk<2>(J, a.pol, tab, red, tail, c, Ec, lo, hi, w, v, stiff, fb, change, thr_lane);
+  else if (W <= 4)
+    direct_chunk<4>(J, a.pol, tab, red, tail, c, Ec, lo, hi, w, v, stiff, fb, change, thr_lane);
+  else
+    direct_chunk<6>(J, a.pol, tab, red, tail, c, Ec, lo, hi, w, v, stiff, fb, change, thr_lane);
   const unsigned ms = __ballot_sync(kFull, stiff), mf = __ballot_sync(kFull, fb);
   if ((threadIdx.x & 31) == 0) {
     if (ms) atomicAdd(&a.ws.hdr[kHdrStiff], (unsigned)__popc(ms));
     if (mf) atomicAdd(&a.ws.hdr[kHdrFallback], (unsigned)__popc(mf));
   }
-  if (a.pol.flags & ION_CONSERVATION_CHECK) warp_max_into(&a.ws.hdr[kHdrCons], abs_bits(d));
+  if (a.pol.flags & ION_CONSERVATION_CHECK) warp_max_into(&a.ws.hdr[kHdrCons], change);
 }
 
 // ---------------------------------------------------------------------------
@@ -1523,24 +1641,22 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
   if (!v) return cudaErrorInvalidValue;
   const int chunk = 32 * v->Q;
   int total = 0, cells = 0;
-  for (int j = 0; j < a.njobs; ++j) {
-    a.job[j].chunk0 = cells;
-    cells += a.job[j].ncells;
-  }
+  for (int j = 0; j < a.njobs; ++j) cells += a.job[j].ncells;
   bool dependent = false;
   cudaError_t e = launch_clear(a.ws.hdr, cells, &dependent, s);
   if (e != cudaSuccess) return e;
   if (cells == 0) return cudaSuccess;
   if (shape.direct && cells <= kDirectCells) {
-    a.nchunks = cells;
-    return launch_after(dependent, ion_direct_kernel, (cells + kDirectThreads - 1) / kDirectThreads,
-                        kDirectThreads, 0, s, a);
+    for (int j = 0; j < a.njobs; ++j) {
+      a.job[j].chunk0 = total;
+      total += (a.job[j].ncells + kDirectThreads - 1) / kDirectThreads;
+    }
+    a.nchunks = total;
+    return launch_after(dependent, ion_direct_kernel, total, kDirectThreads, 0, s, a);
   }
-  cells = 0;
   for (int j = 0; j < a.njobs; ++j) {
     a.job[j].chunk0 = total;
     total += a.job[j].ncells / chunk;
-    cells += a.job[j].ncells;
   }
   a.nchunks = total;
   const size_t smem = v->smem(a.njobs);
