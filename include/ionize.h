@@ -529,7 +529,8 @@ ION_API int ion_surrogate_rates(const ion_surrogate* s, const float* E, int64_t 
  * ION_F32); after the call its header holds, besides the words described
  * for ion_step, word 3: cells that took the network's rates, word 4: cells
  * that took the rates of Eq. 1, word 5: non-zero if a bounded wait for the
- * tensor cores gave up (the results of the call are then invalid).
+ * tensor cores gave up (the call has then failed: every cell was either
+ * stepped whole or left as it was, its dne included).
  * Errors: ION_EINVAL, ION_ECUDA. */
 ION_API int ion_step_surrogate(const ion_surrogate* s, const float* E, float* N, int64_t ld,
                                int64_t ncells, double dt_fs, uint8_t* k_lo, uint8_t* k_hi,
@@ -542,11 +543,13 @@ ION_API int ion_step_surrogate(const ion_surrogate* s, const float* E, float* N,
  * (ion_surrogate_rates, ion_step_surrogate) makes the first tensor-core
  * wait of each tile poll, 64 times, an mbarrier that nothing arrives at, so
  * that the wait gives up exactly as a wait that ran out of its limit would:
- * ion_step_surrogate leaves every cell it would ask the network about
- * untouched and sets word 5 of the workspace header, ion_surrogate_rates writes NaN rates, and each CTA waits
- * (bounded) for the matrix products it skipped before it frees its tensor
- * memory.  on = 0 restores the normal waits.  Synchronous (one 4-byte copy
- * to the device).  Errors: ION_EINVAL, ION_ECUDA. */
+ * ion_step_surrogate leaves every cell it would ask the network about as it
+ * was, its dne included (of a call of at most 320,000 cells those of every
+ * 128-cell tile with such a cell), and sets word 5 of the workspace header,
+ * ion_surrogate_rates writes NaN rates, and each CTA waits (bounded) for the
+ * matrix products it skipped before it frees its tensor memory.  on = 0
+ * restores the normal waits.  Synchronous (one 4-byte copy to the device).
+ * Errors: ION_EINVAL, ION_ECUDA. */
 ION_API int ion_surrogate_test_timeout(ion_surrogate* s, int on);
 
 /* ion_surrogate_validate -- the validation error bound, computed on the GPU

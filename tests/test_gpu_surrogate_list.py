@@ -82,3 +82,46 @@ def test_list_at_the_ends(short_net, pop_tol):
         assert ca == cb and ca[0] > n // 2
         for k in ("N", "lo", "hi", "dne"):
             assert np.array_equal(a[k], b[k])
+
+
+def test_list_after_a_wait_that_gives_up(short_net):
+    """The test hook on the list route: every cell and its dne are either
+    stepped whole (those the network is not asked about) or as they were;
+    the header says that the call failed, and the next calls run."""
+    sd, sp, net = short_net
+    n = LINE + 11
+    wl = W.ladder_cells(sd, n, 47, block=64)
+    E = wl.E.cuda()
+    lo2, hi2, N2 = wl.lo.cuda(), wl.hi.cuda(), wl.N.cuda()
+    dne2 = torch.empty(n, device="cuda")
+    ionize.step(sp, E, N2, lo2, hi2, 0.05, dne2)
+    net.test_timeout(True)
+    try:
+        for rep in range(2):
+            N, lo, hi = wl.N.cuda(), wl.lo.cuda(), wl.hi.cuda()
+            dne = torch.full((n,), -5.0, device="cuda")
+            ws = net.step(E, N, lo, hi, 0.05, dne)
+            torch.cuda.synchronize()
+            n_net, n_plain, timeout = ionize.surrogate_counters(ws)
+            h = ws[:44].cpu().view(torch.int32)
+            kept = (dne == -5.0).cpu()
+            assert timeout > 0 and n_net == 0
+            assert int(kept.sum()) == int(h[9]) and n // 100 < int(h[9]) < n
+            assert n_plain + int(h[9]) == n
+            assert torch.equal(N.cpu()[:, :n][:, kept], wl.N[:, :n][:, kept])
+            assert torch.equal(lo.cpu()[kept], wl.lo[kept])
+            assert torch.equal(hi.cpu()[kept], wl.hi[kept])
+            # ion_step's kernels on the others: its bits where a chunk holds no listed cell
+            whole = ~kept[:n // 64 * 64].view(-1, 64).any(1).repeat_interleave(64)
+            assert int(whole.sum()) > n // 10
+            assert float((N - N2)[:, :n].cpu()[:, ~kept].abs().max()) <= 4e-6
+            for a, b in ((N[:, :n], N2[:, :n]), (lo, lo2), (hi, hi2), (dne, dne2)):
+                assert torch.equal(a[..., :len(whole)].cpu()[..., whole],
+                                   b[..., :len(whole)].cpu()[..., whole])
+    finally:
+        net.test_timeout(False)
+    N, lo, hi = wl.N.cuda(), wl.lo.cuda(), wl.hi.cuda()
+    ws = net.step(E, N, lo, hi, 0.05, torch.empty(n, device="cuda"))
+    torch.cuda.synchronize()
+    assert ionize.surrogate_counters(ws)[2] == 0 and ionize.surrogate_counters(ws)[0] > 0
+    assert float((N - N2).abs().max()) <= 4e-6
