@@ -184,6 +184,8 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
 // kernel of the same call (step_f32.cu).
 cudaError_t launch_stiff_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_fb_f32(const BatchArgs& a, int num_sms, cudaStream_t s);
+// One-time set-up of launch_net_select_f32's kernel on the current device.
+cudaError_t prepare_net_select_f32();
 // One species' cells stepped with the rates of Eq. 1, except those the
 // network could serve, which are listed and left untouched.  The header is
 // already cleared.  *fits: whether the arrays allow it (nothing is launched

@@ -1545,8 +1545,9 @@ bool lean_fits(const BatchArgs& a, int Q) {
 }
 
 // Resident blocks per SM of a variant with `njobs` staged tables, set up and
-// measured once per (device, variant, njobs): later calls (and calls made
-// while a stream is being captured) only read the cache.
+// measured once per (device, variant, njobs); later calls only read the cache.
+// (Nothing of it is a stream operation, so that it may fall into a capture;
+// multistep.StepGraph has it done before.)
 constexpr int kMaxDevices = 64;
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 std::mutex g_fit_mu;
@@ -1673,6 +1674,12 @@ cudaError_t launch_batch_f32(BatchArgs& a, const LaunchShape& shape, int num_sms
     return e;
   if ((e = launch_stiff_f32(a, num_sms, s)) != cudaSuccess) return e;
   return launch_fb_f32(a, num_sms, s);
+}
+
+cudaError_t prepare_net_select_f32() {
+  const StreamVariant* v = find_variant(2, 8, false, true, false, true);
+  int fit = 0;
+  return v ? resident_blocks(*v, 1, v->smem(1), &fit) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_net_select_f32(BatchArgs& a, const NetSelect& sel, int num_sms, bool* fits,

@@ -1038,6 +1038,7 @@ int ion_surrogate_create(const ion_species* sp, const float* P, const ion_surrog
   }
   if (e == cudaSuccess) e = prepare(kernel_of<false>(KP), KP, &s->fit_rates);
   if (e == cudaSuccess) e = prepare(kernel_of<true>(KP), KP, &s->fit_step);
+  if (e == cudaSuccess) e = ion::prepare_net_select_f32();
   if (e != cudaSuccess) {
     if (s->dev) cudaFree(s->dev);
     if (s->bound) cudaFree(s->bound);

@@ -3,7 +3,7 @@
 A PIC code calls the ionization step once per time step with that step's
 field.  StepGraph records K such calls (and, optionally, the conservation
 diagnostic after each) into one CUDA graph, so that replaying K steps costs
-one graph launch instead of K times three kernel launches and their host
+one graph launch instead of K times two to four kernel launches and their host
 argument checks.  Argument checking happens once, during capture; the graph
 then replays the same device pointers: the field tensors, populations,
 windows, dne and workspace must stay alive and in place.
@@ -15,20 +15,25 @@ import torch
 from . import ionize
 
 
-def _prime(sp: ionize.Species, flags: int, device) -> None:
-    """One eager step on a few private cells, so that the library's one-time
-    per-kernel set-up (shared-memory limits, occupancy) is done before any
-    capture."""
-    n = 256
+def _prime(sp: ionize.Species, flags: int, window: dict | None, device) -> None:
+    """Eager steps on private cells, so that the library's one-time per-kernel
+    set-up (shared-memory limits, occupancy) is done before any capture.  The
+    kernels of large steps are reached by FP32 steps of a few cells under the
+    default launch shape, in rows that the single-species kernel takes and in
+    rows that it does not, and by an FP64 step of more than 32 warps per SM."""
     f64 = bool(flags & ionize.ION_F64_PLAIN)
     dt = torch.float64 if f64 else torch.float32
-    E = torch.full((n,), 100.0, dtype=dt, device=device)
-    N = torch.zeros((sp.Z + 1, n), dtype=dt, device=device)
-    N[0] = 1.0
-    lo = torch.zeros(n, dtype=torch.uint8, device=device)
-    hi = torch.full((n,), min(sp.Z, 3), dtype=torch.uint8, device=device)
-    dne = torch.empty(n, dtype=dt, device=device)
-    ionize.step(sp, E, N, lo, hi, 0.05, dne, flags=flags)
+    sms = torch.cuda.get_device_properties(device).multi_processor_count
+    for n, pad, shape in ([(256, 0, None), (32 * 32 * sms + 32, 0, None)] if f64 else
+                          [(256, 0, None), (256, 0, (2, 8, 0)), (256, 1, (2, 8, 0))]):
+        E = torch.full((n,), 100.0, dtype=dt, device=device)
+        N = torch.zeros((sp.Z + 1, n + pad), dtype=dt, device=device)
+        N[0] = 1.0
+        lo = torch.zeros(n, dtype=torch.uint8, device=device)
+        hi = torch.full((n,), min(sp.Z, 3), dtype=torch.uint8, device=device)
+        dne = torch.empty(n, dtype=dt, device=device)
+        ionize.step_batched([(sp, E, N, lo, hi, dne)], 0.05, flags=flags, shape=shape,
+                            window=window)
     torch.cuda.synchronize(device)
 
 
@@ -75,8 +80,7 @@ class StepGraph:
         step_flags = flags | (ionize.ION_CONSERVATION_CHECK if fused else 0)
         # the step's own measure: word 10 of the workspace header
         change = self.ws[40:44].view(torch.float32)
-        _prime(sp, flags, dev)
-        _prime(sp, step_flags, dev)
+        _prime(sp, step_flags, window, dev)
         self.graph = torch.cuda.CUDAGraph()
         side = torch.cuda.Stream(dev)
         side.wait_stream(torch.cuda.current_stream(dev))
