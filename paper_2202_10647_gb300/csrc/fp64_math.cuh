@@ -14,9 +14,9 @@
 // integer instructions each, whose issue time is that of one FP64 instruction at most.  A
 // rate of Eq. 1 keeps the two fused multiply-adds of its exponent.  FP64 step, 33.5M nitrogen
 // cells: 2,347 us with the polynomials in FP64, 1,922 so.
-// Errors (measured over 2^-20..2^60 and -1000..1000, against 113-bit arithmetic): log2
-// 0.57 ulp of max(|log2 E|, 1), 1/E 0.56 ulp, exp2 0.96 ulp, e^z 0.98 ulp down to z = -256 (1.2
-// to -512, 1.9 below).
+// Errors (over 2^-20..2^60 and -1000..1000, against 113-bit arithmetic; the tests restate
+// these integer steps and hold them): log2 0.79 ulp of max(|log2 E|, 1), 0.57 below 2;
+// 1/E 0.56 ulp; exp2 0.97 ulp; e^z 0.99 ulp down to z = -256 (1.2 to -512, 1.9 below).
 // The tables are nearest values of 40-digit ones; the polynomials
 // interpolate at Chebyshev nodes.
 #pragma once
