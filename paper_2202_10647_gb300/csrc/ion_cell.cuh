@@ -78,17 +78,6 @@ __device__ __forceinline__ void warp_max_into(uint32_t* word, uint32_t bits) {
   if ((threadIdx.x & 31) == 0 && m) atomicMax(word, m);
 }
 
-// Per-precision hooks of the generic cell code.
-struct F32Form {
-  using T = float;
-  using Staged = StagedF32;
-  using Field = FieldF32;
-  __device__ static Field field(float E) { return field_f32(E); }
-  __device__ static float rate(const StagedF32& t, int k, const Field& f) {
-    return rate_dt_f32(t, k, f);
-  }
-};
-
 // Warp-aggregated append of (value, tag) for the lanes with `take` set: one
 // atomic per warp.  Every lane of the warp calls this.
 __device__ __forceinline__ void warp_append(uint32_t* counter, uint32_t* queue,
@@ -157,41 +146,41 @@ __device__ __forceinline__ void window_after_step(const JobIO& J, const Policy& 
 }
 
 // ---------------------------------------------------------------------------
-// Update of one cell whose window populations v[0..w-1] and rates
-// lam[r] = W_{lo+r} dt (r < w-1; 0 beyond) are known (2 <= w <= WM): Taylor
+// FP32 update of one cell whose window populations v[0..w-1] and rates
+// lam[r] = W_{lo+r} dt (r < w-1; 0 beyond) are known (w <= WM): Taylor
 // or Bateman form, window slide, stores.  Returns true (and stores nothing)
 // if the cell goes to the FP64 queue.
 // ---------------------------------------------------------------------------
 // With `change` set (ION_CONSERVATION_CHECK), *change receives
 // |sum_r v'_r - sum_r v_r| over the window, 0 if the cell is queued.
-template <typename T, int WM>
+template <int WM>
 __device__ __forceinline__ bool update_cell(const JobIO& J, const Policy& pol, int c, int lo,
-                                            int hi, T (&v)[WM], const T (&lam)[WM],
-                                            bool allow_fb, T* change = nullptr) {
-  T* __restrict__ N = static_cast<T*>(J.N);
+                                            int hi, float (&v)[WM], const float (&lam)[WM],
+                                            float* change) {
+  float* __restrict__ N = static_cast<float*>(J.N);
   const int w = hi - lo + 1;
-  T dne = T(0);
+  float dne = 0.0f;
   int nlo = lo, nhi = hi;
-  if (change) *change = T(0);
+  if (change) *change = 0.0f;
   if constexpr (WM >= 2) {
     if (w >= 2) {
-      T lmax = T(0);
+      float lmax = 0.0f;
 #pragma unroll
       for (int r = 0; r < WM; ++r) lmax = fmax(lmax, lam[r]);
-      ExactSum<T> acc;
+      ExactSum<float> acc;
       if (change) {
 #pragma unroll
         for (int r = 0; r < WM; ++r)
           if (r < w) acc.add(-v[r]);
       }
-      if (lmax <= DDParams<T>::prop_max) {
-        dne = taylor_propagate<T, WM>(v, lam, w, lmax);
+      if (lmax <= DDParams<float>::prop_max) {
+        dne = taylor_propagate<WM>(v, lam, w, lmax);
       } else {
-        if (allow_fb && (pol.flags & ION_NO_FP64_FALLBACK) == 0 &&
+        if ((pol.flags & ION_NO_FP64_FALLBACK) == 0 &&
             ((pol.flags & ION_FORCE_FP64_COEF) != 0 ||
-             (pol_gap<T>(pol) > T(0) && near_degenerate<T, WM>(lam, w, pol_gap<T>(pol)))))
+             (pol.gap_f > 0.0f && near_degenerate<WM>(lam, w, pol.gap_f))))
           return true;
-        dne = dd_update<T, WM>(v, lam, w);
+        dne = dd_update<float, WM>(v, lam, w);
       }
       if (change) {
 #pragma unroll
@@ -199,8 +188,8 @@ __device__ __forceinline__ bool update_cell(const JobIO& J, const Policy& pol, i
           if (r < w) acc.add(v[r]);
         *change = fabs(acc.value());
       }
-      window_after_step<T, WM>(J, pol, v, w, nlo, nhi);
-      T* p = N + (int64_t)lo * J.ld + c;
+      window_after_step<float, WM>(J, pol, v, w, nlo, nhi);
+      float* p = N + (int64_t)lo * J.ld + c;
 #pragma unroll
       for (int r = 0; r < WM; ++r) {
         if (r < w) __stcs(p, v[r]);
@@ -208,8 +197,8 @@ __device__ __forceinline__ bool update_cell(const JobIO& J, const Policy& pol, i
       }
     }
   }
-  const T* __restrict__ G = static_cast<const T*>(J.n_gas);
-  __stcs(static_cast<T*>(J.dne) + c, G ? dne * G[c] : dne);
+  const float* __restrict__ G = static_cast<const float*>(J.n_gas);
+  __stcs(static_cast<float*>(J.dne) + c, G ? dne * G[c] : dne);
   if (nlo != lo || nhi != hi) {
     J.lo[c] = (uint8_t)nlo;
     J.hi[c] = (uint8_t)nhi;
@@ -217,26 +206,23 @@ __device__ __forceinline__ bool update_cell(const JobIO& J, const Policy& pol, i
   return false;
 }
 
-// Full update of one cell whose window populations are loaded: the rates of
+// Full FP32 update of one cell whose window populations are loaded: the rates of
 // Eq. 1, then update_cell.
-template <class F, int WM>
+template <int WM>
 __device__ __forceinline__ bool finish_cell(const JobIO& J, const Policy& pol,
-                                            const typename F::Staged& tab, int c,
-                                            typename F::T Ec, int lo, int hi,
-                                            typename F::T (&v)[WM], bool allow_fb,
-                                            typename F::T* change = nullptr) {
-  using T = typename F::T;
+                                            const StagedF32& tab, int c, float Ec, int lo, int hi,
+                                            float (&v)[WM], float* change) {
   const int w = hi - lo + 1;
-  T lam[WM];
+  float lam[WM];
 #pragma unroll
-  for (int r = 0; r < WM; ++r) lam[r] = T(0);
+  for (int r = 0; r < WM; ++r) lam[r] = 0.0f;
   if (w >= 2 && !pol.zero_dt) {
-    const typename F::Field f = F::field(Ec);
+    const FieldF32 f = field_f32(Ec);
 #pragma unroll
     for (int r = 0; r < WM; ++r)
-      if (r < w - 1) lam[r] = F::rate(tab, lo + r, f);
+      if (r < w - 1) lam[r] = rate_dt_f32(tab, lo + r, f);
   }
-  return update_cell<T, WM>(J, pol, c, lo, hi, v, lam, allow_fb, change);
+  return update_cell<WM>(J, pol, c, lo, hi, v, lam, change);
 }
 
 }  // namespace ion

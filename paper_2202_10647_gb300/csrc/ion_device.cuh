@@ -277,10 +277,6 @@ __device__ __forceinline__ double rate_dt_f64(const StagedF64& t, int k, const F
   return exp2_f64<Top>(exponent_f64(t.a[k], t.b[k], t.C[k], f));
 }
 
-__device__ __forceinline__ double rate_dt_f64(const StagedF64& t, int k, double E_in) {
-  return rate_dt_f64(t, k, field_f64(E_in));
-}
-
 // y clamped to at most 1000, then to at least the floor whose order_f64 is given.
 __device__ __forceinline__ double clamp_log2(double y, double floor, long long floor_order) {
   if (hi_word(y) >= 0x408f4000) y = 1000.0;
@@ -335,11 +331,9 @@ __device__ constexpr float kThrF32[19] = {
     3.18621f};
 // (The FP64 thresholds are floats too: they meet an FP32 upper bound of the
 // rate, as an FP64 comparison occupies the FP64 pipe like an addition.)
-__device__ constexpr float kThrF64[20] = {
+__device__ constexpr float kThrF64[12] = {
     2e-17f,     6.32456e-09f, 4.93242e-06f, 0.000148017f, 0.00119136f, 0.00493242f,
-    0.0139108f, 0.0307836f,   0.0578509f,   0.0968455f,   0.148911f,   0.214675f,
-    0.294354f,  0.387859f,    0.494882f,    0.614969f,    0.747572f,   0.892092f,
-    1.04791f,   1.21439f};
+    0.0139108f, 0.0307836f,   0.0578509f,   0.0968455f,   0.148911f,   0.214675f};
 
 // 1/n! for n = 0..17 (the Taylor branch needs n <= 4 + 12), in each
 // precision (the FP32 path reads no double: conversions run on the FP64 pipe).
@@ -416,11 +410,11 @@ struct DDParams<float> {
   static constexpr int PMAX = 16;      // bound on the terms (14 needed at 2 * prop_max)
   static constexpr bool kUniform = true;  // every Taylor term up to RMAX
   static constexpr float end_ratio = 4.0f;  // dd_exp_ranges' recurrence bound
-  __device__ static __forceinline__ int terms(float x, int rmax) {
+  // terms of the propagation series for x = 2 max W dt
+  __device__ static __forceinline__ int terms(float x) {
     int R = 0;
 #pragma unroll
-    for (int i = 0; i < 17; ++i)
-      if (i < rmax) R += x > kThrF32[i] ? 1 : 0;
+    for (int i = 0; i < PMAX; ++i) R += x > kThrF32[i] ? 1 : 0;
     return R;
   }
   // (|b| lies in [tau / end_ratio, 2^99]: no scaling)
@@ -436,14 +430,13 @@ struct DDParams<double> {
   static constexpr float tau = 0.25f;
   static constexpr int RMAX = 12;
   static constexpr float prop_max = 0.5f;
-  static constexpr int PMAX = 18;
   static constexpr bool kUniform = false;  // terms(s) of them
   static constexpr float end_ratio = 4.0f;
-  __device__ static __forceinline__ int terms(float x, int rmax) {
+  // terms of a divided difference's series for a spread x
+  __device__ static __forceinline__ int terms(float x) {
     int R = 0;
 #pragma unroll
-    for (int i = 0; i < 20; ++i)
-      if (i < rmax) R += x > kThrF64[i] ? 1 : 0;
+    for (int i = 0; i < RMAX; ++i) R += x > kThrF64[i] ? 1 : 0;
     return R;
   }
   __device__ static __forceinline__ double div(double a, double b) { return div_f64(a, b); }
@@ -555,7 +548,7 @@ __device__ __forceinline__ void dd_exp_ranges(const T (&z)[NR], const T (&ez)[NR
   // (a spread of truncated keys lies within 2^-23 of their size of the nodes')
   if (close)
     taylor_chains<T, NR>(
-        z, P::kUniform ? P::RMAX : P::terms(fmaf(0x1p-22f, zmax, smax), P::RMAX), C);
+        z, P::kUniform ? P::RMAX : P::terms(fmaf(0x1p-22f, zmax, smax)), C);
 #pragma unroll
   for (int len = 2; len <= NR; ++len) {
 #pragma unroll
@@ -615,7 +608,7 @@ __device__ __noinline__ T dd_set(T z0, T z1, T z2, T z3, T z4, T e0, T e1, T e2,
       if (P::key(zi) - P::key(z[j]) >= P::tau) {
         d[j] = P::div(d[j + 1] - d[j], s);
       } else {
-        const int R = P::kUniform ? P::RMAX : P::terms((float)s, P::RMAX);
+        const int R = P::kUniform ? P::RMAX : P::terms((float)s);
         T H[P::RMAX + 1];
         H[0] = T(1);
 #pragma unroll
@@ -638,35 +631,35 @@ __device__ __noinline__ T dd_set(T z0, T z1, T z2, T z3, T z4, T e0, T e1, T e2,
   return d[0];
 }
 
-// Small rates: N' = sum_k (dt A)^k N / k! applied to the window vector
+// Small rates in FP32: N' = sum_k (dt A)^k N / k! applied to the window vector
 // directly.  With every W dt <= prop_max the norm of dt A is at most
 // 2 prop_max, the terms shrink from the first, and R terms leave a remainder
 // below (2 prop_max)^(R+1)/(R+1)!.  inc[] collects N' - N without forming
 // the difference, so the freed electrons carry no cancellation.
 //   v, lam, w as in dd_update below; returns the electrons released.
-template <typename T, int WM, int PMAX = DDParams<T>::PMAX>
-__device__ __forceinline__ T taylor_propagate(T (&v)[WM], const T (&lam)[WM],
-                                              int w, T lmax) {
-  using P = DDParams<T>;
-  const int R = P::terms(T(2) * lmax, PMAX);
-  T t[WM], inc[WM];
+template <int WM>
+__device__ __forceinline__ float taylor_propagate(float (&v)[WM], const float (&lam)[WM], int w,
+                                                  float lmax) {
+  constexpr int PMAX = DDParams<float>::PMAX;
+  const int R = DDParams<float>::terms(2.0f * lmax);
+  float t[WM], inc[WM];
 #pragma unroll
   for (int i = 0; i < WM; ++i) {
-    t[i] = i < w ? v[i] : T(0);
-    inc[i] = T(0);
+    t[i] = i < w ? v[i] : 0.0f;
+    inc[i] = 0.0f;
   }
 #pragma unroll
   for (int k = 1; k <= PMAX; ++k) {
     if (k > R) break;
-    const T rk = T(1.0 / k);
+    const float rk = float(1.0 / k);
 #pragma unroll
     for (int i = WM - 1; i >= 0; --i) {
-      const T gain = i > 0 ? lam[i - 1] * t[i - 1] : T(0);
+      const float gain = i > 0 ? lam[i - 1] * t[i - 1] : 0.0f;
       t[i] = (gain - lam[i] * t[i]) * rk;
       inc[i] += t[i];
     }
   }
-  T cum = T(0), dne = T(0);
+  float cum = 0.0f, dne = 0.0f;
 #pragma unroll
   for (int r = 0; r < WM; ++r) {
     if (r < w - 1) {
@@ -718,12 +711,12 @@ __device__ __forceinline__ int flow_terms(float x) {
   return R;
 }
 
-// The same in FP64 for a window of exactly W states, in R terms: the series
+// Small rates in FP64, for a window of exactly W states, in R terms: the series
 // G_r = sum_k u_r^(k-1) / k! of every state, whose flow across the boundary above it
 // is F_r = W_r dt G_r, so that a term takes three FP64 instructions per state (its share of
 // G, its outflow, its next u = inflow - outflow), two for the first and the last,
 // and none for the top state, which only receives; N'_r = N_r + F_{r-1} - F_r, and the
-// freed electrons are sum F.  (The term-by-term form above takes four per slot.)
+// freed electrons are sum F.  (Term by term, as in FP32, it takes four per slot.)
 template <int W>
 __device__ __forceinline__ double taylor_flow_f64(double (&v)[W], const double (&lam)[W], int R) {
   double u[W - 1], F[W - 1];
@@ -769,7 +762,7 @@ __device__ __forceinline__ double taylor_flow_f64(double (&v)[W], const double (
 // others lost, so the window's sum is kept (Eq. 9 is 1 - Eqs. 6-8 column by
 // column).  Returns the electrons released, sum_k k (N'_k - N_k) = the sum
 // over the w-1 internal boundaries of the population that crossed them.
-// (Cells whose rates are all small take taylor_propagate instead.)
+// (Cells whose rates are all small take a series instead.)
 // ---------------------------------------------------------------------------
 template <typename T, int WM>
 __device__ __forceinline__ T dd_update(T (&v)[WM], const T (&lam)[WM], int w) {
@@ -823,11 +816,10 @@ __device__ __forceinline__ T dd_update(T (&v)[WM], const T (&lam)[WM], int w) {
   return dne;
 }
 
-// North-star degeneracy test: some pair of the window's rates with
+// Near-degeneracy: some pair of the window's rates with
 // |W_i - W_j| < gap * max(W_i, W_j).
-template <typename T, int WM>
-__device__ __forceinline__ bool near_degenerate(const T (&lam)[WM], int w,
-                                                T gap) {
+template <int WM>
+__device__ __forceinline__ bool near_degenerate(const float (&lam)[WM], int w, float gap) {
   bool deg = false;
 #pragma unroll
   for (int i = 0; i < WM - 1; ++i)

@@ -60,19 +60,13 @@ struct Policy {
   float eps_f, gap_f, eps_grow_f;  // the same in FP32 (no per-cell conversion)
 };
 
-// eps, gap, eps_grow of the policy in the precision of the caller.
+// eps and eps_grow of the policy in the precision of the caller.
 template <typename T>
 __device__ __forceinline__ T pol_eps(const Policy& p);
 template <>
 __device__ __forceinline__ float pol_eps<float>(const Policy& p) { return p.eps_f; }
 template <>
 __device__ __forceinline__ double pol_eps<double>(const Policy& p) { return p.eps; }
-template <typename T>
-__device__ __forceinline__ T pol_gap(const Policy& p);
-template <>
-__device__ __forceinline__ float pol_gap<float>(const Policy& p) { return p.gap_f; }
-template <>
-__device__ __forceinline__ double pol_gap<double>(const Policy& p) { return p.gap; }
 template <typename T>
 __device__ __forceinline__ T pol_grow(const Policy& p);
 template <>
@@ -155,9 +149,10 @@ int job_from_args(const ion_species* sp, const void* E, void* N, int64_t ld, int
                   const char* who, JobIO* J);
 int workspace_ok(void* workspace, size_t have, size_t need);
 
-// Launches a kernel that follows another of the same call (programmatic dependent launch):
-// its blocks are set up while the last blocks of the one before finish, and what
-// that one writes is there after cudaGridDependencySynchronize, which every thread
+// Launches a kernel that follows another of the same call (programmatic dependent launch): it
+// is launched when all blocks of the one before have exited (or, behind ion_stiff_kernel, have
+// come up: it triggers early), so that its launch overlaps their end, and what that one
+// writes is there after cudaGridDependencySynchronize, which every thread
 // calls.  Only inside a call: the first kernel of each is an ordinary launch, so that it
 // follows all that the stream held before.  `dependent` false: an ordinary launch.
 template <typename... P, typename... A>

@@ -86,10 +86,6 @@ __device__ __forceinline__ void stage(const float* __restrict__ P, int K, Net<KP
   for (int k = threadIdx.x; k < KP; k += blockDim.x) n.b3[k] = k < K ? P[off_b3(K) + k] : 0.0f;
 }
 
-// The loops over hidden units o are kept rolled: each iteration is a dot
-// product over the register arrays (h1, y, dy, acc) fully unrolled, so the
-// arrays stay in registers at a modest code size.
-
 // ---- training --------------------------------------------------------------
 // Shared memory of a training block: the weights in both orders (a product
 // reads its inner index first), and the tile's activations and their
@@ -398,6 +394,9 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// One thread per sample.  The loop over hidden units o is kept rolled: each iteration is a dot
+// product over the register array h1 and an update of y, fully unrolled, so
+// that the arrays stay in registers at a modest code size.
 template <int KP, bool Q>
 __global__ void __launch_bounds__(kThreads)
     mlp_forward(const float* __restrict__ P, int K, const float* __restrict__ x, int B,

@@ -1112,7 +1112,7 @@ __device__ __forceinline__ bool record_cell(const BatchArgs& a, const StagedF32&
 #pragma unroll
   for (int r = 0; r < W; ++r)
     v[r] = r < w ? __ldcs(a.ws.rec_V + (int64_t)r * a.ws.rec_cap + i) : 0.0f;
-  return finish_cell<F32Form, W>(J, a.pol, tab, c, Ec, lo, hi, v, true, change);
+  return finish_cell<W>(J, a.pol, tab, c, Ec, lo, hi, v, change);
 }
 
 __global__ void __launch_bounds__(256, 3)
@@ -1401,8 +1401,8 @@ __device__ __forceinline__ float direct_record(const JobIO& J, const Policy& pol
   }
   stiff = lmax > DDParams<float>::prop_max;
   float d = 0.0f;
-  fb = update_cell<float, W>(J, pol, c, lo, hi, v, lam, true,
-                             (pol.flags & ION_CONSERVATION_CHECK) ? &d : nullptr);
+  fb = update_cell<W>(J, pol, c, lo, hi, v, lam,
+                      (pol.flags & ION_CONSERVATION_CHECK) ? &d : nullptr);
   if (fb) d = fb_cell<W>(J, pol, tab, c, lo, hi);
   return d;
 }
@@ -1702,8 +1702,9 @@ cudaError_t launch_net_select_f32(BatchArgs& a, const NetSelect& sel, int num_sm
   return cudaLaunchKernel(v->fn, blocks, v->W * 32, args, smem, s);
 }
 
-// The record and queue kernels follow the streaming kernel as its dependents, which gives no
-// early trigger: record blocks that come up beside it run under its shared-memory carveout,
+// The record and queue kernels follow the streaming kernel as its dependents (their launch
+// overlaps its last blocks' end; the queue kernel, behind the record kernel's early trigger, is
+// up and has staged its tables by then).  The streaming kernel gives no early trigger: record blocks that come up beside it run under its shared-memory carveout,
 // with next to no L1 (20 Kr-like steps 5 % slower).  One step, us: 33.5M nitrogen cells 318 ->
 // 313, 4M Kr-like adaptive 177 -> 173, 1M Ar-like field 80 -> 74, 30M mixed 987 -> 977.
 

@@ -14,7 +14,7 @@
 //     FP32 estimate of their largest W dt (Taylor by the number of its
 //     terms, Bateman form), and each queue is worked off 32 cells at a time,
 //     so that the FP64 arithmetic runs in full warps whose lanes take the
-//     same path at exactly their width (2 W dt <= kThrF64[R] takes R terms);
+//     same path at exactly their width (in as many terms as that needs: kThrFlow);
 //     at the end the warps of a block put their leftovers together;
 //   * a grid too small to fill those queues runs one cell per lane
 //     (ion_step_f64_direct), on as many SMs as it has warps.
@@ -46,7 +46,7 @@ struct F64Smem {
 };
 
 // The form class of an FP32 estimate of the largest W dt (2 W dt below
-// kThrF64[R] takes at most R terms; above 0.49 the cell most likely takes
+// kThrF64[R] takes at most R terms at any width; above 0.49 the cell most likely takes
 // the Bateman form: its own FP64 rates decide).
 __device__ __forceinline__ int form_class(float lmax) {
   const float x = 2.0f * lmax;

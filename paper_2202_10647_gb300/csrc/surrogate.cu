@@ -362,9 +362,10 @@ __device__ __forceinline__ void taylor_cells(const StepArgs& a, int c, int lo, i
   }
 }
 
-// The rates of Eq. 1 for the window's w-1 transitions as ion_step's
-// streaming kernel takes them: the plain FP32 exponent for every rate, the
-// float-float recompute for those above 2^-6 (W dt).
+// The rates of Eq. 1 for the window's w-1 transitions: the plain FP32
+// exponent for every rate, the float-float recompute for those above 2^-6
+// (W dt).  (The streaming kernel leaves out a's low part and the cutoff test of the plain
+// ones: the last bits of a cell may differ with the route that its call takes.)
 __device__ __forceinline__ void eq1_rates(const StagedF32& tab, int lo, int w, float E,
                                           float (&lam)[ION_MAX_WINDOW]) {
   const FieldF32 f = field_f32(E);
