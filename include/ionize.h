@@ -519,7 +519,8 @@ ION_API int ion_surrogate_rates(const ion_surrogate* s, const float* E, int64_t 
  * never uses the network.  (In a call of more than 320,000 cells whose
  * arrays allow the streaming kernel, a cell whose rates of Eq. 1, lowered by
  * twice their validation bound, already exceed pop_tol takes Eq. 1 without
- * asking the network.)  A cell
+ * asking the network, in another FP32 form of its rates: the last bits of a
+ * cell can differ between the two.)  A cell
  * with some rate W dt > 1 always takes the rates of Eq. 1 (its bound would
  * exceed any useful tolerance) and is finished in the Bateman form by
  * ion_step's record kernel.  The update itself is ion_step's (Taylor or
